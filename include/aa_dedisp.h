@@ -141,7 +141,8 @@ typedef struct aa_range_info {
     int32_t stages;          /* pipeline depth of the staging copies */
     int32_t span_max;        /* largest delay spread across one CTA's trials */
     int32_t smem_bytes;      /* dynamic shared memory per dedispersion CTA */
-    int32_t strategy;        /* aa_dedisp_strategy in use for this range */
+    int32_t strategy;        /* aa_dedisp_strategy in use for this range (given a row buffer,
+                                ranges that share delay patterns run on band rows) */
     int32_t grouped_available;  /* 1 if AA_DEDISP_GROUPED can be selected */
     double grouped_work;     /* adds of the grouped strategy / adds of the direct one */
     int32_t subband_channels;       /* AA_DEDISP_SUBBAND: channels per band (else 0) */
@@ -166,7 +167,7 @@ typedef struct aa_plan_info {
     int64_t nsamp;
     int64_t in_pitch_min;      /* minimum device input row pitch, bytes (nsamp rounded up to 16) */
     int64_t dd_elems;          /* floats in the dedispersed output buffer */
-    int64_t dedisp_ws_bytes;   /* scratch for aa_dedisperse_device */
+    int64_t dedisp_ws_bytes;   /* scratch for aa_dedisperse_device (at its fastest: see there) */
     int64_t sps_ws_bytes;      /* scratch for aa_sps_search_device at max_width */
     int64_t table_bytes;       /* device delay tables owned by the plan */
     int64_t host_path_bytes;   /* peak device bytes of aa_dedisperse + aa_sps_search */
@@ -216,8 +217,11 @@ typedef struct aa_candidate {
  *   d_out    : float [dd_elems] device memory (aa_plan_info.dd_elems);
  *              range r, trial i, sample t is at row_offset_r + i*pitch_r + t
  *              for t < L_r (exact integers); padding is left unwritten.
- *   d_ws     : device scratch of ws_bytes >= dedisp_ws_bytes (may be NULL if
- *              that is 0), 256-byte aligned.
+ *   d_ws     : device scratch, 256-byte aligned, of ws_bytes >= dedisp_ws_bytes.
+ *              At most 2 GiB at its end are a row buffer (the sums of 8, 4 or
+ *              2 consecutive channels that many trials share); with less
+ *              scratch, down to what the decimated inputs and the sub-band and
+ *              FDMT ranges take, the call runs without it: same results, slower.
  * The plan must be bound.  Stream-ordered, asynchronous; returns
  * AA_ERR_ARG/AA_ERR_STATE on bad arguments, AA_ERR_CUDA if a launch fails. */
 aa_status aa_dedisperse_device(const aa_plan* plan, const uint8_t* d_in, int64_t nsamp,
@@ -261,7 +265,12 @@ aa_status aa_workspace_status(void* d_ws, aa_stream_t stream);
  *   AA_DEDISP_GROUPED: within a block of 16 trials and a chunk of channels,
  *     channels whose delays differ from the block's first trial by the same
  *     amounts at every trial are first summed once; each trial then adds the
- *     group sums.  Available when the plan could build the group tables. */
+ *     group sums.  Available when the plan could build the group tables.
+ * Where they are cheaper (AA_DEDISP_GROUPED, or the plan's own choice) and
+ * the call's scratch holds their row buffer, band rows run instead: every
+ * distinct sum of a band of consecutive channels is built once for many
+ * trials and each trial adds one per band.  aa_plan_set_strategy with
+ * AA_DEDISP_DIRECT, and aa_plan_autotune choosing it, keep the direct kernel. */
 typedef enum { AA_DEDISP_DIRECT = 0, AA_DEDISP_GROUPED = 1, AA_DEDISP_SUBBAND = 2,
                AA_DEDISP_FDMT = 3 } aa_dedisp_strategy;
 

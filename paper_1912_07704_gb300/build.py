@@ -23,7 +23,7 @@ LIB = os.path.join(HERE, "libaa_gb300.so")
 SOURCES = ["aa_plan.cpp", "aa_api.cpp", "aa_api_f32.cpp", "aa_profile.cpp", "aa_dedisp.cu",
            "aa_sps.cu", "aa_noalloc.cu", "aa_adjoint.cu", "aa_batch.cpp", "aa_autotune.cpp",
            "aa_server.cpp", "aa_fil.cpp", "aa_corner.cu", "aa_post.cu", "aa_subband.cu",
-           "aa_pipeline.cpp", "aa_fused.cpp", "aa_fdmt.cu"]
+           "aa_pipeline.cpp", "aa_fused.cpp", "aa_fdmt.cu", "aa_band_plan.cpp", "aa_bands.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -48,7 +48,7 @@ def _flags(src: str, verbose: bool) -> list:
 
 def _deps() -> list:
     files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith(".h")]
+    files += [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
     files.append(os.path.join(INCLUDE, "aa_dedisp.h"))
     return files
 

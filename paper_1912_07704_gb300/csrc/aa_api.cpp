@@ -395,8 +395,8 @@ aa_status aa_dedisperse_device(const aa_plan* p, const uint8_t* d_in, int64_t ns
         set_error("d_in/d_out must be 16-byte and d_ws 256-byte aligned");
         return AA_ERR_ARG;
     }
-    if ((int64_t)ws_bytes < L.dedisp_ws) {
-        set_error("workspace %zu bytes < required %lld", ws_bytes, (long long)L.dedisp_ws);
+    if ((int64_t)ws_bytes < L.dedisp_base) {
+        set_error("workspace %zu bytes < required %lld", ws_bytes, (long long)L.dedisp_base);
         return AA_ERR_ARG;
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -433,6 +433,8 @@ aa_status aa_dedisperse_device(const aa_plan* p, const uint8_t* d_in, int64_t ns
         a.out = d_out + L.row_offset[r];
         a.out_pitch = L.pitch[r];
         fill_strategy(a, g);
+        a.band_rows = reinterpret_cast<uint32_t*>(ws + L.dedisp_base);
+        a.band_bytes = (int64_t)ws_bytes - L.dedisp_base;
         a.err = err;
         if (a.length <= 0) continue;
         ProfScope prof(g.elem == 1 ? kKDedispU8 : kKDedispU16, s);

@@ -78,6 +78,13 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
     void* probe = nullptr;
     void* out = nullptr;
     unsigned* err = nullptr;
+    void* rows = nullptr;  // row buffer of the grouped strategy's bands; without it the grouped kernel is timed
+    int64_t row_bytes = 0;
+    for (size_t r = 0; r < p->ranges.size(); ++r) row_bytes = std::max(row_bytes, band_bytes(p->ranges[r].bands, L.length[r]));
+    if (row_bytes > 0 && cudaMalloc(&rows, (size_t)row_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        rows = nullptr;
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     aa_status status = AA_OK;
     if (cudaMalloc(&probe, bytes) != cudaSuccess || cudaMalloc(&out, std::max<size_t>(out_bytes, 256)) != cudaSuccess ||
@@ -131,6 +138,9 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
                     g.strategy = grouped ? 1 : 0;
                     fill_strategy(a, g);
                     g.strategy = saved;
+                    if (!grouped) a.bands = nullptr;
+                    a.band_rows = static_cast<uint32_t*>(rows);
+                    a.band_bytes = rows ? row_bytes : 0;
                     if (!grouped) {
                         a.cc = cc;
                         a.nstage = ns;
@@ -160,6 +170,7 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
             new_lines.push_back(line.str());
         }
         g.strategy = best_strategy;
+        g.pinned = true;
         g.cc = best_cc;
         g.nstage = best_ns;
         g.flush = (std::min(65535 / (255 * g.desc.dec), 256) / best_cc) * best_cc;
@@ -170,6 +181,7 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
     if (probe) cudaFree(probe);
     if (out) cudaFree(out);
     if (err) cudaFree(err);
+    if (rows) cudaFree(rows);
     if (status == AA_OK && cache_path && !new_lines.empty()) {
         std::ofstream f(cache_path, std::ios::app);
         for (auto& l : new_lines) f << l << "\n";

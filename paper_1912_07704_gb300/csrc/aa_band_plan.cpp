@@ -1,0 +1,328 @@
+// Tables of the band rows (see aa_bands.h).  Host only.
+#include <algorithm>
+#include <climits>
+#include <cstring>
+#include <utility>
+
+#include "aa_internal.h"
+
+namespace aa {
+
+namespace {
+
+constexpr size_t kRowSmem = 36 * 1024;   // six CTAs of the row kernel per SM
+constexpr size_t kSumSmem = 220 * 1024;  // one CTA of the summing kernel per SM
+
+// Distinct keys of one band in first-seen order (open addressing; cleared by
+// stamping).
+class KeySet {
+  public:
+    KeySet() : keys_(kSize), ids_(kSize), stamp_(kSize, 0) {}
+    void clear() { ++now_; n_ = 0; }
+    // index of `key`; `fresh` set when it is new
+    int add(uint64_t key, bool& fresh) {
+        size_t h = (size_t)((key * 0x9e3779b97f4a7c15ull) >> 48) & (kSize - 1);
+        while (stamp_[h] == now_) {
+            if (keys_[h] == key) { fresh = false; return ids_[h]; }
+            h = (h + 1) & (kSize - 1);
+        }
+        stamp_[h] = now_;
+        keys_[h] = key;
+        ids_[h] = n_;
+        fresh = true;
+        return n_++;
+    }
+
+  private:
+    static constexpr size_t kSize = 4096;  // a segment has at most kBandSegment keys
+    std::vector<uint64_t> keys_;
+    std::vector<int> ids_;
+    std::vector<uint32_t> stamp_;
+    uint32_t now_ = 0;
+    int n_ = 0;
+};
+
+// Tables for bands of k channels; false where a row's delays, a block's rows
+// or a slot do not fit.
+bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
+    bp = BandPlan{};
+    bp.k = k;
+    bp.nbands = (C + k - 1) / k;
+    const int dec = r.desc.dec, ndm = r.desc.ndm;
+    if (2 * k * 255 * dec > 65535) return false;  // the sum of two rows stays in a 16-bit lane
+    const int npad = (bp.nbands + 1) & ~1;
+    const int nblk_all = (ndm + kBandTrials - 1) / kBandTrials;
+    bp.heads.resize((size_t)nblk_all * npad);
+    bp.offs.resize((size_t)nblk_all * npad * kBandTrials);
+    KeySet row_keys, quad_keys;
+    std::vector<int> id(kBandSegment);
+    std::vector<int32_t> sp(kBandSegment);
+    std::vector<uint64_t> key;
+    std::vector<int32_t> lo, hi, blo, bhi, bdst;
+    std::vector<int> border, pair_dst((size_t)nblk_all, 0);
+    int blk_base = 0;
+    int max_quads = 0, max_e = 0, max_rq = 0;
+    double cost = 0;
+    for (int d0 = 0; d0 < ndm; d0 += kBandSegment) {
+        BandSegment seg;
+        seg.trial0 = d0;
+        seg.ntrials = std::min(kBandSegment, ndm - d0);
+        seg.nblk = (seg.ntrials + kBandTrials - 1) / kBandTrials;
+        seg.blk0 = blk_base;
+        seg.row0 = (uint32_t)bp.rows.size();
+        uint64_t pre = 0;
+        for (int b = 0; b < bp.nbands; ++b) {
+            const int c0 = b * k, nch = std::min(k, C - c0);
+            const int na = std::min(nch, 4), nb = nch - na;
+            row_keys.clear();
+            key.clear();
+            lo.clear();
+            hi.clear();
+            for (int i = 0; i < seg.ntrials; ++i) {
+                const int32_t* s = &r.shifts[(size_t)(d0 + i) * C + c0];
+                int32_t mn = s[0];
+                for (int j = 1; j < nch; ++j) mn = std::min(mn, s[j]);
+                uint64_t kk = 0;
+                for (int j = 0; j < nch; ++j) {
+                    const int32_t e = s[j] - mn;
+                    if (e > 255) return false;
+                    kk |= (uint64_t)e << (8 * j);
+                }
+                bool fresh;
+                const int q = row_keys.add(kk, fresh);
+                if (fresh) {
+                    key.push_back(kk);
+                    lo.push_back(mn);
+                    hi.push_back(mn);
+                } else {
+                    lo[q] = std::min(lo[q], mn);
+                    hi[q] = std::max(hi[q], mn);
+                }
+                id[i] = q;
+                sp[i] = mn;
+            }
+            const int n = (int)key.size();
+            BandInfo info{};
+            info.row0 = (uint32_t)bp.rows.size();
+            info.quad0 = (uint32_t)bp.quads.size();
+            info.nrows = (uint16_t)n;
+            info.c0 = (uint16_t)c0;
+            info.nch = (uint16_t)nch;
+            const size_t first_row = bp.rows.size();
+            int32_t umin = INT32_MAX, umax = 0;
+            // quads of the two halves: their delays with the half's smallest removed
+            auto half = [&](uint64_t kk, int j0, int cnt, uint16_t& e) {
+                uint16_t rr[4];
+                int mn = 255;
+                for (int j = 0; j < cnt; ++j) mn = std::min(mn, (int)(kk >> (8 * (j0 + j)) & 255));
+                uint64_t qk = 0;
+                for (int j = 0; j < 4; ++j) {
+                    rr[j] = j < cnt ? (uint16_t)((kk >> (8 * (j0 + j)) & 255) - mn) : 0xffff;
+                    qk |= (uint64_t)(j < cnt ? rr[j] : 0) << (8 * j);
+                }
+                e = (uint16_t)mn;
+                bool fresh;
+                const int q = quad_keys.add(qk, fresh);
+                if (fresh) {
+                    BandQuad quad;
+                    std::memcpy(quad.r, rr, sizeof rr);
+                    for (int j = 0; j < cnt; ++j) max_rq = std::max(max_rq, (int)rr[j]);
+                    bp.quads.push_back(quad);
+                }
+                return (uint16_t)q;
+            };
+            for (int q = 0; q < n; ++q) {
+                BandRow row{};
+                row.qa = row.qb = 0xffff;
+                row.smin = lo[q];
+                row.span = hi[q] - lo[q];
+                row.blk0 = 0xffff;
+                umin = std::min(umin, lo[q]);
+                umax = std::max(umax, hi[q]);
+                bp.rows.push_back(row);
+            }
+            quad_keys.clear();
+            for (int q = 0; q < n; ++q) bp.rows[first_row + q].qa = half(key[q], 0, na, bp.rows[first_row + q].ea);
+            info.nqa = (uint16_t)(bp.quads.size() - info.quad0);
+            if (nb > 0) {
+                quad_keys.clear();
+                for (int q = 0; q < n; ++q)
+                    bp.rows[first_row + q].qb = (uint16_t)(half(key[q], 4, nb, bp.rows[first_row + q].eb) + info.nqa);
+            }
+            info.nqb = (uint16_t)(bp.quads.size() - info.quad0 - info.nqa);
+            for (int q = 0; q < n; ++q)
+                max_e = std::max({max_e, (int)bp.rows[first_row + q].ea, (int)bp.rows[first_row + q].eb});
+            info.umin = umin;
+            info.ulen = umax - umin;
+            max_quads = std::max(max_quads, (int)info.nqa + info.nqb);
+            bp.max_ulen = std::max(bp.max_ulen, info.ulen);
+            bp.max_rows = std::max(bp.max_rows, n);
+            for (int q = 0; q < n; ++q) {
+                BandRow& row = bp.rows[first_row + q];
+                row.pre = (uint32_t)pre;
+                // a window may start up to 3 words early and end up to 3 late
+                pre += (uint64_t)round_up(row.span + 8, 4);
+            }
+            if (pre > UINT32_MAX / 4) return false;
+            // the blocks: which rows each uses, at which delays
+            for (int g = 0; g < seg.nblk; ++g) {
+                const int i0 = g * kBandTrials, i1 = std::min(seg.ntrials, i0 + kBandTrials);
+                blo.assign((size_t)n, INT32_MAX);
+                bhi.assign((size_t)n, -1);
+                bdst.assign((size_t)n, 0);
+                border.clear();
+                for (int i = i0; i < i1; ++i) {
+                    const int q = id[i];
+                    if (bhi[q] < 0) border.push_back(q);
+                    blo[q] = std::min(blo[q], sp[i]);
+                    bhi[q] = std::max(bhi[q], sp[i]);
+                }
+                if ((int)border.size() > kBandMaxRows) return false;
+                const size_t bb = (size_t)(blk_base + g) * npad + b;
+                BandHead& h = bp.heads[bb];
+                h.first = (uint32_t)bp.copies.size();
+                h.n = (uint16_t)border.size();
+                // the second band of a pair goes behind the first
+                const int dst0 = b & 1 ? pair_dst[blk_base + g] : 0;
+                int dst = dst0;
+                for (int q : border) {
+                    BandRow& row = bp.rows[first_row + q];
+                    row.blk0 = std::min<uint16_t>(row.blk0, (uint16_t)g);
+                    row.blk1 = std::max<uint16_t>(row.blk1, (uint16_t)g);
+                    const int32_t at = blo[q] - row.smin;
+                    BandCopy c;
+                    c.row = (uint32_t)(first_row + q) - seg.row0;
+                    c.rel = row.pre + (uint32_t)(at & ~3);
+                    c.dst = (uint32_t)dst;
+                    c.n = (uint32_t)round_up(kBandWords + (bhi[q] - blo[q]) + (at & 3), 4);
+                    bdst[q] = dst + (at & 3) - blo[q];  // slot word of delay s: bdst + s
+                    dst += (int)c.n;
+                    bp.copies.push_back(c);
+                }
+                if (dst > 65535) return false;
+                pair_dst[blk_base + g] = dst;
+                h.words = (uint16_t)(dst - dst0);
+                uint16_t* of = &bp.offs[bb * kBandTrials];
+                for (int t = 0; t < kBandTrials; ++t) {
+                    const int i = std::min(i0 + t, i1 - 1);
+                    of[t] = (uint16_t)(bdst[id[i]] + sp[i]);
+                }
+                // summing kernel: 8 words a lane for each trial, plus the ring's fill
+                cost += 8.0 * kBandTrials + (dst - dst0) / 32.0;
+            }
+            // row kernel: 256 words of a row take 90 cycles (written at 2.8 TB/s,
+            // measured, 152 SMs), read back once by the way
+            cost += 90.0 * n;
+            bp.infos.push_back(info);
+        }
+        seg.nrows = (int64_t)bp.rows.size() - seg.row0;
+        seg.pre = (int64_t)pre;
+        bp.segs.push_back(seg);
+        blk_base += seg.nblk;
+    }
+    // the ring: places one after the other, from the start again where the end
+    // has no room; a place is free once every pair before it whose place it
+    // overlaps is consumed (pairs are consumed in order)
+    bp.ring_words = (int)(kSumSmem / 4);
+    bp.smem_sum = kSumSmem;
+    for (int g = 0; g < nblk_all; ++g) {
+        BandHead* h = &bp.heads[(size_t)g * npad];
+        std::vector<std::pair<int, int>> place;
+        int pos = 0, after = -1;
+        for (int pr = 0; pr < npad / 2; ++pr) {
+            const int w = kBandTrials + h[2 * pr].words + h[2 * pr + 1].words;
+            if (w > bp.ring_words / (kBandLag + 2)) return false;  // the pair added, the lag behind it, one ahead
+            if (pos + w > bp.ring_words) pos = 0;
+            after = std::max(after, pr - kBandBars);
+            for (int q = after + 1; q < pr; ++q)
+                if (place[q].first < pos + w && pos < place[q].second) after = q;
+            if (after >= 0 && after + kBandLag > pr) return false;
+            place.push_back({pos, pos + w});
+            for (int u = 0; u < 2; ++u) {
+                h[2 * pr + u].place = (uint32_t)pos;
+                h[2 * pr + u].after = (int16_t)after;
+                h[2 * pr + u].at = (int16_t)(after < 0 ? 0 : after + kBandLag);
+            }
+            pos += w;
+        }
+    }
+    bp.max_quads = max_quads;
+    for (bp.tile = 1024; bp.tile >= 128; bp.tile /= 2) {
+        bp.quad_words = (int)round_up(bp.tile + max_e, 4);
+        bp.raw_words = (int)round_up(bp.quad_words + max_rq, 4);
+        bp.smem_rows = ((size_t)k * bp.raw_words + (size_t)max_quads * bp.quad_words) * 4 + (size_t)bp.max_rows * sizeof(BandRow) +
+                       (size_t)max_quads * sizeof(BandQuad);
+        if (bp.smem_rows <= kRowSmem) break;
+    }
+    if (bp.tile < 128) {  // a band of many quads: two CTAs per SM
+        bp.tile = 128;
+        if (bp.smem_rows > 2 * kRowSmem) return false;
+    }
+    bp.cost = cost;
+    bp.ok = true;
+    return true;
+}
+
+}  // namespace
+
+bool band_shifts(const BandPlan& bp, int C, int ndm, int32_t* out) {
+    for (size_t q = 0; q < bp.segs.size(); ++q) {
+        const BandSegment& seg = bp.segs[q];
+        for (int i = 0; i < seg.ntrials; ++i)
+            for (int b = 0; b < bp.nbands; ++b) {
+                const int npad = (bp.nbands + 1) & ~1;
+                const size_t bb = (size_t)(seg.blk0 + i / kBandTrials) * npad + b;
+                const BandHead& h = bp.heads[bb];
+                const uint32_t off = bp.offs[bb * kBandTrials + i % kBandTrials];
+                const BandCopy* c = nullptr;
+                for (uint32_t j = 0; j < h.n; ++j) {
+                    const BandCopy& x = bp.copies[h.first + j];
+                    if (off >= x.dst && off < x.dst + x.n) c = &x;
+                }
+                if (!c || off + kBandWords > c->dst + c->n || c->dst + c->n > (uint32_t)h.words + (b & 1 ? bp.heads[bb - 1].words : 0) ||
+                    h.place + kBandTrials + c->dst + c->n > (uint32_t)bp.ring_words || c->row >= seg.nrows) return false;
+                const BandInfo& info = bp.infos[q * bp.nbands + b];
+                const BandRow& row = bp.rows[seg.row0 + c->row];
+                const int32_t at = (int32_t)(c->rel - row.pre + off - c->dst);  // row delay - row.smin
+                const uint32_t next = c->row + 1 < seg.nrows ? bp.rows[seg.row0 + c->row + 1].pre : (uint32_t)seg.pre;
+                if (at < 0 || at > row.span || c->rel + c->n > next + kBandWords) return false;
+                if (i / kBandTrials < row.blk0 || i / kBandTrials > row.blk1) return false;
+                for (int j = 0; j < info.nch; ++j) {
+                    const BandQuad& quad = bp.quads[info.quad0 + (j < 4 ? row.qa : row.qb)];
+                    out[(size_t)(seg.trial0 + i) * C + info.c0 + j] = row.smin + at + (j < 4 ? row.ea : row.eb) + quad.r[j & 3];
+                }
+            }
+    }
+    return true;
+}
+
+void build_bands(RangePlan& r, int C) {
+    r.bands = BandPlan{};
+    if (C > 65535 || r.desc.ndm < kBandTrials / 2) return;
+    // SM cycles per 512 output samples of the direct kernel: 64 trials of one
+    // channel take 991 (10.4e12 adds/s on 152 SMs at 2.07 GHz, measured).
+    // Bands of 8 channels cost about a seventh of that under fine DM steps;
+    // at DM step 1 over 256 channels, bands of 2 to 8 cost about half and run
+    // in 153 us against 180 (few CTAs: 1.5 waves).  Under half a block of
+    // trials the row kernel's launch is not repaid.
+    const double direct = 991.0 / 64 * (double)r.desc.ndm * C;
+    BandPlan best;
+    for (int k = 8; k >= 2; k /= 2) {
+        BandPlan bp;
+        if (!build(r, C, k, bp)) continue;
+        if (!best.ok || bp.cost < best.cost) best = std::move(bp);
+        // few rows per block: smaller bands only add sums
+        if ((double)best.rows.size() < 40.0 * best.nbands * (double)best.segs.size()) break;
+    }
+    if (best.ok && best.cost < 0.6 * direct) r.bands = std::move(best);
+}
+
+int64_t band_bytes(const BandPlan& bp, int64_t length) {
+    if (!bp.ok || length <= 0) return 0;
+    const int64_t ntiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
+    int64_t words = 0;
+    for (const BandSegment& s : bp.segs) words = std::max(words, s.nrows * ntiles * kBandWords + s.pre);
+    return round_up(std::min(words * 4, kBandBytesMax), 256);
+}
+
+}  // namespace aa

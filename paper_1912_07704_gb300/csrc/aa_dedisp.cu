@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "aa_internal.h"
+#include "aa_row_sums.cuh"
 
 namespace aa {
 namespace {
@@ -90,25 +91,6 @@ __device__ __forceinline__ uint32_t mad_add(uint32_t x, uint32_t one, uint32_t a
 
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
-// Fused statistics of the single-pulse search: the warp's exact sums of one
-// output row's samples (s1 = sum y, s2 = sum y^2 per lane; y < 2^24, at most
-// 16 samples a lane, so every partial fits in 64 bits) are added to the row's
-// accumulators acc = (sum y, sum y^2 low, sum y^2 high); a wrap of the low
-// word is carried into the high one, so the 128-bit total is exact.
-__device__ __forceinline__ void add_row_sums(unsigned long long* acc, unsigned long long s1,
-                                             unsigned long long s2) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&acc[0], s1);
-        const unsigned long long old = atomicAdd(&acc[1], s2);
-        if (old + s2 < old) atomicAdd(&acc[2], 1ull);
-    }
 }
 
 // One CTA's work item: DM block (bid % ndm_blocks) x time tile (bid / ndm_blocks).
@@ -918,6 +900,8 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     const int64_t ntiles = (a.length + kTau - 1) / kTau;
     const int64_t nblocks = (int64_t)ndmb * ntiles;
     if (nblocks >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    // (the staging-fault hook is one of the direct kernel)
+    if (bands_fit(a) && (a.grouped || g_fault_skip_chunk < 0)) return launch_bands(a, s);
     if (a.grouped) {
         auto kern = a.elem == 1 ? (a.gflush == 0 ? dedisperse_grouped_kernel<1, true> : dedisperse_grouped_kernel<1, false>)
                                 : (a.gflush == 0 ? dedisperse_grouped_kernel<2, true> : dedisperse_grouped_kernel<2, false>);

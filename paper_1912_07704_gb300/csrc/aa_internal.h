@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/aa_dedisp.h"
+#include "aa_bands.h"
 
 namespace aa {
 
@@ -160,6 +161,8 @@ struct RangePlan {
     GroupMember* d_gmem = nullptr;
     SubbandPlan sb;        // valid once aa_plan_set_subband chose it (strategy 2)
     FdmtPlan fd;           // valid once aa_plan_set_fdmt chose it (strategy 3)
+    BandPlan bands;        // band rows (ok: tables exist and pay)
+    bool pinned = false;   // the strategy was set or tuned, not the plan's own choice
 };
 
 }  // namespace aa
@@ -203,7 +206,10 @@ struct Layout {
     // FDMT ranges: two 32-bit depth buffers of fdmt_rows rows at pitch
     // fdmt_pitch (bytes into the workspace; -1 when no range uses FDMT)
     int64_t fdmt_offset = -1, fdmt_pitch = 0, fdmt_rows = 0;
-    int64_t dedisp_ws = 0;
+    // [.. dedisp_base) is what the call cannot do without; behind it the row
+    // buffer of the ranges' bands (a call with less scratch takes the grouped
+    // or the direct kernel)
+    int64_t dedisp_base = 0, dedisp_ws = 0;
     // single-pulse workspace: [error word + chunk counter][1/sqrt(w)][row stats]
     //                         [width tables][candidate chunk headers]
     int32_t max_width = 0;
@@ -296,7 +302,27 @@ struct DedispArgs {
     // fused statistics (non-NULL): each output row r adds its exact sums to
     // st_acc[3 r .. 3 r + 2] = (sum y, sum y^2 low 64 bits, high 64 bits)
     unsigned long long* st_acc;
+    // band rows (NULL or no row buffer: the strategy's kernel): the range's host
+    // tables, a row buffer of band_bytes, and the launch's first trial
+    const BandPlan* bands;
+    uint32_t* band_rows;
+    int64_t band_bytes;
+    int32_t trial0;
 };
+// Given a row buffer, a range runs on band rows where it has them, unless the
+// direct strategy was asked for.
+inline bool uses_bands(const RangePlan& r) { return r.bands.ok && (r.strategy == 1 || (r.strategy == 0 && !r.pinned)); }
+// Tables of a range's band rows; leaves r.bands.ok false where they do not
+// fit or would not pay.
+void build_bands(RangePlan& r, int nchans);
+constexpr int64_t kBandBytesMax = int64_t(2) << 30;  // row buffer asked for at most
+// bytes of the row buffer that `length` output samples take, kBandBytesMax at most
+int64_t band_bytes(const BandPlan& bp, int64_t length);
+// the delays [ndm][nchans] that the tables add up to, read back from them as
+// the kernels do; false if a table entry is inconsistent
+bool band_shifts(const BandPlan& bp, int nchans, int ndm, int32_t* out);
+bool bands_fit(const DedispArgs& a);  // a row buffer is there and large enough
+cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s);
 // Strategy fields of a range's kernel arguments.
 void fill_strategy(DedispArgs& a, const RangePlan& r);
 cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s);

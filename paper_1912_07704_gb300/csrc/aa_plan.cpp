@@ -278,6 +278,7 @@ void fill_strategy(DedispArgs& a, const RangePlan& r) {
         a.gdesc = nullptr;
         a.gmem = nullptr;
     }
+    a.bands = uses_bands(r) ? &r.bands : nullptr;
 }
 
 static aa_status build_strategy(aa_plan& p) {
@@ -332,6 +333,7 @@ static aa_status build_strategy(aa_plan& p) {
         // channel and trial (measured break-even well above 0.6).
         build_groups(r, C);
         r.strategy = (r.grouped_ok && r.gwork <= 0.6) ? 1 : 0;
+        build_bands(r, C);
     }
     // decimation cascade: each decimated buffer is built from the largest
     // already-built decimation that divides it (or from the raw input).
@@ -393,7 +395,11 @@ Layout make_layout(const aa_plan& p, int64_t nsamp, int32_t max_width) {
         L.fdmt_offset = ws;
         ws += 2 * round_up(L.fdmt_rows * L.fdmt_pitch * 4, 256);
     }
-    L.dedisp_ws = ws;  // always holds at least the error word
+    L.dedisp_base = ws;  // always holds at least the error word
+    int64_t rows = 0;
+    for (size_t q = 0; q < p.ranges.size(); ++q)
+        if (uses_bands(p.ranges[q])) rows = std::max(rows, band_bytes(p.ranges[q].bands, L.length[q]));
+    L.dedisp_ws = ws + rows;
     L.max_width = max_width;
     if (max_width > 0) {
         L.wpad = (int32_t)round_up(max_width, kSpsSlots);
@@ -581,6 +587,12 @@ aa_status aa_plan_create(const aa_plan_desc* d, aa_plan** out) {
         p->table_bytes += round_up((int64_t)r.grec.size() * sizeof(GroupRec), 256);
         p->table_bytes += round_up((int64_t)r.gdesc.size() * sizeof(GroupDesc), 256);
         p->table_bytes += round_up((int64_t)r.gmem.size() * sizeof(GroupMember), 256);
+        p->table_bytes += round_up((int64_t)r.bands.rows.size() * sizeof(BandRow), 256);
+        p->table_bytes += round_up((int64_t)r.bands.quads.size() * sizeof(BandQuad), 256);
+        p->table_bytes += round_up((int64_t)r.bands.infos.size() * sizeof(BandInfo), 256);
+        p->table_bytes += round_up((int64_t)r.bands.copies.size() * sizeof(BandCopy), 256);
+        p->table_bytes += round_up((int64_t)r.bands.heads.size() * sizeof(BandHead), 256);
+        p->table_bytes += round_up((int64_t)r.bands.offs.size() * 2, 256);
     }
     *out = p;
     return AA_OK;
@@ -631,6 +643,13 @@ aa_status aa_plan_bind(aa_plan* p, int device) {
         r.d_grec = (GroupRec*)upload(r.grec.data(), r.grec.size() * sizeof(GroupRec));
         r.d_gdesc = (GroupDesc*)upload(r.gdesc.data(), r.gdesc.size() * sizeof(GroupDesc));
         r.d_gmem = (GroupMember*)upload(r.gmem.data(), r.gmem.size() * sizeof(GroupMember));
+        BandPlan& bp = r.bands;
+        bp.d_rows = (const BandRow*)upload(bp.rows.data(), bp.rows.size() * sizeof(BandRow));
+        bp.d_quads = (const BandQuad*)upload(bp.quads.data(), bp.quads.size() * sizeof(BandQuad));
+        bp.d_infos = (const BandInfo*)upload(bp.infos.data(), bp.infos.size() * sizeof(BandInfo));
+        bp.d_copies = (const BandCopy*)upload(bp.copies.data(), bp.copies.size() * sizeof(BandCopy));
+        bp.d_heads = (const BandHead*)upload(bp.heads.data(), bp.heads.size() * sizeof(BandHead));
+        bp.d_offs = (const uint16_t*)upload(bp.offs.data(), bp.offs.size() * 2);
         if (e != cudaSuccess) break;
     }
     if (e != cudaSuccess) {
@@ -742,6 +761,7 @@ aa_status aa_plan_set_strategy(aa_plan* p, int32_t r, int32_t strategy) {
         return AA_ERR_CONFIG;
     }
     g.strategy = strategy;
+    g.pinned = true;
     return AA_OK;
 }
 
@@ -1037,6 +1057,11 @@ aa_status aa_plan_effective_shifts(const aa_plan* p, int32_t r, int32_t* out, in
         };
         for (int32_t i = 0; i < ndm; ++i) walk(walk, 0, i, 0, out + (int64_t)i * C);
         return AA_OK;
+    }
+    if (uses_bands(g)) {
+        if (band_shifts(g.bands, C, ndm, out)) return AA_OK;
+        set_error("internal: inconsistent band tables");
+        return AA_ERR_STATE;
     }
     std::memcpy(out, g.shifts.data(), g.shifts.size() * 4);
     return AA_OK;

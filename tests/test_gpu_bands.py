@@ -1,0 +1,54 @@
+"""Band rows of the grouped strategy against the direct kernel (bit for bit):
+last bands of 1 to 8 channels, parts of blocks and segments, one tile and
+several slabs, both halves of a word past the series end, and the least
+scratch, with which the grouped kernel runs instead."""
+import pytest
+import torch
+
+from paper_1912_07704_gb300 import abi, synth
+from paper_1912_07704_gb300.api import Plan
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # nchans, foff, ranges, output samples of the first range
+    (1024, -300.0 / 1024, ((0.0, 0.1, 600, 1), (60.0, 0.2, 70, 2)), 1),
+    (1001, -0.3, ((0.0, 0.1, 65, 1), (7.0, 0.1, 513, 3)), 511),
+    (1004, -0.3, ((3.0, 0.2, 64, 1), (300.0, 0.5, 100, 4)), 513),
+    (1005, -0.3, ((0.0, 0.05, 1025, 1),), 20001),
+    (1007, -0.3, ((0.0, 0.0, 70, 1), (50.0, 0.3, 200, 16)), 33000),
+    (800, 0.375, ((0.0, 0.1, 300, 1), (30.0, 0.4, 150, 5)), 12345),  # rising band
+    (4096, -300.0 / 4096, ((0.0, 0.1, 130, 1), (600.0, 1.0, 66, 8)), 40000),
+]
+
+
+def _run(plan, x, nsamp, ws_bytes):
+    out = torch.full((plan.query(nsamp).dd_elems,), -1.0, device="cuda")
+    ws = torch.full((ws_bytes,), 0xA5, dtype=torch.uint8, device="cuda")  # the row buffer starts as garbage
+    abi.aa_dedisperse_device(plan.handle, x.data_ptr(), nsamp, x.stride(0), out.data_ptr(), ws.data_ptr(), ws.numel(),
+                             torch.cuda.current_stream().cuda_stream)
+    abi.aa_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    return out
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+@pytest.mark.parametrize("data", ["noise", "saturated"])
+def test_bands_equal_the_direct_kernel(case, data):
+    C, foff, ranges, length = CASES[case]
+    plan = Plan(C, 1508.0 if foff < 0 else 1208.0, foff, 64e-6, ranges)
+    nsamp = length + int(plan.shifts(0).max())
+    plan.bind()
+    x, n = plan.device_input(synth.noise_filterbank(C, nsamp, 31 + case, device="cuda"))
+    if data == "saturated":  # the largest sums in every 16-bit lane, and whatever lies behind the rows' ends
+        x.fill_(255)
+    for r in range(len(ranges)):
+        plan.set_strategy(r, abi.AA_DEDISP_DIRECT)
+    base = plan.query(n).dedisp_ws_bytes
+    want = _run(plan, x, n, base)
+    for r in range(len(ranges)):
+        plan.set_strategy(r, abi.AA_DEDISP_GROUPED)
+    full = plan.query(n).dedisp_ws_bytes
+    assert full > base
+    for nbytes in (full, base + (full - base) // 3, base):
+        got = _run(plan, x, n, nbytes)
+        for a, b in zip(plan.range_views(got, n), plan.range_views(want, n)):
+            assert torch.equal(a, b), nbytes
