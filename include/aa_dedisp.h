@@ -394,7 +394,8 @@ aa_status aa_plan_autotune(aa_plan* plan, int64_t nsamp_probe, const char* cache
 /* Many independent beams (each with its own plan and length) searched by one
  * CUDA graph.  Beams are grouped into waves whose working set fits
  * wave_budget_bytes (<= 0: half of the free device memory) and waves reuse
- * one buffer region; within a wave the graph issues each beam's kernels on 8
+ * one buffer region (beside it 8 row buffers of at most 256 MiB each and the
+ * region's size in all, where memory allows); within a wave the graph issues each beam's kernels on 8
  * concurrent branches (see aa_batch_set_branches for the other form).
  * Plans are bound to the current device if needed; they must stay alive
  * while the batch exists.  The library allocates all device memory at
@@ -608,8 +609,9 @@ void aa_candidates_destroy(aa_candidates* c);
  * aa_plan_query dd_elems x 4 bytes of the unfused path, and the largest
  * decimated input replaces all of them.
  * aa_search_fused_device: d_in as in aa_dedisperse_device; candidates as in
- * aa_sps_search_device; d_ws 256-byte aligned, >= the bytes above.  Its
- * first word is the error word (aa_workspace_status).  Stream-ordered.
+ * aa_sps_search_device; d_ws 256-byte aligned, >= the bytes above (for plans
+ * whose decimated inputs leave little room for a row buffer these include up
+ * to 512 MiB for one, without which the call runs slower).  Its first word is the error word (aa_workspace_status).  Stream-ordered.
  * AA_ERR_CONFIG for plans with sub-band or FDMT ranges; AA_ERR_ARG on bad
  * arguments. */
 aa_status aa_search_fused_ws_bytes(const aa_plan* plan, int64_t nsamp, int32_t max_width,

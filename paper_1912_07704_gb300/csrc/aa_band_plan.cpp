@@ -317,12 +317,22 @@ void build_bands(RangePlan& r, int C) {
     if (best.ok && best.cost < 0.6 * direct) r.bands = std::move(best);
 }
 
-int64_t band_bytes(const BandPlan& bp, int64_t length) {
-    if (!bp.ok || length <= 0) return 0;
-    const int64_t ntiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
+static int64_t bytes_for(const BandPlan& bp, int64_t ntiles) {
     int64_t words = 0;
     for (const BandSegment& s : bp.segs) words = std::max(words, s.nrows * ntiles * kBandWords + s.pre);
     return round_up(std::min(words * 4, kBandBytesMax), 256);
+}
+
+int64_t band_bytes(const BandPlan& bp, int64_t length) {
+    if (!bp.ok || length <= 0) return 0;
+    return bytes_for(bp, (length + 2 * kBandWords - 1) / (2 * kBandWords));
+}
+
+int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials) {
+    if (!bp.ok || length <= 0) return 0;
+    const int64_t nblk = std::max(1, trials / kBandTrials);
+    const int64_t tiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
+    return bytes_for(bp, std::min<int64_t>(tiles, (2 * 152 + nblk - 1) / nblk));
 }
 
 }  // namespace aa

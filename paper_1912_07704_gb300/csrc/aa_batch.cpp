@@ -34,6 +34,7 @@ aa_status fail(cudaError_t e, const char* what) {
 // branches the batch runs at 1.00x and 1.05x the speed of the same beams
 // issued one after another; the persistent work-queue form at 0.96x / 0.97x.
 constexpr int kDefaultBranches = 8;
+constexpr int64_t kBranchRowsMax = int64_t(256) << 20;
 
 struct WaveTables {
     // host copies (uploaded into the arena)
@@ -92,6 +93,8 @@ struct aa_batch {
     std::vector<std::vector<DedispArgs>> beam_dd;
     std::vector<std::vector<SpsArgs>> beam_sps;
     std::vector<char*> beam_dec_ws;
+    char* rows = nullptr;    // row buffers of the branches' band rows (branched form), shared out evenly
+    int64_t rows_bytes = 0;
     std::vector<double> beam_work;  // channel-adds + boxcar samples, for dealing beams to branches
 };
 
@@ -105,7 +108,7 @@ struct BeamNeeds {
 BeamNeeds beam_needs(const aa_plan& p, int64_t nsamp, int32_t W) {
     const Layout L = make_layout(p, nsamp, W);
     BeamNeeds n;
-    n.dec_bytes = round_up(L.dedisp_ws, 256);
+    n.dec_bytes = round_up(L.dedisp_base, 256);
     n.dd_bytes = round_up(L.dd_elems * 4, 256);
     n.sps_bytes = round_up((int64_t)p.ndm_total * (int64_t)sizeof(RowStats), 256) +
                   round_up((int64_t)p.ndm_total * L.wpad * 8, 256);
@@ -123,13 +126,17 @@ void free_batch(aa_batch* b) {
 // One beam's stages as the single-beam path issues them: decimation cascade,
 // one dedispersion launch per range, then statistics and boxcar + peaks per
 // range.
-cudaError_t issue_beam(const aa_batch* b, int bi, cudaStream_t s) {
+cudaError_t issue_beam(const aa_batch* b, int bi, int branch, cudaStream_t s) {
     const aa_plan& pl = *b->plans[bi];
     const Layout L = make_layout(pl, b->nsamps[bi], b->max_width);
     const uint8_t* d_in = reinterpret_cast<const uint8_t*>(b->arena + b->in_offset[bi]);
     cudaError_t e = launch_decimation_cascade(pl, L, d_in, b->in_pitch[bi], b->beam_dec_ws[bi], s);
-    for (const DedispArgs& a : b->beam_dd[bi])
+    const int64_t per = b->rows_bytes / std::max(b->branches, 1) / 256 * 256;
+    for (DedispArgs a : b->beam_dd[bi]) {
+        a.band_rows = reinterpret_cast<uint32_t*>(b->rows + branch * per);
+        a.band_bytes = per;
         if (e == cudaSuccess) e = launch_dedisperse(a, s);
+    }
     for (const SpsArgs& a : b->beam_sps[bi]) {
         if (e == cudaSuccess) e = launch_sps_stats(a, s);
         if (e == cudaSuccess) e = launch_sps_boxcar(a, s);
@@ -190,7 +197,7 @@ cudaError_t capture_graph(aa_batch* b) {
             for (int k = 0; k < nbr; ++k) {
                 if (lanes[k].empty()) continue;
                 chk(cudaStreamWaitEvent(bs[k], ev[nbr], 0));
-                for (int bi : lanes[k]) chk(issue_beam(b, bi, bs[k]));
+                for (int bi : lanes[k]) chk(issue_beam(b, bi, k, bs[k]));
                 chk(cudaEventRecord(ev[k], bs[k]));
                 chk(cudaStreamWaitEvent(cs, ev[k], 0));  // join
             }
@@ -305,8 +312,26 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
     const int64_t cand_bytes = round_up(cand_capacity * (int64_t)sizeof(aa_candidate), 256);
     const int64_t chunk_bytes = round_up(b->chunk_cap * (int64_t)sizeof(CandChunk), 256);
     const int64_t small_bytes = 256 + 256 + round_up((int64_t)b->wpad * 8, 256);
-    b->arena_bytes = (size_t)(in_bytes + wave_bytes + table_bytes + cand_bytes + chunk_bytes + small_bytes);
+    // row buffers: what keeps a branch's launches busy, kBranchRowsMax a branch
+    // and the waves' working set in all at most; without memory for them the
+    // beams run on the grouped and direct kernels
+    int64_t rows = 0;
+    for (int i = 0; i < nbeams; ++i) {
+        const Layout L = make_layout(*plans[i], nsamps[i], max_width);
+        for (size_t r = 0; r < plans[i]->ranges.size(); ++r)
+            if (uses_bands(plans[i]->ranges[r]))
+                rows = std::max(rows, band_bytes_busy(plans[i]->ranges[r].bands, L.length[r], plans[i]->ranges[r].desc.ndm));
+    }
+    rows = std::min({rows, kBranchRowsMax, wave_bytes / kDefaultBranches / 256 * 256}) * kDefaultBranches;
+    const size_t least = (size_t)(in_bytes + wave_bytes + table_bytes + cand_bytes + chunk_bytes + small_bytes);
+    b->arena_bytes = least + (size_t)rows;
     cudaError_t e = cudaMalloc(&b->arena, b->arena_bytes);
+    if (e != cudaSuccess && rows > 0) {
+        cudaGetLastError();
+        rows = 0;
+        b->arena_bytes = least;
+        e = cudaMalloc(&b->arena, b->arena_bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("batch needs %zu device bytes: %s", b->arena_bytes, cudaGetErrorString(e));
@@ -317,6 +342,9 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
     p += in_bytes;  // beam inputs first (aa_batch_input)
     char* wave_area = p;
     p += wave_bytes;
+    b->rows = p;
+    b->rows_bytes = rows;
+    p += rows;
     b->d_cands = reinterpret_cast<aa_candidate*>(p);
     p += cand_bytes;
     b->d_chunks = reinterpret_cast<CandChunk*>(p);

@@ -900,8 +900,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     const int64_t ntiles = (a.length + kTau - 1) / kTau;
     const int64_t nblocks = (int64_t)ndmb * ntiles;
     if (nblocks >= (1ll << 31)) return cudaErrorInvalidConfiguration;
-    // (the staging-fault hook is one of the direct kernel)
-    if (bands_fit(a) && (a.grouped || g_fault_skip_chunk < 0)) return launch_bands(a, s);
+    if (bands_fit(a)) return launch_bands(a, s);
     if (a.grouped) {
         auto kern = a.elem == 1 ? (a.gflush == 0 ? dedisperse_grouped_kernel<1, true> : dedisperse_grouped_kernel<1, false>)
                                 : (a.gflush == 0 ? dedisperse_grouped_kernel<2, true> : dedisperse_grouped_kernel<2, false>);

@@ -45,8 +45,14 @@ struct FusedLayout {
     Layout L;
     int32_t stripe = 0;
     int64_t stripe_pitch = 0;  // floats per stripe row (the widest range's pitch)
-    int64_t dec_offset = 0, sps_offset = 0, stripe_offset = 0, acc_offset = 0, bytes = 0;
+    int64_t dec_offset = 0, sps_offset = 0, stripe_offset = 0, acc_offset = 0;
+    // base: what the call cannot do without.  The band rows' buffer is the
+    // part of the decimated input's region that the range leaves free; where
+    // that is small, a row buffer of its own behind base (at most
+    // kRowBufferMax; a call with less scratch does without it).
+    int64_t dec_bytes = 0, base = 0, bytes = 0;
 };
+constexpr int64_t kRowBufferMax = int64_t(512) << 20;
 
 aa_status fused_layout(const aa_plan& p, int64_t nsamp, int32_t max_width, int32_t stripe, FusedLayout& f) {
     if (stripe == 0) stripe = kDefaultStripe;
@@ -67,15 +73,29 @@ aa_status fused_layout(const aa_plan& p, int64_t nsamp, int32_t max_width, int32
     int64_t dec_bytes = 0;
     for (size_t k = 0; k < p.decs.size(); ++k)
         dec_bytes = std::max(dec_bytes, (int64_t)p.nchans * f.L.dec_pitch[k] * 2);
+    f.dec_bytes = round_up(dec_bytes, 256);
     f.dec_offset = kErrBlock;
-    f.sps_offset = f.dec_offset + round_up(dec_bytes, 256);
+    f.sps_offset = f.dec_offset + f.dec_bytes;
     f.stripe_offset = f.sps_offset + round_up(f.L.sps_ws, 256);
     f.acc_offset = f.stripe_offset + round_up((int64_t)f.stripe * f.stripe_pitch * 4, 256);
-    f.bytes = f.acc_offset + round_up((int64_t)f.stripe * 3 * 8, 256);
+    f.base = f.acc_offset + round_up((int64_t)f.stripe * 3 * 8, 256);
+    int64_t rows = 0;
+    for (size_t r = 0; r < p.ranges.size(); ++r)
+        if (uses_bands(p.ranges[r]))
+            rows = std::max(rows, std::min(kRowBufferMax, band_bytes_busy(p.ranges[r].bands, f.L.length[r], f.stripe)));
+    f.bytes = f.base + (rows > f.dec_bytes ? rows : 0);
     return AA_OK;
 }
 
 }  // namespace
+
+aa_status aa::fused_bytes(const aa_plan& p, int64_t nsamp, int32_t max_width, int64_t& least, int64_t& full) {
+    FusedLayout f;
+    const aa_status st = fused_layout(p, nsamp, max_width, 0, f);
+    least = f.base;
+    full = f.bytes;
+    return st;
+}
 
 extern "C" {
 
@@ -116,8 +136,8 @@ aa_status aa_search_fused_device(const aa_plan* p, const uint8_t* d_in, int64_t 
     aa_status st = fused_layout(*p, nsamp, max_width, stripe_trials, f);
     if (st != AA_OK) return st;
     const Layout& L = f.L;
-    if (!d_ws || (int64_t)ws_bytes < f.bytes) {
-        set_error("workspace %zu bytes < required %lld", ws_bytes, (long long)f.bytes);
+    if (!d_ws || (int64_t)ws_bytes < f.base) {
+        set_error("workspace %zu bytes < required %lld", ws_bytes, (long long)f.base);
         return AA_ERR_ARG;
     }
     if (reinterpret_cast<uintptr_t>(d_ws) % 256 || (d_in && reinterpret_cast<uintptr_t>(d_in) % 16) ||
@@ -159,7 +179,44 @@ aa_status aa_search_fused_device(const aa_plan* p, const uint8_t* d_in, int64_t 
         const int C = p->nchans;
         const void* in = d_in;
         int64_t pitch_in = in_pitch;
-        if (g.desc.dec > 1) {  // this range's decimated input, from the 8-bit input
+        // (163072 samples of 4096 channels, four ranges: dedispersion 48.0 -> 29.1
+        // ms; a stripe builds the rows of its own trials, which takes over half
+        // of that.)
+        // Row buffer: what the range's decimated input leaves of its region, or
+        // the scratch behind base.  Where neither keeps the SMs busy, the row
+        // kernel decimates the 8-bit input itself and the whole region is the
+        // buffer (it reads dec bytes a sample for 2, stripe by stripe).
+        char* dec_region = ws + f.dec_offset;
+        char* row_buf = ws + f.base;
+        int64_t row_bytes = (int64_t)ws_bytes - f.base;
+        int32_t row_dec = 0;
+        if (uses_bands(g)) {
+            int64_t used = 0;
+            if (g.desc.dec > 1) {
+                const size_t k = std::find(p->decs.begin(), p->decs.end(), g.desc.dec) - p->decs.begin();
+                used = round_up((int64_t)C * L.dec_pitch[k] * 2, 256);
+            }
+            const int64_t busy = band_bytes_busy(g.bands, L.length[r], f.stripe);
+            if (f.dec_bytes - used > row_bytes) {
+                row_buf = dec_region + used;
+                row_bytes = f.dec_bytes - used;
+            }
+            if (g.desc.dec > 1 && row_bytes < busy && row_bytes < f.dec_bytes) {
+                DedispArgs t{};
+                t.length = L.length[r];
+                t.ndm = g.desc.ndm;
+                t.grouped = g.strategy == 1;
+                t.bands = &g.bands;
+                t.band_rows = reinterpret_cast<uint32_t*>(dec_region);
+                t.band_bytes = f.dec_bytes;
+                if (bands_fit(t)) {
+                    row_buf = dec_region;
+                    row_bytes = f.dec_bytes;
+                    row_dec = g.desc.dec;
+                }
+            }
+        }
+        if (g.desc.dec > 1 && row_dec == 0) {  // this range's decimated input, from the 8-bit input
             const size_t k = std::find(p->decs.begin(), p->decs.end(), g.desc.dec) - p->decs.begin();
             uint16_t* xd = reinterpret_cast<uint16_t*>(ws + f.dec_offset);
             ProfScope prof(kKDecimate, s);
@@ -184,6 +241,10 @@ aa_status aa_search_fused_device(const aa_plan* p, const uint8_t* d_in, int64_t 
             a.out_pitch = L.pitch[r];
             fill_strategy(a, g);
             a.err = err;
+            a.band_rows = reinterpret_cast<uint32_t*>(row_buf);
+            a.band_bytes = row_bytes;
+            a.trial0 = s0;
+            a.row_dec = row_dec;
             a.dmb0 = s0 / kDmPerBlock;
             a.st_acc = fused_stats ? acc : nullptr;
             {

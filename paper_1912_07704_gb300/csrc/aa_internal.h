@@ -308,6 +308,9 @@ struct DedispArgs {
     uint32_t* band_rows;
     int64_t band_bytes;
     int32_t trial0;
+    // > 1: `in` is the 8-bit input (in_pitch bytes) and the row kernel sums
+    // row_dec samples as it reads it; only for launches that bands_fit takes
+    int32_t row_dec;
 };
 // Given a row buffer, a range runs on band rows where it has them, unless the
 // direct strategy was asked for.
@@ -318,6 +321,9 @@ void build_bands(RangePlan& r, int nchans);
 constexpr int64_t kBandBytesMax = int64_t(2) << 30;  // row buffer asked for at most
 // bytes of the row buffer that `length` output samples take, kBandBytesMax at most
 int64_t band_bytes(const BandPlan& bp, int64_t length);
+// bytes with which launches of `trials` trials keep the SMs busy: two CTAs
+// each, or the whole length where that is less
+int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials);
 // the delays [ndm][nchans] that the tables add up to, read back from them as
 // the kernels do; false if a table entry is inconsistent
 bool band_shifts(const BandPlan& bp, int nchans, int ndm, int32_t* out);
@@ -330,6 +336,9 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s);
 cudaError_t launch_decimate(const void* in, int in_elem, int64_t in_pitch, int32_t nchans,
                             int64_t nout, int factor, uint16_t* out, int64_t out_pitch,
                             cudaStream_t s);
+// Workspace of aa_search_fused_device with the default stripes: the least it
+// accepts, and what aa_search_fused_ws_bytes asks for.
+aa_status fused_bytes(const aa_plan& p, int64_t nsamp, int32_t max_width, int64_t& least, int64_t& full);
 // Every decimated input of the plan into the dedispersion workspace `ws`
 // (layout L), each built from the largest decimation dividing it.
 cudaError_t launch_decimation_cascade(const aa_plan& p, const Layout& L, const uint8_t* d_in, int64_t in_pitch,

@@ -104,7 +104,7 @@ struct aa_server {
     // fused dedispersion -> search (aa_search_fused_device) when the plan
     // allows it: a slot then holds one stripe of series, not every row
     bool fused = false;
-    size_t fused_ws = 0;
+    size_t ws_bytes = 0;  // of a slot's dd_ws
 };
 
 namespace {
@@ -132,12 +132,12 @@ aa_status launch_chunk(aa_server& s, Slot& sl, Request& r) {
             "chunk upload");
     if (s.fused) {
         const aa_status e = aa_search_fused_device(s.plan, dst, len, s.pitch, s.W, s.thr, 0, sl.cands, s.cap,
-                                                   sl.count, nullptr, sl.dd_ws, s.fused_ws,
+                                                   sl.count, nullptr, sl.dd_ws, s.ws_bytes,
                                                    reinterpret_cast<aa_stream_t>(st));
         if (e != AA_OK) return e;
     } else {
         const Layout L = make_layout(*s.plan, len, s.W);
-        aa_status e = aa_dedisperse_device(s.plan, dst, len, s.pitch, sl.dd, sl.dd_ws, (size_t)L.dedisp_ws,
+        aa_status e = aa_dedisperse_device(s.plan, dst, len, s.pitch, sl.dd, sl.dd_ws, s.ws_bytes,
                                            reinterpret_cast<aa_stream_t>(st));
         if (e != AA_OK) return e;
         e = aa_sps_search_device(s.plan, len, sl.dd, s.W, s.thr, sl.cands, s.cap, sl.count, nullptr,
@@ -251,9 +251,14 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
     s->pitch = L.in_pitch_min;
     // resident state: two block buffers per beam
     const int64_t beam_bytes = 2 * (int64_t)plan->nchans * s->pitch;
-    s->fused = aa_search_fused_ws_bytes(plan, block, max_width, 0, &s->fused_ws, nullptr) == AA_OK;
+    int64_t least = 0, full = 0;  // dd_ws without and with its row buffer
+    s->fused = fused_bytes(*plan, block, max_width, least, full) == AA_OK;
     clear_error();  // plans with sub-band or FDMT ranges keep the unfused path
-    const int64_t work_bytes = s->fused ? (int64_t)s->fused_ws : L.dedisp_ws + L.dd_elems * 4 + L.sps_ws;
+    if (!s->fused) {
+        least = L.dedisp_base;
+        full = L.dedisp_ws;
+    }
+    const int64_t work_bytes = s->fused ? least : least + L.dd_elems * 4 + L.sps_ws;
     const int64_t slot_bytes = work_bytes + cand_capacity * (int64_t)sizeof(aa_candidate) + 4096;
     if (memory_budget <= 0) {
         size_t fr = 0, tot = 0;
@@ -268,6 +273,8 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
         delete s;
         return AA_ERR_NOMEM;
     }
+    // the slots' row buffers when the budget has room for all of them
+    s->ws_bytes = (size_t)(avail - nslots * slot_bytes >= nslots * (full - least) ? full : least);
     s->beams.resize(nbeams);
     for (auto& b : s->beams) {
         cudaError_t e = cudaMalloc(&b.buf[0], (size_t)plan->nchans * s->pitch);
@@ -280,9 +287,9 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
         cudaError_t e = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
         if (s->fused) {  // one fused workspace per slot
-            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, std::max<size_t>(s->fused_ws, 256));
+            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, std::max<size_t>(s->ws_bytes, 256));
         } else {
-            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, (size_t)L.dedisp_ws);
+            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, s->ws_bytes);
             if (e == cudaSuccess) e = cudaMalloc(&sl.dd, (size_t)std::max<int64_t>(L.dd_elems * 4, 256));
             if (e == cudaSuccess) e = cudaMalloc(&sl.sps_ws, (size_t)L.sps_ws);
         }

@@ -52,3 +52,32 @@ def test_bands_equal_the_direct_kernel(case, data):
         got = _run(plan, x, n, nbytes)
         for a, b in zip(plan.range_views(got, n), plan.range_views(want, n)):
             assert torch.equal(a, b), nbytes
+
+
+@pytest.mark.parametrize("stripe", [16, 64, 0])
+def test_bands_in_the_fused_search(stripe):
+    """Stripes on band rows (every decimation, read from the decimated input
+    or decimated by the row kernel; row sums added by its epilogue) give the
+    unfused direct path's candidates and B(t); also with the least scratch."""
+    from paper_1912_07704_gb300.api import candidates_from_device
+    C, nsamp, W, thr, cap = 1003, 30011, 24, 4.5, 1 << 18
+    ranges = ((0.0, 0.1, 70, 1), (10.0, 0.2, 64, 2), (30.0, 0.5, 40, 3), (60.0, 1.0, 64, 4), (100.0, 1.0, 64, 8), (160.0, 2.0, 70, 16))
+    plan = Plan(C, 1508.0, -0.3, 64e-6, ranges)
+    x, n = plan.device_input(synth.noise_filterbank(C, nsamp, 77, device="cuda"))
+    for r in range(len(ranges)):
+        plan.set_strategy(r, abi.AA_DEDISP_DIRECT)
+    least = plan.fused_ws_bytes(n, W, stripe)[0]
+    dd = plan.dedisperse_device(x, n)
+    snr = torch.zeros_like(dd)
+    c, count, _ = plan.sps_search_device(dd, n, W, thr, cap, snr_out=snr)
+    want = candidates_from_device(c, count, cap)
+    assert len(want) > 0
+    for r in range(len(ranges)):
+        plan.set_strategy(r, abi.AA_DEDISP_GROUPED)
+    for nbytes in (plan.fused_ws_bytes(n, W, stripe)[0], plan.fused_ws_bytes(n, W, stripe)[0] + (64 << 20), least):
+        got = torch.zeros_like(dd)
+        ws = torch.full((nbytes,), 0x5A, dtype=torch.uint8, device="cuda")
+        c, count, _ = plan.search_fused_device(x, n, W, thr, cap, stripe, snr_out=got, ws=ws)
+        assert (candidates_from_device(c, count, cap) == want).all()
+        for a, b in zip(plan.range_views(got, n), plan.range_views(snr, n)):
+            assert torch.equal(a, b)
