@@ -247,8 +247,9 @@ aa_status aa_sps_search_device(const aa_plan* plan, int64_t nsamp, const float* 
                                aa_stream_t stream);
 
 /* Width-samples the last aa_sps_search_device call on this workspace actually
- * evaluated (width blocks whose SNR bound is below the threshold are skipped
- * when no B(t) output is requested).  Synchronises `stream`. */
+ * evaluated (chunks of 16 widths in which a thread's 16 starts can reach
+ * neither their running maximum nor, when no B(t) output is requested, the
+ * threshold are skipped).  Synchronises `stream`. */
 aa_status aa_sps_workspace_work(const void* d_ws, aa_stream_t stream, int64_t* evaluated);
 
 /* Read and clear the device error word kept at the start of a workspace used

@@ -303,47 +303,47 @@ __device__ long long block_exclusive_scan_total(long long v, long long* scratch,
     return ex;
 }
 
-// Block-wide exclusive scan of one int64 `run` per thread, together with the
-// block total and the smallest and largest prefix value min(before + mn) /
-// max(before + mx) (mn <= 0 <= mx relative to the thread's own start), in two
-// barriers.  scratch: 3 * NT / 32 entries.
+// Block-wide exclusive scan of one `run` per thread, together with the block
+// total and the smallest and largest prefix value before + mn / before + mx (mn
+// <= 0 <= mx relative to the thread's own start), in one barrier; a second use
+// needs one between.  Values are clamped on the way so that 32 bits hold every
+// sum (a thread's at 2^25 and 2^26, a warp's at 2^27 and 2^28): results whose
+// range stays within 2^24 are exact, and any clamp shows as a range beyond it.
+// scratch: 3 * NT / 32 entries.
 template <int NT>
-__device__ void block_scan_minmax(long long run, long long mn, long long mx, long long* scratch,
-                                  long long& before, long long& total, long long& gmn, long long& gmx) {
+__device__ __forceinline__ void block_scan_minmax(int run, int mn, int mx, int* scratch, int& before, int& total, int& gmn,
+                                                  int& gmx) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    long long inc = run;
+    auto clamp = [](int v, int m) { return max(-m, min(m, v)); };
+    run = clamp(run, 1 << 25);
+    int inc = run;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const long long u = __shfl_up_sync(0xffffffffu, inc, o);
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += u;
     }
-    const long long ex = inc - run;
-    long long lmn = ex + mn, lmx = ex + mx;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lmn = min(lmn, __shfl_xor_sync(0xffffffffu, lmn, o));
-        lmx = max(lmx, __shfl_xor_sync(0xffffffffu, lmx, o));
-    }
-    if (lane == 31) scratch[warp] = inc;
-    if (lane == 0) {
-        scratch[NW + warp] = lmn;
-        scratch[2 * NW + warp] = lmx;
+    const int ex = inc - run;
+    const int lmn = __reduce_min_sync(0xffffffffu, ex + clamp(mn, 1 << 26));
+    const int lmx = __reduce_max_sync(0xffffffffu, ex + clamp(mx, 1 << 26));
+    if (lane == 31) {
+        scratch[warp] = clamp(inc, 1 << 27);
+        scratch[NW + warp] = clamp(lmn, 1 << 28);
+        scratch[2 * NW + warp] = clamp(lmx, 1 << 28);
     }
     __syncthreads();
-    long long t = 0, wbase = 0, bmn = LLONG_MAX, bmx = LLONG_MIN;
+    int t = 0, wbase = 0;
+    gmn = INT_MAX;
+    gmx = INT_MIN;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-        bmn = min(bmn, t + scratch[NW + w]);
-        bmx = max(bmx, t + scratch[2 * NW + w]);
+        gmn = min(gmn, t + scratch[NW + w]);
+        gmx = max(gmx, t + scratch[2 * NW + w]);
         if (w == warp) wbase = t;
         t += scratch[w];
     }
     before = wbase + ex;
     total = t;
-    gmn = bmn;
-    gmx = bmx;
-    __syncthreads();  // scratch may be reused after this
 }
 
 template <int NT>
@@ -383,150 +383,287 @@ constexpr int NT = kSpsThreads;
 // it alone.
 constexpr float kBig = 1.2676506002282294e30f;  // 2^100
 
-// Block maxima of the prefix sums: Q[j] = max P[i] over i in
-// [kQSpan j, kQSpan (j+1)), for the pruning bounds of the wide widths.
-constexpr int kQSpan = 128;
-__host__ __device__ constexpr int sps_q_count(int wpad) {
-    return (kSpsTile + wpad + M + kQSpan - 1) / kQSpan;
-}
+// The width search of one thread's M starts.  Widths come in chunks of M
+// (chunk c: widths M c + 1 .. M c + M); chunk 0 is evaluated by every thread.
+// Of the others a thread evaluates those that can still raise the B of one of
+// its starts, each thread at its own chunk: before a bright pulse the 32
+// threads of a warp need 32 different widths, each of them few.
+//
+// Block maxima of P decide it: Q16[j] = max P over [16 j, 16 j + 16).  A window
+// of chunk c from a start p of thread t (p in [16 t, 16 t + 15]) ends in the
+// blocks t + c and t + c + 1, so
+//   SNR_w(p) <= (max of the two - pmin - w f) / (sigma sqrt(w)),  reaches(),
+// and the largest end of block t + c + 1 gives a window to every start, of
+// width M c + 1 .. M c + 31, so every start of the thread has
+//   B >= (Q16[t + c + 1] - pmax - w f) / (sigma sqrt(w)),         lower().
+// A first pass over the chunks takes the largest lower bound, a second one
+// evaluates the chunks whose upper bound reaches max(cut, that, the smallest
+// running B).  The passes go through the chunks together (the threads of a
+// warp at the same c, with sliding maxima over 2, 9 and 65 blocks: S1, S8,
+// S64): the first 8 chunks one by one, then groups of 8, from 64 on groups of
+// 64, opened where a thread's bound reaches its floor.  Eight bounds of one
+// level are computed side by side before the warp looks at them (one by one,
+// each with its vote, they took 330 cycles each).  A chunk to evaluate waits
+// until its thread has a second one.  Both are written down once, in one loop:
+// with an evaluation and bounds at each place that wants them the kernel
+// waited for instructions more than for anything else (2.6 of 10 stalls).
+// Skipping below
+// the running B, or below a lower bound of it, is exact for every start (such
+// a chunk changes neither B nor the first chunk that reaches it; the chunk
+// that the lower bound comes from is not skipped); below the threshold's cut
+// it is exact for every B >= threshold and for every peak decision.
+//
+// FP32 with the roundings covered: P's differences are exact integers, each
+// further step is within 2^-22 relative of |num| or of the drift |w f|
+// (|f| <= 1/2 since m0 = round(mu)); the factor 1 + 1.02e-4 in rs and the
+// margin S (1.02e-4 and the largest drift's part) bound them many times over.
+constexpr int kTabWidths = 1024;  // widths whose table entries are staged in shared memory
+__host__ __device__ constexpr int sps_tab_smem(int wpad) { return wpad < kTabWidths ? wpad : kTabWidths; }
+// entries of Q16 and of each sliding maximum (the end padded for the longest)
+__host__ __device__ constexpr int sps_q16(int wpad) { return (kSpsTile / M + wpad / M + 1 + 64 + 31) / 32 * 32; }
+// entries of rs: c <= the last chunk + 65, and what a pass reads as it begins
+// (chunks 64 k and the 64 after them, k < 8, whatever the last chunk)
+__host__ __device__ constexpr int sps_rs(int wpad) { return ((wpad / M + 66 > 513 ? wpad / M + 66 : 513) + 3) / 4 * 4; }
 
-// Bound of one thread's M starts over a width segment [w1, w2].  For a start
-// p in [ps, pl] (pl = ps + M - 1) and a width w, the window's end is p + w, so
-// S_w(p) <= P[end] - pmin and w >= max(w1, end - pl); -w f <= -wlo f (f >= 0)
-// or -w2 f (f < 0).  So SNR_w(p) <= (P[end] - pmin - drift) / (sigma sqrt(wlo))
-// for every end, maximised over the ends:
-//  * w1 <= kQSpan: the ends [ps + w1, pl + w2] read one by one (as aligned
-//    16-byte vectors from ps + w1 - 1, a superset), wlo = w1;
-//  * wider: per block j of Q overlapping the ends, Q[j] with
-//    wlo = max(w1, kQSpan j - pl).
-// FP32 with the rounding of each step bounded and added (|f| <= 1/2 since
-// m0 = round(mu); the differences of the exact integer sums P are exact;
-// rsqrtf within 2 ulp), then widened by 1e-4 relative and absolute.
-struct ThreadBound {
-    const float* Q;
-    float pmin;       // min of P over the thread's valid starts (FLT_MAX: none)
-    float f;          // mu - m0
-    float inv_sigma;
-    float cut;        // segments bounded below this are skipped (-FLT_MAX: none)
-    int max_width, ylen, nq, ps;
-    bool active;      // pruning enabled
+// A chunk's 16 table entries are 8 16-byte blocks; in shared memory block b of
+// chunk c lies at b ^ (c & 7), so that threads at neighbouring chunks read
+// different banks.
+__device__ __forceinline__ int tab_block(int c, int b) { return 8 * c + (b ^ (c & 7)); }
+
+struct WidthBounds {
+    const float* rs;   // rs[c] = (1 + 1.02e-4) / (sigma sqrt(M c + 1))
+    float pmin, pmax;  // of P over the thread's valid starts (pmin = FLT_MAX: none)
+    float f;           // mu - m0
+    float S;
+
+    // w of the smallest drift w f over chunks c .. c + n - 1, less M c
+    __device__ __forceinline__ float w_first(int n) const { return f >= 0.0f ? 1.0f : (float)(M * n); }
+    // can windows ending at prefix sums <= top reach F + S?  r = rs + first chunk, w = M (first chunk) + w_first;
+    // where F may be negative (LOW) the widest window bounds a negative sum
+    template <bool LOW>
+    __device__ __forceinline__ bool reaches(float top, float w, const float* r, int n, float F) const {
+        const float num = fmaf(-f, w, top - pmin);
+        if (LOW && num < 0.0f) return num * (r[n] * (1.0f - 2.1e-4f)) >= F;
+        return num * r[0] >= F;
+    }
+    // an SNR that every start reaches with an end of prefix sum q, widths M c + 1 .. M c + 31
+    __device__ __forceinline__ float lower(float q, int c) const {
+        const float num = fmaf(-f, (float)(f >= 0.0f ? M * c + 31 : M * c + 1), q - pmax);
+        return num > 0.0f ? num * (rs[c + 2] * (1.0f - 2.1e-4f)) - S : -FLT_MAX;
+    }
 };
 
-__device__ __forceinline__ float piece_bound(float top, const ThreadBound& b, int wlo, int whi) {
-    const float drift = b.f >= 0.0f ? (float)wlo * b.f : (float)whi * b.f;
-    const float diff = top - b.pmin;
-    const float rs = rsqrtf((float)wlo);
-    // 6 roundings of at most 2^-24 relative each on magnitudes <= |diff| + |drift|
-    const float slack = (fabsf(diff) + fabsf(drift)) * b.inv_sigma * rs * 1e-6f + 1e-6f;
-    return (diff - drift) * b.inv_sigma * rs + slack;
-}
-
-__device__ __forceinline__ float thread_segment_bound(const float* __restrict__ P, const ThreadBound& b,
-                                                      int w1, int w2) {
-    if (b.pmin == FLT_MAX) return -FLT_MAX;
-    const int pl = b.ps + M - 1;
-    const int hi = min(b.ylen - 1, pl + w2);
-    float ub;
-    if (w1 <= kQSpan) {
-        // ylen is a multiple of 4, so the last vector ends inside the staged series
-        float pmax = -FLT_MAX;
-        for (int e = (b.ps + w1 - 1) & ~3; e <= hi; e += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(P + e);
-            pmax = fmaxf(fmaxf(pmax, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-        }
-        ub = piece_bound(pmax, b, w1, w2);
-    } else {
-        ub = -FLT_MAX;
-        const int j1 = min(b.nq - 1, hi / kQSpan);
-        for (int j = (b.ps + w1) / kQSpan; j <= j1; ++j)
-            ub = fmaxf(ub, piece_bound(b.Q[j], b, max(w1, j * kQSpan - pl), w2));
+// Chunk at window base pw = P + first start + M c with its 16 table entries
+// (blocks tb[b ^ x]): the best SNR of each start.
+__device__ __forceinline__ void eval_chunk(const float* __restrict__ pw, const float4* tb, int x,
+                                           const float (&base)[M], float (&Bc)[M]) {
+    float win[2 * M];  // win[k] = P[p_thread + M c + k]
+#pragma unroll
+    for (int k = 0; k < 2 * M; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(pw + k);
+        win[k] = v.x; win[k + 1] = v.y; win[k + 2] = v.z; win[k + 3] = v.w;
     }
-    return ub + fabsf(ub) * 1e-4f + 1e-4f;
+#pragma unroll
+    for (int s = 0; s < M; s += 2) {
+        const float4 rc = tb[(s >> 1) ^ x];
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            const float v0 = fmaf(win[i + s + 1] - base[i], rc.x, rc.y);
+            const float v1 = fmaf(win[i + s + 2] - base[i], rc.z, rc.w);
+            Bc[i] = s == 0 ? fmaxf(v0, v1) : max3f(Bc[i], v0, v1);
+        }
+    }
 }
 
-// Main loop.  With pruning, the widths after the first chunk are checked in
-// power-of-two blocks [w0+1, 2 w0] (w0 = 16, 32, ...), and inside a block
-// that survives and spans more than 128 widths, in segments [w0+1, w0+128].
-// A thread can skip a block or segment when its bound is below max(cut, min
-// over its slots of the running B): below the running B it can change
-// neither B nor C of any of its slots (exact for every slot); below the
-// threshold cut it can only change sub-threshold values (exact for every
-// B >= threshold and for every peak decision).  The warp skips it when all
-// of its threads can (the warp evaluates chunks in lockstep; evaluating a
-// chunk a thread could skip changes nothing of the above).  Widths are
-// visited in increasing order, so the running B of the small widths prunes
-// the wide ones; a thread before a bright pulse evaluates the widths whose
-// windows end near the pulse, not the wider ones, whose bound the pulse's
-// SNR at the narrower width already exceeds.
-__device__ __forceinline__ int boxcar_prefix(const float* __restrict__ P,
-                                             const float2* __restrict__ tab, int wpad,
-                                             const float (&base)[M], const ThreadBound& bnd,
-                                             const uint32_t* lmask, float (&B)[M], int (&C)[M]) {
+// Without a threshold up to kEvery chunks are simply evaluated in turn: noise
+// leaves over a third of them to evaluate and the bounds cost more (B(t) of
+// 96 series of 64006 samples, W = 256 / 1024 / 2048: in turn 220 / 752 / 1449
+// us, by bounds 307 / 802 / 1084).
+constexpr int kEvery = kTabWidths / M;
+// Returns the chunks this thread evaluated.  C: the first chunk reaching B[i] in
+// 16-bit halves, starts 2 k and 2 k + 1 in C[k] (16 registers of them spilled).
+// Q: Q16, S1, S8 and S64, nq entries each.  LOW: cut is not above zero.
+template <bool LOW>
+__device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const float4* tab, const float2* __restrict__ gtab,
+                                             int nch, int max_width, const float (&base)[M], const WidthBounds& bnd,
+                                             const float* Q, int nq, float cut, const uint32_t* lmask, float (&B)[M],
+                                             uint32_t (&C)[M / 2]) {
+    const int t = threadIdx.x;
+    const float* pb = P + M * t;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        B[i] = -FLT_MAX;
+        C[i / 2] = 0;
+    }
+    if (LOW && nch <= kEvery) {
+        for (int c = 0; c < nch; ++c) {
+            if (lmask && !ladder_has(lmask, M * c + 1)) continue;
+            float Bc[M];
+            eval_chunk(pb + M * c, tab + 8 * c, c & 7, base, Bc);
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                if (Bc[i] > B[i]) {
+                    B[i] = Bc[i];
+                    C[i / 2] = __byte_perm(C[i / 2], (uint32_t)c, i & 1 ? 0x5410 : 0x3254);
+                }
+            }
+        }
+        return nch;
+    }
+    const float *s1 = Q + nq + t, *s8 = s1 + nq, *s64 = s8 + nq;
+    float F = cut - bnd.S;              // the floor less the bounds' margin
+    int evaluated = 0, pend = 0;        // pend: chunk waiting to be evaluated (-1: none), first chunk 0
+    bool last = nch == 1, found = false;
+    int pass = -1;
+    // Groups of 64 chunks from c512, of 8 from c64, chunks from c8: a thread's
+    // own (m..) and the warp's (u..) that reach the floor and are still to open.
+    unsigned m64 = 0, u64 = 0, m8 = 0, u8 = 0, in = 0;
+    int c512 = 0, c64 = 0, c8 = 0;
+    enum { kFirst, kEval, kBounds, kChunks } step = kEval;
+    int level = 1;        // chunks per bit of the next bounds
+    unsigned keep = ~0u;  // bits that the level above lets through
+    for (;;) {
+        if (step == kEval) {
+            if (pend >= 0) {
+                float Bc[M];
+                const bool staged = M * pend < kTabWidths;
+                eval_chunk(pb + M * pend, staged ? tab + 8 * pend : reinterpret_cast<const float4*>(gtab) + 8 * pend,
+                           staged ? pend & 7 : 0, base, Bc);
+                float low = FLT_MAX;  // smallest B over the valid starts (none: the floor is above every bound)
+#pragma unroll
+                for (int i = 0; i < M; ++i) {
+                    if (Bc[i] > B[i]) {  // strict: an equal later chunk keeps the earlier one
+                        B[i] = Bc[i];
+                        C[i / 2] = __byte_perm(C[i / 2], (uint32_t)pend, i & 1 ? 0x5410 : 0x3254);
+                    }
+                    low = fminf(low, base[i] < kBig ? B[i] : FLT_MAX);
+                }
+                F = fmaxf(F, low - bnd.S);
+                ++evaluated;
+                pend = -1;
+            }
+            if (last) break;
+            step = pass < 0 ? kFirst : kBounds;
+        }
+        if (step == kFirst) {  // a pass begins: chunks 1-7, groups of 8 up to 63, groups of 64 up to 511, side by side
+            ++pass;
+            in = m8 = m64 = 0;
+            const float w1 = bnd.w_first(1), w8 = bnd.w_first(8), w64 = bnd.w_first(64);
+#pragma unroll
+            for (int k = 1; k < 8; ++k) in |= bnd.reaches<LOW>(s1[k], w1 + M * k, bnd.rs + k, 1, F) ? 1u << k : 0u;
+            if (nch > 8) {
+#pragma unroll
+                for (int k = 1; k < 8; ++k) m8 |= bnd.reaches<LOW>(s8[8 * k], w8 + M * 8 * k, bnd.rs + 8 * k, 8, F) ? 1u << k : 0u;
+            }
+            if (nch > 64) {
+#pragma unroll
+                for (int k = 1; k < 8; ++k) m64 |= bnd.reaches<LOW>(s64[64 * k], w64 + M * 64 * k, bnd.rs + 64 * k, 64, F) ? 1u << k : 0u;
+            }
+            in &= nch < 8 ? (1u << nch) - 1 : ~0u;
+            m8 &= nch < 64 ? (1u << ((nch + 7) >> 3)) - 1 : ~0u;
+            m64 &= nch < 512 ? (1u << ((nch + 63) >> 6)) - 1 : ~0u;
+            u8 = __reduce_or_sync(0xffffffffu, m8);
+            u64 = __reduce_or_sync(0xffffffffu, m64);
+            c512 = c64 = c8 = 0;
+            step = kChunks;
+        } else if (step == kBounds) {
+            // bit k: chunks c + n k .. c + n k + n - 1 (below nch) can reach the floor
+            const int c0 = level == 1 ? c8 : level == 8 ? c64 : c512;
+            const float* q = (level == 1 ? s1 : level == 8 ? s8 : s64) + c0;
+            const float* r = bnd.rs + c0;
+            const int have = min(8, (nch - c0 + level - 1) / level);  // groups below nch
+            const float w0 = (float)(M * c0) + bnd.w_first(level), dw = (float)(M * level);
+            unsigned m = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int o = level * min(k, have - 1);
+                m |= bnd.reaches<LOW>(q[o], fmaf(dw, (float)k, w0), r + o, level, F) ? 1u << k : 0u;
+            }
+            m &= keep & ((1u << have) - 1);
+            if (level == 64) {
+                m64 = m;
+                u64 = __reduce_or_sync(0xffffffffu, m);
+            } else if (level == 8) {
+                m8 = m;
+                u8 = __reduce_or_sync(0xffffffffu, m);
+            } else {
+                in = m;
+                step = kChunks;
+            }
+        }
+        if (step == kChunks) {  // chunks c8 + k of the bits set in `in`
+            if (lmask) in &= lmask[c8 >> 5] >> (c8 & 31);
+            if (__any_sync(0xffffffffu, in)) {
+                found = true;
+                if (pass == 0) {
+                    if (!lmask) {  // (on the sparse ladder the window behind the bound may not take part)
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (((in >> k) & 1u) && M * (c8 + k) + 31 <= max_width)
+                                F = fmaxf(F, bnd.lower(Q[t + c8 + k + 1], c8 + k) - bnd.S);
+                    }
+                } else {
+                    if (in && pend < 0) {
+                        pend = c8 + __ffs((int)in) - 1;
+                        in &= in - 1;
+                    }
+                    if (__any_sync(0xffffffffu, in)) {  // evaluate, then look at the rest again
+                        step = kEval;
+                        level = 1;
+                        keep = in;
+                        continue;
+                    }
+                }
+            }
+        }
+        step = kBounds;
+        if (u8) {
+            const int g = __ffs((int)u8) - 1;
+            u8 &= u8 - 1;
+            c8 = c64 + 8 * g;
+            level = 1;
+            keep = (m8 >> g) & 1u ? ~0u : 0u;
+        } else if (u64) {
+            const int g = __ffs((int)u64) - 1;
+            u64 &= u64 - 1;
+            c64 = c512 + 64 * g;
+            level = 8;
+            keep = (m64 >> g) & 1u ? ~0u : 0u;
+        } else if (c512 + 512 < nch) {
+            c512 += 512;
+            level = 64;
+            keep = ~0u;
+        } else if (pass == 0 && found) {
+            step = kFirst;
+        } else {
+            step = kEval;
+            last = true;
+        }
+    }
+    return evaluated;
+}
+
+// Every width in order (the decimated ladder's level 0: few widths, all in
+// `tab`).  C[i] receives w0 of the first chunk reaching B[i].
+__device__ __forceinline__ void boxcar_prefix(const float* __restrict__ P, const float2* __restrict__ tab, int wpad,
+                                              const float (&base)[M], float (&B)[M], int (&C)[M]) {
     const float* pb = P + M * threadIdx.x;
-    int evaluated = 0;
 #pragma unroll
     for (int i = 0; i < M; ++i) {
         B[i] = -FLT_MAX;
         C[i] = 0;
     }
-    constexpr int kSeg = 128;  // widths per segment inside the wide power-of-two blocks
     for (int w0 = 0; w0 < wpad; w0 += M) {
-        const bool blk = (w0 & (w0 - 1)) == 0;  // first chunk of a power-of-two block
-        if (bnd.active && w0 >= 16 && (blk || (w0 >= 2 * kSeg && (w0 & (kSeg - 1)) == 0))) {
-            int w_end = blk ? 2 * w0 : w0 + kSeg;
-            float bmin = B[0];
-#pragma unroll
-            for (int i = 1; i < M; ++i) bmin = fminf(bmin, B[i]);
-            const float floor_b = fmaxf(bnd.cut, bmin);
-            bool skip = !__any_sync(0xffffffffu,
-                                    thread_segment_bound(P, bnd, w0 + 1, min(w_end, bnd.max_width)) >= floor_b);
-            if (!skip && blk && w0 >= 2 * kSeg) {
-                w_end = w0 + kSeg;
-                skip = !__any_sync(0xffffffffu,
-                                   thread_segment_bound(P, bnd, w0 + 1, min(w_end, bnd.max_width)) >= floor_b);
-            }
-            if (skip) {
-                w0 = w_end - M;  // next block or segment
-                continue;
-            }
-        }
-        if (lmask && !ladder_has(lmask, w0 + 1)) continue;  // chunk not on the width ladder
-        ++evaluated;
-        float win[2 * M];  // win[k] = P[p_thread + w0 + k]
-#pragma unroll
-        for (int k = 0; k < 2 * M; k += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(pb + w0 + k);
-            win[k] = v.x; win[k + 1] = v.y; win[k + 2] = v.z; win[k + 3] = v.w;
-        }
-        float Bc[M];  // best SNR of this chunk, per slot
-        {
-            const float2 rc0 = tab[w0];
-            const float2 rc1 = tab[w0 + 1];
-#pragma unroll
-            for (int i = 0; i < M; ++i)
-                Bc[i] = fmaxf(fmaf(win[i + 1] - base[i], rc0.x, rc0.y),
-                              fmaf(win[i + 2] - base[i], rc1.x, rc1.y));
-        }
-#pragma unroll
-        for (int s = 2; s < M; s += 2) {
-            const float2 rc0 = tab[w0 + s];
-            const float2 rc1 = tab[w0 + s + 1];
-#pragma unroll
-            for (int i = 0; i < M; ++i) {
-                const float v0 = fmaf(win[i + s + 1] - base[i], rc0.x, rc0.y);
-                const float v1 = fmaf(win[i + s + 2] - base[i], rc1.x, rc1.y);
-                Bc[i] = max3f(Bc[i], v0, v1);
-            }
-        }
+        float Bc[M];
+        eval_chunk(pb + w0, reinterpret_cast<const float4*>(tab + w0), 0, base, Bc);
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            if (Bc[i] > B[i]) {  // strict: an equal later chunk keeps the earlier one
+            if (Bc[i] > B[i]) {
                 B[i] = Bc[i];
                 C[i] = w0;
             }
         }
     }
-    return evaluated;
 }
 
 // Exact int64 running sums for slot i, for tiles whose partial sums may
@@ -549,10 +686,13 @@ __device__ __noinline__ float boxcar_exact_slot(const float* __restrict__ ys,
     return best;
 }
 
-// Shared memory after the main loop: the end of the table region is reused
-// for B(t) (kSpsTile floats) followed by the candidate entries (kSpsTile u32).
-__host__ __device__ constexpr int sps_region_bytes(int wpad) {
-    return (wpad * 8 > kSpsTile * 8) ? wpad * 8 : kSpsTile * 8;
+// Shared memory: the series, the table's first widths, the block maxima (in
+// their place, once they are done with, B(t) where it is written out, then the
+// candidate entries: at most every second start is a peak), the next tile's
+// new samples, the bounds' factors, the ladder's mask.
+__host__ __device__ constexpr int sps_lists_words(int wpad) {
+    const int q = 4 * sps_q16(wpad);
+    return q > 2 * kSpsTile ? q : 2 * kSpsTile;
 }
 
 // One CTA's work: tiles [tile_lo, tile_hi) of series `row`, in order.  `sm`
@@ -565,19 +705,40 @@ __host__ __device__ constexpr int sps_region_bytes(int wpad) {
 // summed, continuing from the exact sum at the old end.  Prefix sums are then
 // relative to the first fully staged tile; sliding is allowed while every
 // staged prefix sum lies within +-2^23 (so every window sum, a difference of
-// two, is an exact FP32 integer); otherwise the tile is staged afresh.
+// two, is an exact FP32 integer); otherwise the tile is staged afresh.  The new
+// samples are copied to shared memory (cp.async) while the previous tile's
+// widths are searched.
+//
+// With 16 warps an SM (128 registers: a thread's starts, their B, the window of
+// a chunk) the tile's chain of short phases is what takes the time, so the
+// phases are kept few and their barriers fewer.  4096 channels x 2^20 samples,
+// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 40.5 ms; of that (clock64) the
+// width search 14.6, waiting for a tile's slowest warp 8.0, block maxima 4.4,
+// sums of new samples 2.8, candidates' widths 2.1, fresh tiles 1.5, peaks 1.4,
+// sliding 1.4.  Steps on the way: a warp's union of 128-width segments 92, the
+// chunks of each thread by lower bounds 66, their bounds eight at a time in one
+// loop 57, the new samples by cp.async, 32-bit sums, peaks from registers and
+// widths by half-warps 45, chunk numbers packed 40.5.
+template <bool LOW>
 __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t tile_lo, int64_t tile_hi,
                                              float* sm) {
-    __shared__ long long scratch[3 * NT / 32];
+    constexpr int NW = NT / 32;
+    __shared__ int scratch[3 * NW];
+    __shared__ float s_edge[2 * NW];  // B of each warp's first and last start
+    __shared__ int s_cnt[NW];
     __shared__ unsigned long long s_base;
-    __shared__ long long s_pend;  // exact prefix sum just past the staged series
+    __shared__ int s_pend;  // exact prefix sum just past the staged series (while sliding)
     const int wpad = a.wpad;
     const int ylen = kSpsTile + wpad + M;
     float* ys = sm;
-    float2* tab = reinterpret_cast<float2*>(sm + ((ylen + 3) & ~3));
-    float* Qs = sm + ((ylen + 3) & ~3) + sps_region_bytes(wpad) / 4;
-    const int nq = sps_q_count(wpad);
-    uint32_t* s_ladder = reinterpret_cast<uint32_t*>(Qs + ((nq + 3) & ~3));
+    const int wtab = sps_tab_smem(wpad);
+    float4* tab = reinterpret_cast<float4*>(sm + ylen);
+    float* lists = sm + ylen + 2 * wtab;
+    float* Q = lists;  // block maxima and their sliding maxima, nq each
+    const int nq = sps_q16(wpad);
+    float* nbuf = lists + sps_lists_words(wpad);  // the next tile's new samples
+    float* rs = nbuf + kSpsTile;
+    uint32_t* s_ladder = reinterpret_cast<uint32_t*>(rs + sps_rs(wpad));
     const uint32_t* lmask = a.ladder_g16 > 0 ? s_ladder : nullptr;
     if (lmask) fill_ladder(s_ladder, wpad / M, a.ladder_g16);  // visible after the staging barrier
     const int64_t L = a.length;
@@ -586,12 +747,27 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
     const float m0 = st.m0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float2* gtab = a.table + (int64_t)row * wpad;
-    // B(t) and the candidate list take the last kSpsTile * 8 bytes of the
-    // table region after the width loop: the entries of widths up to
-    // 2 * lists4 stay in shared memory for the candidates' widths
-    const int lists4 = (sps_region_bytes(wpad) - kSpsTile * 8) / 16;
+    // entry of width w (the candidates' widths read single ones)
+    auto entry = [&](int w) {
+        if (w > wtab) return __ldg(gtab + w - 1);
+        const int c = (w - 1) / M, e = (w - 1) % M;
+        return reinterpret_cast<const float2*>(tab + tab_block(c, e >> 1))[e & 1];
+    };
+    WidthBounds bnd;
+    bnd.rs = rs;
+    bnd.f = (float)(st.mu - (double)m0);
+    {   // the table's first widths, staged once for all tiles, and the bounds' factors
+        const float4* g4 = reinterpret_cast<const float4*>(gtab);
+        for (int i = threadIdx.x; i < wtab / 2; i += NT) tab[tab_block(i >> 3, i & 7)] = __ldg(g4 + i);
+        const float inv = (float)st.inv_sigma;
+        for (int c = threadIdx.x; c < sps_rs(wpad); c += NT) rs[c] = inv * (rsqrtf((float)(M * c + 1)) * (1.0f + 1.02e-4f));
+        // 1.02e-4, and 2.1e-6 of the largest drift over sigma sqrt(w) (w f r <= |f| 2 sqrt(W + 64 M) / sigma)
+        bnd.S = 1.02e-4f + 2.1e-6f * inv * sqrtf((float)(wpad + 64 * M));
+    }
+    // B(t) of every start asked for: only the running B prunes
+    const float cut = a.prune && a.threshold > 0.0f ? a.threshold - 1e-3f : -FLT_MAX;
     constexpr int kBatch = 8;
-    constexpr long long kSlideMax = 1ll << 23;
+    constexpr int kSlideMax = 1 << 23;
     bool slide = false;  // ys holds the previous tile's prefix sums, all within +-2^23
 
     for (int64_t tile = tile_lo; tile < tile_hi; ++tile) {
@@ -600,95 +776,60 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
         const int va = t0 == 0 ? 1 : 0;
         const int vb = (int)min((int64_t)ylen - 1, L - t0);
         const int nkeep = ylen - kSpsOwned;  // staged samples shared with the previous tile
-
-        // The width table, then the series: after a slide only the new samples
-        // (minus m0, sentinel outside [0, L)), else all of them.  The previous
-        // tile's B(t) and candidate list overwrote only the table's last
-        // kSpsTile * 8 bytes (from float4 lists4 on), so after a slide only
-        // those are staged again.
-        {
-            const float4* g4 = reinterpret_cast<const float4*>(gtab);  // wpad is even
-            float4* t4 = reinterpret_cast<float4*>(tab);
-            const int n4 = wpad / 2;
-            for (int i0b = (slide ? lists4 : 0) + threadIdx.x; i0b < n4; i0b += NT * kBatch) {
-                float4 v[kBatch];
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) {
-                    const int i = i0b + u * NT;
-                    if (i < n4) v[u] = __ldg(g4 + i);
-                }
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u)
-                    if (i0b + u * NT < n4) t4[i0b + u * NT] = v[u];
-            }
-        }
         bool fast = false;
         if (slide) {
-            // slide P down by kSpsOwned: rounds of NT x 16 values, all loads of a
+            // slide P down by kSpsOwned: rounds of NT x 16 pairs, all loads of a
             // round before its stores (a round's source and destination overlap;
             // a later round's source never meets an earlier round's destination)
             constexpr int kR = 16;
-            for (int r0 = 0; r0 < nkeep; r0 += NT * kR) {
-                float v[kR];
+            static_assert(kSpsOwned % 2 == 0, "pairs");
+            for (int r0 = 0; r0 < nkeep / 2; r0 += NT * kR) {
+                float2 v[kR];
 #pragma unroll
                 for (int u = 0; u < kR; ++u) {
                     const int i = r0 + u * NT + threadIdx.x;
-                    v[u] = i < nkeep ? ys[i + kSpsOwned] : 0.0f;
+                    if (i < nkeep / 2) v[u] = *reinterpret_cast<const float2*>(ys + 2 * i + kSpsOwned);
                 }
-                __syncthreads();
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncthreads();  // (after the last round: the new samples have arrived too)
 #pragma unroll
                 for (int u = 0; u < kR; ++u) {
                     const int i = r0 + u * NT + threadIdx.x;
-                    if (i < nkeep) ys[i] = v[u];
+                    if (i < nkeep / 2) *reinterpret_cast<float2*>(ys + 2 * i) = v[u];
                 }
             }
-            __syncthreads();  // the last round's loads are done before the new samples land
-            for (int i0b = nkeep + threadIdx.x; i0b < ylen; i0b += NT * kBatch) {
-                float v[kBatch];
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) {
-                    const int i = i0b + u * NT;
-                    const int64_t t = t0 - 1 + i;
-                    v[u] = (i < ylen && t >= 0 && t < L) ? __ldg(y + t) - m0 : kSentinel;
-                }
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u)
-                    if (i0b + u * NT < ylen) ys[i0b + u * NT] = v[u];
-            }
-            __syncthreads();
             // exact sums of the new samples, continuing from the old end
             const int segn = ((kSpsOwned + NT - 1) / NT) | 1;  // odd: distinct banks
-            const int j0 = min(ylen, nkeep + threadIdx.x * segn), j1 = min(ylen, j0 + segn);
-            long long run = 0, mn = 0, mx = 0;
-            for (int i = j0; i < j1; ++i) {
-                const float v = ys[i];
-                if (v > kSentinelTest) {
-                    run += (long long)(int)v;
+            const int j0 = min(kSpsOwned, (int)threadIdx.x * segn), j1 = min(kSpsOwned, j0 + segn);
+            const int jv = vb + 1 - nkeep;  // new samples below the series' end
+            int run = 0, mn = 0, mx = 0;
+            for (int j = j0; j < j1; ++j) {
+                const float v = nbuf[j] - m0;
+                if (j < jv && v > kSentinelTest) {
+                    run += (int)v;
                     mn = min(mn, run);
                     mx = max(mx, run);
                 }
             }
-            long long tot = 0, ex = 0, gmn = 0, gmx = 0;
-            const long long pend = s_pend;
+            int tot, ex, gmn, gmx;
+            const int pend = s_pend;
             block_scan_minmax<NT>(run, mn, mx, scratch, ex, tot, gmn, gmx);
-            const long long before = pend + ex;
-            gmn += pend;
-            gmx += pend;
-            fast = gmn >= -kSlideMax && gmx <= kSlideMax;
+            fast = (long long)gmn + pend >= -kSlideMax && (long long)gmx + pend <= kSlideMax;
             if (fast) {
-                float runf = (float)before;
-                for (int i = j0; i < j1; ++i) {
-                    const float v = ys[i];
-                    ys[i] = i > vb + 1 ? -kBig : runf;
-                    if (v > kSentinelTest) runf += v;
+                float runf = (float)(pend + ex);
+                for (int j = j0; j < j1; ++j) {
+                    const float v = nbuf[j] - m0;
+                    ys[nkeep + j] = j > jv ? -kBig : runf;
+                    if (j < jv && v > kSentinelTest) runf += v;
                 }
+                // (the reads of s_pend above precede the scan's barrier)
                 if (threadIdx.x == 0) s_pend = pend + tot;
             }
-            // (the reads of s_pend above precede this barrier, its write follows it)
             __syncthreads();
         }
         if (!fast) {
-            // stage every sample afresh; loads in batches so that latencies overlap
+            // stage every sample afresh (minus m0, sentinel outside [0, L)); loads in
+            // batches so that latencies overlap
             for (int i0b = threadIdx.x; i0b < ylen; i0b += NT * kBatch) {
                 float v[kBatch];
 #pragma unroll
@@ -706,23 +847,22 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
             // Largest |partial sum| of the tile = range of the prefix sums of ys over
             // its valid samples: FP32 sums are exact when it is <= 2^24.
             const int seg = ((ylen + NT - 1) / NT) | 1;  // odd: the threads' segments fall on distinct banks
-            const int i0 = min(ylen, threadIdx.x * seg), i1 = min(ylen, i0 + seg);
-            long long run = 0, mn = 0, mx = 0;
+            const int i0 = min(ylen, (int)threadIdx.x * seg), i1 = min(ylen, i0 + seg);
+            int run = 0, mn = 0, mx = 0;
             for (int i = i0; i < i1; ++i) {
                 const float v = ys[i];
                 if (v > kSentinelTest) {
-                    run += (long long)(int)v;
+                    run += (int)v;
                     mn = min(mn, run);
                     mx = max(mx, run);
                 }
             }
-            long long tot = 0, before = 0, gmn = 0, gmx = 0;
+            int tot, before, gmn, gmx;
             block_scan_minmax<NT>(run, mn, mx, scratch, before, tot, gmn, gmx);
-            fast = (gmx - gmn) <= (1ll << 24);
+            fast = (long long)gmx - gmn <= (1 << 24);
             slide = gmn >= -kSlideMax && gmx <= kSlideMax;  // the next tile may slide
             if (fast) {
                 // ys -> prefix sums P, in place (exact FP32 integers)
-                __syncthreads();
                 float runf = (float)before;
                 for (int i = i0; i < i1; ++i) {
                     const float v = ys[i];
@@ -734,97 +874,145 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
             }
         }
         slide = slide && fast && (tile + 1 < tile_hi);
+        if (slide) {  // the next tile's new samples, copied while this one is searched
+            const int64_t tn = t0 + kSpsOwned - 1 + nkeep;
+#pragma unroll 4
+            for (int j = threadIdx.x; j < kSpsOwned; j += NT) {
+                const int64_t t = tn + j;
+                const unsigned dst = (unsigned)__cvta_generic_to_shared(nbuf + j);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(y + min(t, L - 1)), "r"(t < L ? 4 : 0)
+                             : "memory");
+            }
+        }
 
         float B[M];
-        int C[M];  // per slot: w0 of the first width chunk reaching B (0 on the exact path)
+        uint32_t C[M / 2];  // the first width chunk reaching B, 16 bits a slot (0 on the exact path)
         if (fast) {
             const float* P = ys;
-            if (a.prune) {  // block maxima Q: a warp reduces 4 blocks at once
-                for (int j0 = 4 * warp; j0 < nq; j0 += 4 * (NT / 32)) {
-                    float m[4];
+            float base[M];
+            // block maxima, a thread per block of 16 (those past the staged series
+            // hold no end), and the sliding maxima over 2, 9 and 65 of them
+            {
+                float m = -FLT_MAX;
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        m[b] = -FLT_MAX;
+                for (int k = 0; k < M; k += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(P + M * threadIdx.x + k);
+                    base[k] = v.x; base[k + 1] = v.y; base[k + 2] = v.z; base[k + 3] = v.w;
+                    m = max3f(max3f(m, v.x, v.y), v.z, v.w);
+                }
+                Q[threadIdx.x] = m;
+                for (int j = threadIdx.x + NT; j < nq; j += NT) {
+                    m = -kBig;
+                    if (M * j < ylen) {  // ylen is a multiple of M
 #pragma unroll
-                        for (int u = 0; u < kQSpan / 32; ++u) {
-                            const int i = (j0 + b) * kQSpan + u * 32 + lane;
-                            if (i < ylen) m[b] = fmaxf(m[b], P[i]);
+                        for (int k = 0; k < M; k += 4) {
+                            const float4 v = *reinterpret_cast<const float4*>(P + M * j + k);
+                            m = max3f(max3f(m, v.x, v.y), v.z, v.w);
                         }
                     }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) m[b] = fmaxf(m[b], __shfl_xor_sync(0xffffffffu, m[b], o));
-                    if (lane < 4 && j0 + lane < nq) Qs[j0 + lane] = lane == 0 ? m[0] : lane == 1 ? m[1] : lane == 2 ? m[2] : m[3];
+                    Q[j] = m;
                 }
-                __syncthreads();
             }
-            float base[M];
-            float pmin = FLT_MAX;
+            float pmin = FLT_MAX, pmax = -FLT_MAX;
 #pragma unroll
             for (int i = 0; i < M; ++i) {
                 const int p = M * threadIdx.x + i;
                 const bool valid = p >= va && p <= vb;
-                base[i] = valid ? P[p] : kBig;
-                if (valid) pmin = fminf(pmin, base[i]);
+                if (valid) {
+                    pmin = fminf(pmin, base[i]);
+                    pmax = fmaxf(pmax, base[i]);
+                } else {
+                    base[i] = kBig;
+                }
             }
-            ThreadBound bnd;
-            bnd.Q = Qs;
             bnd.pmin = pmin;
-            bnd.f = (float)(st.mu - (double)m0);
-            bnd.inv_sigma = (float)st.inv_sigma;
-            bnd.cut = a.threshold > 0.0f ? a.threshold - 1e-3f : -FLT_MAX;
-            bnd.max_width = a.max_width;
-            bnd.ylen = ylen;
-            bnd.nq = nq;
-            bnd.ps = M * threadIdx.x;
-            bnd.active = a.prune != 0;
-            const int chunks = boxcar_prefix(P, tab, wpad, base, bnd, lmask, B, C);
-            if (a.evaluated && (threadIdx.x & 31) == 0)
-                atomicAdd(a.evaluated, (unsigned long long)chunks * 32ull * M * M);
-            if (slide) {
-                // A warp that finishes its widths early waits for the tile's
-                // slowest one: meanwhile it asks L2 for the next tile's new
-                // samples (every warp covers them all; later requests hit L2).
-                const int64_t t_new = t0 + kSpsOwned - 1 + nkeep;  // first new sample of the next tile
-                const int64_t t_end = min(L, t_new + kSpsOwned);
-                for (int64_t t = t_new + 32 * lane; t < t_end; t += 32 * 32)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(y + t));
+            bnd.pmax = pmax;
+            __syncthreads();
+            const bool bounds = wpad > M && !(LOW && wpad <= kEvery * M);  // boxcar_search looks at them
+            if (bounds) {
+                for (int j = threadIdx.x; j < nq; j += NT) {
+                    const float a1 = fmaxf(Q[j], j + 1 < nq ? Q[j + 1] : -kBig);
+                    float m = a1;
+#pragma unroll
+                    for (int k = 2; k < 9; ++k)
+                        if (j + k < nq) m = fmaxf(m, Q[j + k]);
+                    Q[nq + j] = a1;
+                    Q[2 * nq + j] = m;
+                }
+                __syncthreads();
+            }
+            if (wpad > 64 * M) {
+                for (int j = threadIdx.x; j < nq; j += NT) {
+                    float m = Q[2 * nq + j];
+#pragma unroll
+                    for (int k = 8; k < 64; k += 8)
+                        if (j + k < nq) m = fmaxf(m, Q[2 * nq + j + k]);
+                    Q[3 * nq + j] = m;
+                }
+                __syncthreads();
+            }
+            int chunks = boxcar_search<LOW>(P, tab, gtab, wpad / M, a.max_width, base, bnd, Q, nq, cut, lmask, B, C);
+            if (a.evaluated) {
+                chunks = __reduce_add_sync(0xffffffffu, chunks);
+                if (lane == 0) atomicAdd(a.evaluated, (unsigned long long)chunks * M * M);
             }
         } else {
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                B[i] = boxcar_exact_slot(ys, tab, wpad, i, lmask);
-                C[i] = 0;
+                B[i] = boxcar_exact_slot(ys, gtab, wpad, i, lmask);
+                C[i / 2] = 0;
             }
             if (a.evaluated && threadIdx.x == 0)
                 atomicAdd(a.evaluated, (unsigned long long)wpad * NT * M);
         }
-
-        __syncthreads();  // everyone done with the table
-        float* Bs = reinterpret_cast<float*>(tab) + 4 * lists4;  // B(t) of every slot
-        // candidate entries: slot p (bits 0-15) | first chunk w0 / M (bits 16-31)
-        uint32_t* plist = reinterpret_cast<uint32_t*>(Bs + kSpsTile);
-#pragma unroll
-        for (int i = 0; i < M; ++i) Bs[M * threadIdx.x + i] = B[i];
-        __syncthreads();
+        if (lane == 0) s_edge[2 * warp] = B[0];
+        if (lane == 31) s_edge[2 * warp + 1] = B[M - 1];
+        __syncthreads();  // edges visible; everyone done with the block maxima
 
         const bool zero_sigma = st.zero_sigma != 0;
+        if (a.snr_out) {  // through shared memory, so that consecutive threads write consecutive starts
+            float* Bs = lists;
+#pragma unroll
+            for (int k = 0; k < M; k += 4)
+                *reinterpret_cast<float4*>(Bs + M * threadIdx.x + k) = make_float4(B[k], B[k + 1], B[k + 2], B[k + 3]);
+            __syncthreads();
+            float* dst = a.snr_out + (int64_t)row * a.pitch + t0 - 1;
+            const int pe = (int)min((int64_t)kSpsTile - 2, L - t0);  // owned starts below the series' end
+            for (int p = 1 + threadIdx.x; p <= pe; p += NT) dst[p] = zero_sigma ? 0.0f : Bs[p];
+        }
+        // peaks: a start's neighbours are the thread's own, the next thread's or
+        // the next warp's
+        float left = __shfl_up_sync(0xffffffffu, B[M - 1], 1), right = __shfl_down_sync(0xffffffffu, B[0], 1);
+        if (lane == 0 && warp > 0) left = s_edge[2 * warp - 1];
+        if (lane == 31 && warp + 1 < NW) right = s_edge[2 * warp + 2];
         unsigned cmask = 0;
 #pragma unroll
         for (int i = 0; i < M; ++i) {
             const int p = M * threadIdx.x + i;
-            const int64_t t = t0 - 1 + p;
-            if (p >= 1 && p <= kSpsTile - 2 && t < L) {
-                const float v = Bs[p];
-                if (a.snr_out) a.snr_out[(int64_t)row * a.pitch + t] = zero_sigma ? 0.0f : v;
-                if (!zero_sigma && v >= a.threshold && v > Bs[p - 1] && v >= Bs[p + 1]) cmask |= 1u << i;
-            }
+            const float v = B[i], l = i > 0 ? B[i - 1] : left, r = i + 1 < M ? B[i + 1] : right;
+            if (p >= 1 && p <= kSpsTile - 2 && p <= vb && v >= a.threshold && v > l && v >= r) cmask |= 1u << i;
         }
+        if (zero_sigma) cmask = 0;
         // One atomic per tile: the tile's candidates form one contiguous run in t order.
-        long long total = 0;
-        const long long my_off = block_exclusive_scan_total<NT>(__popc(cmask), scratch, total);
+        const int mine = __popc(cmask);
+        int inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) s_cnt[warp] = inc;
+        __syncthreads();  // (and Bs has been read)
+        int total = 0, off = inc - mine;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            if (w < warp) off += s_cnt[w];
+            total += s_cnt[w];
+        }
         if (total > 0) {
+            // candidate entries: slot p (bits 0-15) | first chunk (bits 16-31), and B
+            uint32_t* plist = reinterpret_cast<uint32_t*>(lists);
+            float* blist = lists + kSpsTile;
             const uint32_t dm_index = (uint32_t)(a.dm_offset + row);
             if (threadIdx.x == 0) {
                 s_base = atomicAdd(a.count, (unsigned long long)total);
@@ -832,45 +1020,57 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
                 if (ci < (unsigned long long)a.chunk_cap)
                     a.chunks[ci] = CandChunk{s_base, (uint32_t)total, dm_index, (uint32_t)t0, (uint32_t)a.beam};
             }
-            {
-                int j = (int)my_off;
 #pragma unroll
-                for (int i = 0; i < M; ++i)
-                    if ((cmask >> i) & 1u)
-                        plist[j++] = (uint32_t)(M * threadIdx.x + i) | ((uint32_t)(C[i] / M) << 16);
-            }
+            for (int i = 0; i < M; ++i)
+                if ((cmask >> i) & 1u) {
+                    plist[off] = (uint32_t)(M * threadIdx.x + i) | ((i & 1 ? C[i / 2] >> 16 : C[i / 2]) << 16);
+                    blist[off] = B[i];
+                    ++off;
+                }
             __syncthreads();
 
-            // Width of each candidate: the smallest w reaching B(t), recomputed from
-            // the staged series with the main loop's arithmetic (exact running sums,
-            // fmaf of the correctly rounded sum), one warp per candidate, widths
-            // interleaved over lanes with a warp prefix sum.
-            for (int q = warp; q < (int)total; q += NT / 32) {
-                const int p = (int)(plist[q] & 0xffffu);
-                const int cw0 = (int)(plist[q] >> 16) * M;
-                const int64_t t = t0 - 1 + p;
-                const int wmax = (int)min((int64_t)a.max_width, L - t);
-                const float* yq = ys + p;  // exact path: yq[w-1] = y[t+w-1] - m0
-                const float target = Bs[p];
-                float best = -FLT_MAX;
-                int bw = 0x7fffffff;
-                if (fast) {
-                    // prefix form: S_w = P[p+w] - P[p], exact
-                    const float* P = ys;
-                    const float b0 = P[p];
-                    for (int w0 = cw0; w0 < wmax; w0 += 32) {
-                        const int w = w0 + lane + 1;
-                        if (w <= wmax && (!lmask || ladder_has(lmask, w))) {
-                            const float2 rc = w <= 2 * lists4 ? tab[w - 1] : __ldg(gtab + w - 1);
-                            const float snr = fmaf(P[p + w] - b0, rc.x, rc.y);
-                            if (snr > best) { best = snr; bw = w; }
+            auto store = [&](int q, int p, int w) {
+                const unsigned long long idx = s_base + (unsigned long long)q;
+                if (idx < (unsigned long long)a.capacity) {
+                    aa_candidate c;
+                    c.dm_index = dm_index;
+                    c.t = (uint32_t)(t0 - 1 + p);
+                    c.width = (uint16_t)w;
+                    c.range = (uint8_t)a.range;
+                    c.reserved = (uint8_t)a.beam;
+                    c.snr = blist[q];
+                    a.cands[idx] = c;
+                }
+            };
+            if (fast) {
+                // Width of each candidate: the smallest w reaching B(t) lies in its
+                // chunk: half a warp per candidate evaluates the chunk's 16 widths with
+                // the search's arithmetic
+                const int half = lane >> 4, e = lane & 15;
+                for (int q0 = 2 * warp; q0 < total; q0 += 2 * NW) {
+                    const int q = q0 + half;
+                    bool hit = false;
+                    int p = 0, w = 0;
+                    if (q < total) {
+                        p = (int)(plist[q] & 0xffffu);
+                        w = (int)(plist[q] >> 16) * M + e + 1;
+                        if (w <= a.max_width) {
+                            const float2 rc = entry(w);
+                            hit = fmaf(ys[p + w] - ys[p], rc.x, rc.y) == blist[q];
                         }
-                        // widths are visited in increasing order: stop at the chunk
-                        // where B(t) is first reached
-                        if (__any_sync(0xffffffffu, best == target)) break;
                     }
-                } else {
-                    long long base = 0;
+                    const unsigned hits = __ballot_sync(0xffffffffu, hit) & (0xffffu << (16 * half));
+                    if (hit && lane == __ffs((int)hits) - 1) store(q, p, w);
+                }
+            } else {
+                // exact running sums, widths interleaved over a warp's lanes
+                for (int q = warp; q < total; q += NW) {
+                    const int p = (int)(plist[q] & 0xffffu);
+                    const int wmax = (int)min((int64_t)a.max_width, L - (t0 - 1 + p));
+                    const float* yq = ys + p;  // yq[w-1] = y[t+w-1] - m0
+                    const float target = blist[q];
+                    int bw = 0x7fffffff;
+                    long long sum = 0;
                     for (int w0 = 0; w0 < wmax; w0 += 32) {
                         const int w = w0 + lane + 1;
                         long long v = (w <= wmax) ? (long long)yq[w - 1] : 0;
@@ -879,47 +1079,34 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
                             const long long u = __shfl_up_sync(0xffffffffu, v, o);
                             if (lane >= o) v += u;
                         }
-                        const long long S = base + v;
-                        base += __shfl_sync(0xffffffffu, v, 31);
+                        const long long S = sum + v;
+                        sum += __shfl_sync(0xffffffffu, v, 31);
                         if (w <= wmax && (!lmask || ladder_has(lmask, w))) {
-                            const float2 rc = w <= 2 * lists4 ? tab[w - 1] : __ldg(gtab + w - 1);
-                            const float snr = fmaf(__ll2float_rn(S), rc.x, rc.y);
-                            if (snr > best) { best = snr; bw = w; }
+                            const float2 rc = entry(w);
+                            if (fmaf(__ll2float_rn(S), rc.x, rc.y) == target) bw = w;
                         }
-                        if (__any_sync(0xffffffffu, best == target)) break;
+                        bw = __reduce_min_sync(0xffffffffu, bw);
+                        if (bw != 0x7fffffff) break;  // widths are visited in increasing order
                     }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-                    const int ow = __shfl_xor_sync(0xffffffffu, bw, o);
-                    if (ob > best || (ob == best && ow < bw)) { best = ob; bw = ow; }
-                }
-                const unsigned long long idx = s_base + (unsigned long long)q;
-                if (lane == 0 && idx < (unsigned long long)a.capacity) {
-                    aa_candidate c;
-                    c.dm_index = dm_index;
-                    c.t = (uint32_t)t;
-                    c.width = (uint16_t)bw;
-                    c.range = (uint8_t)a.range;
-                    c.reserved = (uint8_t)a.beam;
-                    c.snr = best;
-                    a.cands[idx] = c;
+                    if (lane == 0) store(q, p, bw);
                 }
             }
         }  // total > 0
-        __syncthreads();  // the next tile overwrites the series, table and lists
+        __syncthreads();  // the next tile overwrites the series and the lists
     }  // tiles
 }
 
 // CTA = seg_tiles consecutive tiles of one series (the last segment of a
 // series may be shorter).
+// LOW: B below zero counts (B(t) asked for, or a threshold not above zero).
+__host__ __device__ inline bool sps_low(const SpsArgs& a) { return !(a.prune && a.threshold > 0.0f); }
+template <bool LOW>
 __global__ void __launch_bounds__(NT, 2) sps_boxcar_kernel(SpsArgs a, int ntiles, int seg_tiles) {
     extern __shared__ __align__(16) float sm[];
     const int nseg = (ntiles + seg_tiles - 1) / seg_tiles;
     const int row = (int)(blockIdx.x / (unsigned)nseg);
     const int64_t lo = (int64_t)(blockIdx.x - (unsigned)row * (unsigned)nseg) * seg_tiles;
-    boxcar_block(a, row, lo, min((int64_t)ntiles, lo + seg_tiles), sm);
+    boxcar_block<LOW>(a, row, lo, min((int64_t)ntiles, lo + seg_tiles), sm);
 }
 
 constexpr int kMaxDecLevels = 16;
@@ -1064,9 +1251,7 @@ __device__ __forceinline__ void boxcar_dec_block(const SpsArgs& a, int ntiles, i
             const int q = H + M * threadIdx.x + i;
             base[i] = (q >= va && q <= vb) ? P[q] : kBig;
         }
-        ThreadBound bnd{};
-        bnd.active = false;
-        boxcar_prefix(P + H, tab, d.wpad0, base, bnd, nullptr, B, C);
+        boxcar_prefix(P + H, tab, d.wpad0, base, B, C);
         // the levels' strided prefix sums: P_k[i] = P at t = (jk0 + i) 2^k
         for (int k = 1; k <= K; ++k) {
             const int64_t jk0 = (t0 - 1) >> k;
@@ -1330,7 +1515,7 @@ __global__ void __launch_bounds__(NT, 2) sps_boxcar_batch_kernel(
         } else {
             const int row = (int)(bid / ntiles[k]);
             const int64_t tile = bid - (int64_t)row * ntiles[k];
-            boxcar_block(descs[k], row, tile, tile + 1, sm);
+            boxcar_block<true>(descs[k], row, tile, tile + 1, sm);
         }
     }
 }
@@ -1379,14 +1564,20 @@ cudaError_t launch_rsqrt_table(double* t, int wpad, cudaStream_t s) {
 
 size_t sps_boxcar_smem(int wpad) {
     const int ylen = kSpsTile + wpad + M;
-    return (size_t)((ylen + 3) & ~3) * 4 + (size_t)sps_region_bytes(wpad) +
-           (size_t)((sps_q_count(wpad) + 3) & ~3) * 4 + (size_t)ladder_words(wpad) * 4;
+    return ((size_t)ylen + 2 * sps_tab_smem(wpad) + sps_lists_words(wpad) + kSpsTile + sps_rs(wpad) + ladder_words(wpad)) * 4;
 }
 
 int g_boxcar_seg_tiles = 0;
 
 size_t sps_boxcar_smem_for(int32_t max_width, int32_t wpad, int32_t dec_w0) {
-    return dec_w0 > 0 ? dec_layout(max_width, dec_w0).bytes : sps_boxcar_smem(wpad);
+    if (dec_w0 > 0) return dec_layout(max_width, dec_w0).bytes;
+    // The exhaustive search takes the widths whose series, whole width table
+    // (or B(t) and the candidate entries in its place) and 128-sample block
+    // maxima fit a CTA; the kernel itself holds less.
+    const size_t ylen = (size_t)kSpsTile + wpad + M;
+    const size_t full = ylen * 4 + std::max((size_t)wpad * 8, (size_t)kSpsTile * 8) + ((ylen + 127) / 128 + 3) / 4 * 16 +
+                        (size_t)ladder_words(wpad) * 4;
+    return full > kMaxBoxcarSmem ? full : sps_boxcar_smem(wpad);
 }
 
 cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s) {
@@ -1412,9 +1603,10 @@ cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s) {
                         ? (int)std::min<int64_t>(g_boxcar_seg_tiles, ntiles)
                         : (int)std::max<int64_t>(1, std::min<int64_t>({16, ntiles, nblocks / (sms * 2 * 16)}));
     const int64_t ncta = (int64_t)a.nrows * ((ntiles + seg - 1) / seg);
-    cudaError_t e = cudaFuncSetAttribute(sps_boxcar_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = sps_low(a) ? sps_boxcar_kernel<true> : sps_boxcar_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    sps_boxcar_kernel<<<(unsigned)ncta, NT, smem, s>>>(a, (int)ntiles, seg);
+    kern<<<(unsigned)ncta, NT, smem, s>>>(a, (int)ntiles, seg);
     return cudaGetLastError();
 }
 
