@@ -310,9 +310,10 @@ void build_bands(RangePlan& r, int C) {
     for (int k = 8; k >= 2; k /= 2) {
         BandPlan bp;
         if (!build(r, C, k, bp)) continue;
+        // rows that many trials share: smaller bands would only add sums
+        const bool shared = (double)bp.rows.size() < 64.0 * bp.nbands * (double)bp.segs.size();
         if (!best.ok || bp.cost < best.cost) best = std::move(bp);
-        // few rows per block: smaller bands only add sums
-        if ((double)best.rows.size() < 40.0 * best.nbands * (double)best.segs.size()) break;
+        if (shared) break;
     }
     if (best.ok && best.cost < 0.6 * direct) r.bands = std::move(best);
 }

@@ -34,12 +34,16 @@ static constexpr double kDM = 4.148808e3;
 // decimated by dec: round half away from zero of ((kDM*dm)*delta_c)/(tsamp*dec)
 // with delta_c = f_c^-2 - f_top^-2, every step an IEEE double rounded in the
 // order written (this file is compiled without FP contraction).
-static int32_t delay_samples(double fch1, double foff, double f_top, int32_t c, double tsamp,
-                             double dm, int32_t dec) {
+static double channel_delta(double fch1, double foff, double f_top, int32_t c) {
     double fc = fch1 + (double)c * foff;
-    double delta = 1.0 / (fc * fc) - 1.0 / (f_top * f_top);
-    double v = kDM * dm * delta / (tsamp * (double)dec);
-    return (int32_t)std::llround(v);
+    return 1.0 / (fc * fc) - 1.0 / (f_top * f_top);
+}
+// Round half away from zero.  For 0 <= v < 2^31 the fraction v - trunc(v) is
+// exact, so this is llround, without its call.
+static inline int32_t round_samples(double v) {
+    if (!(v >= 0.0 && v < 2147483647.0)) return (int32_t)std::llround(v);
+    const int32_t i = (int32_t)v;
+    return i + (v - (double)i >= 0.5 ? 1 : 0);
 }
 
 // Delay of channel c relative to channel cref at dispersion measure dm, in
@@ -145,6 +149,10 @@ static void build_groups(RangePlan& r, int C) {
     double direct = 0, grouped = 0;
     std::vector<GroupDesc> local;
     std::vector<std::vector<uint16_t>> members;
+    // pattern -> index in `local` (open addressing, cleared by stamping)
+    constexpr size_t kSlotsLog = 13;
+    std::vector<uint32_t> stamp((size_t)1 << kSlotsLog, 0), slot((size_t)1 << kSlotsLog);
+    uint32_t now = 0;
     int run = 0;  // members summed into the trials' 16-bit lanes since the last flush
     for (int b = 0; b < nblk; ++b) {
         const int d0 = b * B, nb = std::min(B, ndm - d0);
@@ -152,6 +160,7 @@ static void build_groups(RangePlan& r, int C) {
             const int c0 = k * gcc, nch = std::min(gcc, C - c0);
             local.clear();
             members.clear();
+            ++now;
             for (int cl = 0; cl < nch; ++cl) {
                 const int c = c0 + cl;
                 GroupDesc g{};
@@ -161,13 +170,20 @@ static void build_groups(RangePlan& r, int C) {
                     g.delta[d] = (uint16_t)(r.shifts[(size_t)dd * C + c] - s0);
                 }
                 g.span = g.delta[B - 1];
-                size_t gi = 0;
-                while (gi < local.size() && std::memcmp(local[gi].delta, g.delta, sizeof g.delta) != 0) ++gi;
-                if (gi == local.size()) {
+                uint64_t key[sizeof g.delta / 8], hash = 0;
+                static_assert(sizeof g.delta % 8 == 0, "pattern words");
+                std::memcpy(key, g.delta, sizeof g.delta);
+                for (uint64_t k2 : key) hash = (hash ^ k2) * 0x9e3779b97f4a7c15ull;
+                size_t h = (size_t)(hash >> (64 - kSlotsLog));
+                while (stamp[h] == now && std::memcmp(local[slot[h]].delta, g.delta, sizeof g.delta) != 0)
+                    h = (h + 1) & (((size_t)1 << kSlotsLog) - 1);
+                if (stamp[h] != now) {
+                    stamp[h] = now;
+                    slot[h] = (uint32_t)local.size();
                     local.push_back(g);
                     members.emplace_back();
                 }
-                members[gi].push_back((uint16_t)cl);
+                members[slot[h]].push_back((uint16_t)cl);
             }
             // Phase 1 of the kernel gives the unit(s) of the group at batch
             // position j to slot j % kSlots (a warp or a warp pair), and a unit
@@ -555,6 +571,8 @@ aa_status aa_plan_create(const aa_plan_desc* d, aa_plan** out) {
         p->tsamp = d->tsamp_s;
         p->f_top = f_last > d->fch1_mhz ? f_last : d->fch1_mhz;
         int32_t off = 0;
+        std::vector<double> delta((size_t)p->nchans);
+        for (int c = 0; c < p->nchans; ++c) delta[(size_t)c] = channel_delta(p->fch1, p->foff, p->f_top, c);
         for (int r = 0; r < d->nranges; ++r) {
             RangePlan rp;
             rp.desc = d->ranges[r];
@@ -562,12 +580,15 @@ aa_status aa_plan_create(const aa_plan_desc* d, aa_plan** out) {
             off += rp.desc.ndm;
             rp.shifts.resize((size_t)rp.desc.ndm * p->nchans);
             int32_t ms = 0;
+            const double unit = p->tsamp * (double)rp.desc.dec;
             for (int i = 0; i < rp.desc.ndm; ++i) {
                 double dm = rp.desc.dm_lo + (double)i * rp.desc.dm_step;
                 p->dm_max = std::max(p->dm_max, dm);
+                const double kdm = kDM * dm;
+                int32_t* row = &rp.shifts[(size_t)i * p->nchans];
                 for (int c = 0; c < p->nchans; ++c) {
-                    int32_t s = delay_samples(p->fch1, p->foff, p->f_top, c, p->tsamp, dm, rp.desc.dec);
-                    rp.shifts[(size_t)i * p->nchans + c] = s;
+                    const int32_t s = round_samples(kdm * delta[(size_t)c] / unit);
+                    row[c] = s;
                     ms = std::max(ms, s);
                 }
             }
