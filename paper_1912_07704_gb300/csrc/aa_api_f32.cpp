@@ -47,7 +47,7 @@ F32FwdArgs fwd_args(const aa_plan* p, const Layout& L, size_t r, const float* x,
     a.d_begin = 0;
     a.d_end = g.desc.ndm;
     a.length = L.length[r];
-    a.rowlen = f32_fwd_rowlen(g.f32_span);
+    a.span = g.f32_span;
     a.pitch = L.pitch[r];
     return a;
 }
@@ -63,7 +63,7 @@ F32AdjArgs adj_args(const aa_plan* p, const Layout& L, size_t r, const float* x,
     a.w = w;
     a.shifts = g.d_shifts;
     a.length = L.length[r];
-    a.rowlen = f32_adj_rowlen(g.f32_cspan);
+    a.span = g.f32_cspan;
     a.gx = gx;
     a.gw = gw;
     a.gw_part = reinterpret_cast<float*>(ws + L.f32_part_offset);

@@ -438,7 +438,7 @@ struct F32FwdArgs {
     const int32_t* shifts;
     int32_t d_begin, d_end;
     int64_t length;
-    int32_t rowlen;
+    int32_t span;  // delay spread over any 16 consecutive trials
     float* y;
     int64_t pitch;
     const float* tmpl;
@@ -458,14 +458,12 @@ struct F32AdjArgs {
     const float* gy;
     int64_t gpitch;
     int64_t length;
-    int32_t rowlen;
+    int32_t span;  // delay spread over any 16 consecutive channels
     float* gx;
     float* gw_part;
     float* gw;
 };
 constexpr int kF32Chunk = 256;  // DM trials per recomputation chunk of the loss gradient
-int f32_fwd_rowlen(int span);
-int f32_adj_rowlen(int cspan);
 int f32_adj_tiles(int64_t nsamp);
 cudaError_t launch_f32_forward(int mode, const F32FwdArgs& p, cudaStream_t s);
 cudaError_t launch_f32_adjoint(const F32AdjArgs& p, cudaStream_t s);

@@ -153,3 +153,46 @@ def test_full_size_sampled_rows(oracle):
     euler = float((2.0 / n) * ((yv - tv) * yv).sum())
     assert abs(float((gw.double() * w.double()).sum()) - euler) <= 1e-4 * abs(euler)
     assert abs(float(loss) - float(((yv - tv) ** 2).mean())) <= 1e-5 * float(loss)
+
+
+@pytest.mark.parametrize("C,T,ndm,step", [
+    (1, 300, 1, 0.1),        # one row of each
+    (9, 1111, 17, 0.3),      # odd pitch (4-byte copies), a second block of one row, stages of 8 and 1
+    (33, 2052, 40, 1.0),     # pitch a multiple of 4 (16-byte copies), wide windows
+    (64, 20000, 600, 0.05),  # 16 samples a lane and row
+    (40, 9000, 16, 9.0),     # spreads that leave fewer source rows per stage
+])
+def test_gather_shapes_against_64_bits(C, T, ndm, step):
+    """Forward and adjoint against a plain 64-bit evaluation; a sum of n terms
+    in 32 bits is within n * 2^-24 of the sum of their magnitudes."""
+    foff = -200.0 / C
+    plan = Plan(C, 1500.0, foff, 64e-6, [(0.0, step, ndm, 1)])
+    plan.bind()
+    s = torch.from_numpy(plan.shifts(0).astype(np.int64)).cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(C)
+    x = torch.randn((C, T), generator=g, device="cuda")
+    w = torch.rand(C, generator=g, device="cuda") + 0.5
+    lay = plan.layout(T)[0]
+    L = lay.length
+    assert L > 0
+    y = plan.range_views(plan.f32_forward(x, w), T)[0]
+    flat = torch.full((plan.query(T).dd_elems,), float("nan"), device="cuda")  # padding must not be read
+    gy = plan.range_views(flat, T)[0]
+    gy.copy_(torch.randn((ndm, L), generator=g, device="cuda"))
+    gx, gw = plan.f32_adjoint(x, w, flat)
+    xd, wd, gd = x.double(), w.double(), gy.double()
+    want_y, mag_y = torch.empty((ndm, L), dtype=torch.float64, device="cuda"), torch.empty((ndm, L), dtype=torch.float64, device="cuda")
+    A, mag = torch.zeros_like(xd), torch.zeros_like(xd)
+    for d in range(ndm):
+        at = s[d][:, None] + torch.arange(L, device="cuda")[None, :]
+        v = torch.gather(xd, 1, at) * wd[:, None]
+        want_y[d], mag_y[d] = v.sum(0), v.abs().sum(0)
+        A.scatter_add_(1, at, gd[d][None, :].expand(C, L))
+        mag.scatter_add_(1, at, gd[d].abs()[None, :].expand(C, L))
+    eps = 2.0 ** -24
+    assert ((y.double() - want_y).abs() <= (C + 1) * eps * mag_y).all()
+    assert ((gx.double() - A * wd[:, None]).abs() <= (ndm + 2) * eps * mag * wd[:, None]).all()
+    want_w = (xd * A).sum(1)
+    assert ((gw.double() - want_w).abs() <= (ndm + T) * eps * (xd.abs() * mag).sum(1)).all()
+    plan.close()
