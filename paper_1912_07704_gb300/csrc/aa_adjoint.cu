@@ -260,7 +260,7 @@ __global__ void finish_loss_kernel(const double* sum, double n, double* loss) {
 }
 
 // Samples per lane and row: 16, or 8 where 16 would leave the SMs without two
-// CTAs each (256 ch x 4096 x 256 trials: TRAINSMALL).
+// CTAs each (256 ch x 4096 x 256 trials: 128 CTAs of 16, 256 of 8).
 constexpr int kSmallTile = 32 * 8;
 
 template <int MODE>
