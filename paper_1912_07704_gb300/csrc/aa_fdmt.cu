@@ -1,12 +1,22 @@
 // FDMT-style tree dedispersion (arXiv:1912.07704 Sec. 1, the dedispersion
-// module's cited work): one launch per depth of the channel tree, deepest
-// first.  Row r of a depth holds a subband's series at one delay:
+// module's cited work).  Row r of a depth of the channel tree holds a
+// subband's series at one delay:
 //   out[r][t] = U[t] + Lo[t + gap],   t < nsamp - delta_r,
 // where U and Lo are rows of the next-deeper depth (32-bit) or input channel
 // rows (8- or 16-bit leaves).  The root depth writes one FP32 row per trial
 // of the range (t < the range's output length).  Sums are exact integers.
-// HBM-bound: each output sample reads two samples and writes one; CTA = one
-// row x 1024 samples, consecutive threads on consecutive samples.
+//
+// A launch merges a group of up to five depths: a CTA takes one block (some
+// consecutive rows of the group's top depth) x one tile of samples, loads the
+// windows it needs into slots of shared memory and merges depth after depth
+// there; only the top depth's rows go to memory.  With one launch per depth every
+// sum read two samples and wrote one: 75 GB and 15.2 ms for 2^17 samples of 4096
+// channels under the four ranges of the SKA plan; in groups of 4-3-5 depths it
+// is 10 GB and 5.9 ms.  Shared memory bounds it (its pipe is 61-68 % busy; two
+// CTAs of an SM hide the loads of each other).  A lane sums four consecutive
+// samples: with one sample a lane (12 wavefronts for 128 sums instead of 16, but
+// twice the instructions) it was 7.0 ms; blocks of 52 and 71 KB, four and three to
+// an SM, 8.2 and 6.9 ms (more of their windows is overlap).
 #include <cstdint>
 
 #include "aa_internal.h"
@@ -14,59 +24,161 @@
 namespace aa {
 namespace {
 
-constexpr int kFdmtThreads = 256;
-constexpr int kFdmtPerThread = 4;
-constexpr int kFdmtTile = kFdmtThreads * kFdmtPerThread;
+constexpr int kFdmtThreads = 512;
+constexpr int kFdmtWarps = kFdmtThreads / 32;
 
-template <int EB>
-__device__ __forceinline__ uint32_t fdmt_leaf(const void* leaves, int64_t pitch, int32_t c, int64_t t) {
-    if constexpr (EB == 1) return static_cast<const uint8_t*>(leaves)[(int64_t)c * pitch + t];
-    else return static_cast<const uint16_t*>(leaves)[(int64_t)c * pitch + t];
+struct FdmtArgs {
+    const FdmtBlock* blocks;
+    const FdmtLoad* loads;
+    const FdmtOp* ops;
+    const void* leaves;
+    int64_t leaf_pitch;
+    const uint32_t* prev;
+    uint32_t* out;
+    int64_t pitch;
+    int64_t nsamp;
+    float* fout;
+    int64_t fpitch, flen;
+    int32_t nblocks, tile, levels;
+    int32_t op_words;  // words before the slots
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t* dst, const uint32_t* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(bytes)
+                 : "memory");
+}
+
+// Sums of one op, four consecutive samples a lane: the upper series starts at a
+// multiple of four words, the lower one anywhere (its place within four words
+// is the same for all lanes).
+template <class Put>
+__device__ __forceinline__ void merge(const uint32_t* slots, const int4& op, int lane, Put put) {
+    const uint32_t* u = slots + (op.x & 0xffff);
+    const uint32_t lo = (uint32_t)op.x >> 16;
+    const uint32_t* l = slots + (lo & ~3u);
+    const int r = lo & 3;
+    auto run = [&](auto pick) {
+#pragma unroll 2
+        for (int i = 4 * lane; i < op.z; i += 128) {
+            const uint4 a = *reinterpret_cast<const uint4*>(u + i);
+            const uint4 b = pick(i);
+            put(i, make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w));
+        }
+    };
+    auto at = [&](int i) { return *reinterpret_cast<const uint4*>(l + i); };
+    if (r == 0) run([&](int i) { return at(i); });
+    else if (r == 1) run([&](int i) { const uint4 p = at(i); return make_uint4(p.y, p.z, p.w, l[i + 4]); });
+    else if (r == 2) run([&](int i) { const uint4 p = at(i); const uint2 q = *reinterpret_cast<const uint2*>(l + i + 4); return make_uint4(p.z, p.w, q.x, q.y); });
+    else run([&](int i) { const uint4 p = at(i), q = at(i + 4); return make_uint4(p.w, q.x, q.y, q.z); });
 }
 
 template <int EB, bool FINAL>
-__global__ void __launch_bounds__(kFdmtThreads)
-    fdmt_depth_kernel(const FdmtRow* __restrict__ rows, const void* __restrict__ leaves, int64_t leaf_pitch,
-                      const uint32_t* __restrict__ prev, uint32_t* __restrict__ out, int64_t pitch, int64_t nsamp,
-                      float* __restrict__ fout, int64_t fpitch, int64_t flen) {
-    const FdmtRow r = rows[blockIdx.y];
-    const int64_t n = FINAL ? flen : nsamp - r.delta;
-    const int64_t t0 = (int64_t)blockIdx.x * kFdmtTile;
-    if (t0 >= n) return;
-    const bool uleaf = r.u < 0, lleaf = r.l < 0;
-    const uint32_t* up = uleaf ? nullptr : prev + (int64_t)r.u * pitch;
-    const uint32_t* lp = lleaf ? nullptr : prev + (int64_t)r.l * pitch + r.gap;
-    const int32_t uc = uleaf ? -(r.u + 1) : 0, lc = lleaf ? -(r.l + 1) : 0;
-#pragma unroll
-    for (int k = 0; k < kFdmtPerThread; ++k) {
-        const int64_t t = t0 + threadIdx.x + k * kFdmtThreads;
-        if (t < n) {
-            const uint32_t a = uleaf ? fdmt_leaf<EB>(leaves, leaf_pitch, uc, t) : __ldg(up + t);
-            const uint32_t b = lleaf ? fdmt_leaf<EB>(leaves, leaf_pitch, lc, t + r.gap) : __ldg(lp + t);
-            if constexpr (FINAL) fout[(int64_t)blockIdx.y * fpitch + t] = (float)(a + b);
-            else out[(int64_t)blockIdx.y * pitch + t] = a + b;
+__global__ void __launch_bounds__(kFdmtThreads, 2) fdmt_group_kernel(FdmtArgs a) {
+    extern __shared__ __align__(16) uint32_t fdmt_smem[];
+    FdmtOp* ops = reinterpret_cast<FdmtOp*>(fdmt_smem);
+    uint32_t* slots = fdmt_smem + a.op_words;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const FdmtBlock& b = a.blocks[blockIdx.x % a.nblocks];  // neighbouring blocks share rows: side by side
+    const int64_t t0 = (int64_t)(blockIdx.x / a.nblocks) * a.tile;
+    const int load0 = __ldg(&b.load0), nload = __ldg(&b.nload), op0 = __ldg(&b.op0), nops = __ldg(&b.end[a.levels - 1]);
+    for (int i = warp; i < nload; i += kFdmtWarps) {
+        const int4 l = __ldg(reinterpret_cast<const int4*>(a.loads + load0 + i));  // ref, lo, dst, n
+        const int64_t t = t0 + l.y;
+        uint32_t* dst = slots + l.z;
+        if (l.x >= 0) {
+            const uint32_t* src = a.prev + (int64_t)l.x * a.pitch;
+            for (int j = 4 * lane; j < l.w; j += 128) {
+                const bool in = t + j < a.pitch;  // beyond the row: zeros, which no valid output reads
+                cp_async16(dst + j, in ? src + t + j : a.prev, in ? 16 : 0);
+            }
+        } else {
+            const int64_t row = (int64_t)(-(l.x + 1)) * a.leaf_pitch;
+#pragma unroll 4
+            for (int j = 4 * lane; j < l.w; j += 128) {
+                uint4 v = make_uint4(0, 0, 0, 0);
+                if (t + j < a.nsamp) {  // the pitch is a multiple of four samples
+                    if constexpr (EB == 1) {
+                        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.leaves) + row + t + j));
+                        v = make_uint4(w & 0xff, (w >> 8) & 0xff, (w >> 16) & 0xff, w >> 24);
+                    } else {
+                        const uint2 w = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(a.leaves) + row + t + j));
+                        v = make_uint4(w.x & 0xffff, w.x >> 16, w.y & 0xffff, w.y >> 16);
+                    }
+                }
+                *reinterpret_cast<uint4*>(dst + j) = v;
+            }
         }
+    }
+    for (int i = threadIdx.x; i < nops; i += kFdmtThreads)
+        reinterpret_cast<int4*>(ops)[i] = __ldg(reinterpret_cast<const int4*>(a.ops + op0) + i);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    int begin = 0;
+#pragma unroll 1
+    for (int lev = 0; lev < a.levels - 1; ++lev) {
+        const int end = __ldg(&b.end[lev]);
+        for (int o = begin + warp; o < end; o += kFdmtWarps) {
+            const int4 op = reinterpret_cast<const int4*>(ops)[o];
+            uint32_t* d = slots + op.y;
+            merge(slots, op, lane, [&](int i, uint4 v) { *reinterpret_cast<uint4*>(d + i) = v; });
+        }
+        begin = end;
+        __syncthreads();
+    }
+    for (int o = begin + warp; o < nops; o += kFdmtWarps) {
+        const int4 op = reinterpret_cast<const int4*>(ops)[o];
+        const int64_t left = (FINAL ? a.flen : a.nsamp - op.w) - t0;
+        const int n = left < op.z ? (int)left : op.z;  // op.z: the tile
+        merge(slots, op, lane, [&](int i, uint4 v) {
+            if constexpr (FINAL) {
+                float* row = a.fout + (int64_t)op.y * a.fpitch + t0 + i;
+                if (i + 4 <= n) *reinterpret_cast<float4*>(row) = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
+                else {
+                    if (i < n) row[0] = (float)v.x;
+                    if (i + 1 < n) row[1] = (float)v.y;
+                    if (i + 2 < n) row[2] = (float)v.z;
+                }
+            } else if (i < n) {  // the pitch is a multiple of four samples; beyond a row's valid part nothing is read
+                *reinterpret_cast<uint4*>(a.out + (int64_t)op.y * a.pitch + t0 + i) = v;
+            }
+        });
     }
 }
 
 }  // namespace
 
-cudaError_t launch_fdmt_depth(const FdmtRow* rows, int nrows, int leaf_elem, const void* leaves,
+cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_elem, const void* leaves,
                               int64_t leaf_pitch, const uint32_t* prev, uint32_t* out, int64_t pitch,
                               int64_t nsamp, float* fout, int64_t fpitch, int64_t flen, cudaStream_t s) {
-    if (nrows <= 0) return cudaSuccess;
-    if (nrows > 65535) return cudaErrorInvalidConfiguration;
     const bool fin = fout != nullptr;
     const int64_t n = fin ? flen : nsamp;
-    if (n <= 0) return cudaSuccess;
-    const dim3 grid((unsigned)((n + kFdmtTile - 1) / kFdmtTile), (unsigned)nrows);
-    if (leaf_elem == 1) {
-        if (fin) fdmt_depth_kernel<1, true><<<grid, kFdmtThreads, 0, s>>>(rows, leaves, leaf_pitch, prev, out, pitch, nsamp, fout, fpitch, flen);
-        else fdmt_depth_kernel<1, false><<<grid, kFdmtThreads, 0, s>>>(rows, leaves, leaf_pitch, prev, out, pitch, nsamp, fout, fpitch, flen);
-    } else {
-        if (fin) fdmt_depth_kernel<2, true><<<grid, kFdmtThreads, 0, s>>>(rows, leaves, leaf_pitch, prev, out, pitch, nsamp, fout, fpitch, flen);
-        else fdmt_depth_kernel<2, false><<<grid, kFdmtThreads, 0, s>>>(rows, leaves, leaf_pitch, prev, out, pitch, nsamp, fout, fpitch, flen);
-    }
+    if (n <= 0 || g.nblocks <= 0) return cudaSuccess;
+    const int64_t grid = (n + g.tile - 1) / g.tile * g.nblocks;
+    if (grid >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    FdmtArgs a{};
+    a.blocks = fd.d_blocks + g.block0;
+    a.loads = fd.d_loads;
+    a.ops = fd.d_ops;
+    a.leaves = leaves;
+    a.leaf_pitch = leaf_pitch;
+    a.prev = prev;
+    a.out = out;
+    a.pitch = pitch;
+    a.nsamp = nsamp;
+    a.fout = fout;
+    a.fpitch = fpitch;
+    a.flen = flen;
+    a.nblocks = g.nblocks;
+    a.tile = g.tile;
+    a.levels = g.bottom - g.top + 1;
+    a.op_words = g.max_ops * 4;
+    const size_t smem = ((size_t)a.op_words + (size_t)g.words) * 4;
+    auto kern = leaf_elem == 1 ? (fin ? fdmt_group_kernel<1, true> : fdmt_group_kernel<1, false>)
+                               : (fin ? fdmt_group_kernel<2, true> : fdmt_group_kernel<2, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)grid, kFdmtThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -112,15 +112,54 @@ struct FdmtRow {
     int32_t delta;  // this row's delay: valid for t < nsamp_dec - delta
 };
 static_assert(sizeof(FdmtRow) == 16, "FDMT row layout");
+// A launch merges a group of depths in blocks: consecutive rows of the group's
+// top depth, the windows they read loaded into slots of shared memory, the
+// depths between merged there.  Offsets are in 32-bit words of the slots.
+constexpr int kFdmtMaxLevels = 5;
+constexpr int kFdmtSlotWords = 108 * 1024 / 4;  // most words of the slots
+struct FdmtLoad {
+    int32_t ref;  // row of the next-deeper stored depth, or channel -(ref + 1)
+    int32_t lo;   // first sample, relative to the tile (multiple of 4)
+    int32_t dst, n;  // n samples (multiple of 4) to word dst
+};
+struct FdmtOp {
+    uint32_t src;  // words of the upper (low half) and lower (high half) series
+    int32_t dst;   // word of the sum; the top depth's ops: output row
+    int32_t n;     // samples
+    int32_t delta; // the row's delay
+};
+struct FdmtBlock {
+    int32_t load0, nload, op0;
+    int32_t end[kFdmtMaxLevels];  // ops of the depths, deepest first, end here (from op0)
+};
+static_assert(sizeof(FdmtLoad) == 16 && sizeof(FdmtOp) == 16 && sizeof(FdmtBlock) == 32, "FDMT block tables");
+struct FdmtGroup {
+    int top = 0, bottom = 0;  // depths merged
+    int tile = 0;             // samples of a block
+    int32_t width = 0, words = 0;  // words of a slot, of all slots
+    int32_t max_ops = 0;
+    int64_t block0 = 0;
+    int32_t nblocks = 0;
+};
 struct FdmtPlan {
     int depths = 0;               // merge levels (the root is depth 0)
     std::vector<FdmtRow> rows;    // deepest depth first, the root's (one per trial) last
     std::vector<int64_t> first;   // [depths + 1]: start of each depth's rows in that order
     int32_t max_rows = 0;         // rows of the largest intermediate depth
     double work = 1.0;            // rows computed / (ndm x nchans): adds relative to direct
-    FdmtRow* d_rows = nullptr;
+    std::vector<FdmtGroup> groups;  // shallowest first
+    std::vector<FdmtBlock> blocks;
+    std::vector<FdmtLoad> loads;
+    std::vector<FdmtOp> ops;
+    const FdmtBlock* d_blocks = nullptr;
+    const FdmtLoad* d_loads = nullptr;
+    const FdmtOp* d_ops = nullptr;
 };
-cudaError_t launch_fdmt_depth(const FdmtRow* rows, int nrows, int leaf_elem, const void* leaves,
+// nodes: first row of each subband of each depth.  False: a block that fits no tile.
+bool build_fdmt_groups(FdmtPlan& fd, int32_t nchans, int elem, const std::vector<std::vector<int32_t>>& nodes);
+bool fdmt_shifts(const FdmtPlan& fd, int32_t nchans, int32_t ndm, int32_t* out);
+// One group: rows of its top depth to `out` (pitch), or to `fout` (the root).
+cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_elem, const void* leaves,
                               int64_t leaf_pitch, const uint32_t* prev, uint32_t* out, int64_t pitch,
                               int64_t nsamp, float* fout, int64_t fpitch, int64_t flen, cudaStream_t s);
 

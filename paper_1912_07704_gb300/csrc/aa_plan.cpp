@@ -9,6 +9,7 @@
 #include <cstring>
 #include <cstdint>
 #include <new>
+#include <type_traits>
 
 #include "aa_internal.h"
 
@@ -458,7 +459,8 @@ static aa_status upload_subband(aa_plan* p) {
     size_t bytes = 0;
     for (const auto& r : p->ranges) {
         if (r.strategy == 2) bytes += table_bytes(r.sb.rel.size()) + table_bytes(r.sb.s2.size());
-        if (r.strategy == 3) bytes += table_bytes(r.fd.rows.size() * 4);
+        if (r.strategy == 3)  // 16-byte rows of 4 words, 32-byte blocks
+            bytes += table_bytes(r.fd.blocks.size() * 8) + table_bytes(r.fd.loads.size() * 4) + table_bytes(r.fd.ops.size() * 4);
     }
     int prev = -1;
     cudaGetDevice(&prev);
@@ -469,7 +471,9 @@ static aa_status upload_subband(aa_plan* p) {
     }
     for (auto& r : p->ranges) {
         r.sb.d_rel = r.sb.d_s2 = nullptr;
-        r.fd.d_rows = nullptr;
+        r.fd.d_blocks = nullptr;
+        r.fd.d_loads = nullptr;
+        r.fd.d_ops = nullptr;
     }
     aa_status st = AA_OK;
     if (bytes) {
@@ -484,11 +488,16 @@ static aa_status upload_subband(aa_plan* p) {
             size_t off = 0;
             for (auto& r : p->ranges) {
                 if (r.strategy == 3) {
-                    r.fd.d_rows = reinterpret_cast<FdmtRow*>((char*)mem + off);
-                    off += table_bytes(r.fd.rows.size() * 4);
-                    if (e == cudaSuccess)
-                        e = cudaMemcpy(r.fd.d_rows, r.fd.rows.data(), r.fd.rows.size() * sizeof(FdmtRow),
-                                       cudaMemcpyHostToDevice);
+                    auto put = [&](auto*& d, const auto& v) {
+                        void* at = (char*)mem + off;
+                        const size_t n = v.size() * sizeof(v[0]);
+                        off += table_bytes(n / 4);
+                        d = static_cast<std::remove_reference_t<decltype(d)>>(at);
+                        if (e == cudaSuccess && n) e = cudaMemcpy(at, v.data(), n, cudaMemcpyHostToDevice);
+                    };
+                    put(r.fd.d_blocks, r.fd.blocks);
+                    put(r.fd.d_loads, r.fd.loads);
+                    put(r.fd.d_ops, r.fd.ops);
                     continue;
                 }
                 if (r.strategy != 2) continue;
@@ -1027,6 +1036,13 @@ aa_status aa_plan_set_fdmt(aa_plan* p, int32_t r) {
             return AA_ERR_STATE;
         }
     fd.work = ndm > 0 ? (double)fd.rows.size() / ((double)ndm * C) : 1.0;
+    std::vector<std::vector<int32_t>> nodes(depth.size());  // first row of each node
+    for (size_t d = 0; d < depth.size(); ++d)
+        for (const Node& n : depth[d]) nodes[d].push_back(n.row0);
+    if (!build_fdmt_groups(fd, C, g.elem, nodes)) {
+        set_error("internal: FDMT blocks fit no tile");
+        return AA_ERR_STATE;
+    }
     const FdmtPlan old = g.fd;
     const int old_strategy = g.strategy;
     g.fd = std::move(fd);
@@ -1064,20 +1080,10 @@ aa_status aa_plan_effective_shifts(const aa_plan* p, int32_t r, int32_t* out, in
         }
         return AA_OK;
     }
-    if (g.strategy == 3) {  // walk the tree from each trial's root row
-        const FdmtPlan& fd = g.fd;
-        // rows of depth d start at fd.first[depths - 1 - d]
-        auto walk = [&](auto&& self, int d, int32_t row, int64_t base, int32_t* e) -> void {
-            const FdmtRow& x = fd.rows[(size_t)(fd.first[(size_t)(fd.depths - 1 - d)] + row)];
-            for (int half = 0; half < 2; ++half) {
-                const int32_t ref = half ? x.l : x.u;
-                const int64_t b = base + (half ? x.gap : 0);
-                if (ref < 0) e[-(ref + 1)] = (int32_t)b;
-                else self(self, d + 1, ref, b, e);
-            }
-        };
-        for (int32_t i = 0; i < ndm; ++i) walk(walk, 0, i, 0, out + (int64_t)i * C);
-        return AA_OK;
+    if (g.strategy == 3) {
+        if (ndm == 0 || fdmt_shifts(g.fd, C, ndm, out)) return AA_OK;
+        set_error("internal: inconsistent FDMT tables");
+        return AA_ERR_STATE;
     }
     if (uses_bands(g)) {
         if (band_shifts(g.bands, C, ndm, out)) return AA_OK;

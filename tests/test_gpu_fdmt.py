@@ -85,3 +85,21 @@ def test_fdmt_refused_where_not_striped(oracle):
     with pytest.raises(abi.AAError):
         plan.fused_ws_bytes(T, 32)
     plan.close()
+
+
+@pytest.mark.parametrize("nchans,foff,T,dm", [
+    (3, -1.0, 5000, (3.0, 0.0, 5, 1)),         # equal trials, a leaf beside a node
+    (33, -1.5, 6001, (0.0, 0.05, 70, 1)),      # six depths, trials that share a delay
+    (65, 0.75, 4099, (20.0, 9.0, 33, 3)),      # rising band, decimated, trials far apart
+    (129, -0.75, 3001, (30.0, 4.0, 1, 1)),     # one trial
+    (300, -1.0, 12345, (0.0, 0.7, 130, 2)),    # several blocks and groups, a ragged last tile
+])
+def test_fdmt_groups_of_depths(oracle, nchans, foff, T, dm):
+    """Rows merged in groups of depths: exact sums at the edges of blocks, groups and tiles."""
+    x = np.random.default_rng(nchans).integers(0, 256, size=(nchans, T), dtype=np.uint8)
+    with Plan(nchans, 1400.0, foff, 64e-6, [dm]) as plan:
+        plan.set_fdmt(0)
+        out, *_ = run_gpu(plan, x, 8, 6.0)
+        g = oracle.plan(nchans, 1400.0, foff, 64e-6, [dm], T)[0]
+        y, _ = oracle.dedisperse_fdmt(x, nchans, 1400.0, foff, 64e-6, g)
+        assert np.array_equal(plan.range_views(out, T)[0].double().cpu().numpy(), y.astype(np.float64))
