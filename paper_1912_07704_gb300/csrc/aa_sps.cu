@@ -403,10 +403,15 @@ constexpr float kBig = 1.2676506002282294e30f;  // 2^100
 // S64): the first 8 chunks one by one, then groups of 8, from 64 on groups of
 // 64, opened where a thread's bound reaches its floor.  Eight bounds of one
 // level are computed side by side before the warp looks at them (one by one,
-// each with its vote, they took 330 cycles each).  A chunk to evaluate waits
-// until its thread has a second one.  Both are written down once, in one loop:
-// with an evaluation and bounds at each place that wants them the kernel
-// waited for instructions more than for anything else (2.6 of 10 stalls).
+// each with its vote, they took 330 cycles each).  The chunks to evaluate wait
+// in a queue of the thread, eight groups of eight as their bits, and are looked
+// at again when their turn comes: a warp evaluates when a queue is full and at
+// the end of the pass, so that most of its threads take part (a beam of 1024
+// channels x 48611 samples with two pulses, 2000 trials, W = 8192: 3.14 ms with
+// one chunk waiting, 2.23 with the queue; without pulses 0.92).  Both are
+// written down once, in one loop: with an evaluation and bounds at each place
+// that wants them the kernel waited for instructions more than for anything
+// else (2.6 of 10 stalls).
 // Skipping below
 // the running B, or below a lower bound of it, is exact for every start (such
 // a chunk changes neither B nor the first chunk that reaches it; the chunk
@@ -480,14 +485,16 @@ __device__ __forceinline__ void eval_chunk(const float* __restrict__ pw, const f
 // 96 series of 64006 samples, W = 256 / 1024 / 2048: in turn 220 / 752 / 1449
 // us, by bounds 307 / 802 / 1084).
 constexpr int kEvery = kTabWidths / M;
+constexpr unsigned kQueue = 8;
 // Returns the chunks this thread evaluated.  C: the first chunk reaching B[i] in
 // 16-bit halves, starts 2 k and 2 k + 1 in C[k] (16 registers of them spilled).
-// Q: Q16, S1, S8 and S64, nq entries each.  LOW: cut is not above zero.
+// Q: Q16, S1, S8 and S64, nq entries each.  queue: the thread's entries, kQueue of them NT apart.
+// LOW: cut is not above zero.
 template <bool LOW>
 __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const float4* tab, const float2* __restrict__ gtab,
                                              int nch, int max_width, const float (&base)[M], const WidthBounds& bnd,
-                                             const float* Q, int nq, float cut, const uint32_t* lmask, float (&B)[M],
-                                             uint32_t (&C)[M / 2]) {
+                                             const float* Q, int nq, uint16_t* queue, float cut, const uint32_t* lmask,
+                                             float (&B)[M], uint32_t (&C)[M / 2]) {
     const int t = threadIdx.x;
     const float* pb = P + M * t;
 #pragma unroll
@@ -512,7 +519,9 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
     }
     const float *s1 = Q + nq + t, *s8 = s1 + nq, *s64 = s8 + nq;
     float F = cut - bnd.S;              // the floor less the bounds' margin
-    int evaluated = 0, pend = 0;        // pend: chunk waiting to be evaluated (-1: none), first chunk 0
+    int evaluated = 0;
+    unsigned fill = 0;                  // entries in the queue << 16 | the first one's place (mod kQueue)
+    unsigned cur = 0;                   // the taken entry: chunk of its first bit << 5 | bits
     bool last = nch == 1, found = false;
     int pass = -1;
     // Groups of 64 chunks from c512, of 8 from c64, chunks from c8: a thread's
@@ -524,6 +533,17 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
     unsigned keep = ~0u;  // bits that the level above lets through
     for (;;) {
         if (step == kEval) {
+            int pend = pass < 0 ? 0 : -1;  // chunk to evaluate: first chunk 0, then the queue's
+            while (pend < 0 && ((cur & 0xffu) || fill >> 16)) {
+                if (!(cur & 0xffu)) {
+                    cur = queue[(fill % kQueue) * NT];
+                    fill -= 0xffffu;  // one entry fewer, the next place
+                }
+                const int c = (int)(cur >> 8) * 8 + __ffs((int)cur) - 1;
+                cur &= cur - 1;
+                if (bnd.reaches<LOW>(s1[c], (float)(M * c) + bnd.w_first(1), bnd.rs + c, 1, F)) pend = c;
+            }
+            __syncwarp();
             if (pend >= 0) {
                 float Bc[M];
                 const bool staged = M * pend < kTabWidths;
@@ -540,8 +560,8 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
                 }
                 F = fmaxf(F, low - bnd.S);
                 ++evaluated;
-                pend = -1;
             }
+            if (__any_sync(0xffffffffu, last ? (cur & 0xffu) || fill >> 16 : fill >> 16 == kQueue)) continue;
             if (last) break;
             step = pass < 0 ? kFirst : kBounds;
         }
@@ -602,17 +622,9 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
                             if (((in >> k) & 1u) && M * (c8 + k) + 31 <= max_width)
                                 F = fmaxf(F, bnd.lower(Q[t + c8 + k + 1], c8 + k) - bnd.S);
                     }
-                } else {
-                    if (in && pend < 0) {
-                        pend = c8 + __ffs((int)in) - 1;
-                        in &= in - 1;
-                    }
-                    if (__any_sync(0xffffffffu, in)) {  // evaluate, then look at the rest again
-                        step = kEval;
-                        level = 1;
-                        keep = in;
-                        continue;
-                    }
+                } else if (in) {
+                    queue[((fill + (fill >> 16)) % kQueue) * NT] = (uint16_t)(c8 << 5 | in);
+                    fill += 0x10000u;
                 }
             }
         }
@@ -636,9 +648,9 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
         } else if (pass == 0 && found) {
             step = kFirst;
         } else {
-            step = kEval;
             last = true;
         }
+        if (__any_sync(0xffffffffu, last || fill >> 16 == kQueue)) step = kEval;
     }
     return evaluated;
 }
@@ -691,7 +703,7 @@ __device__ __noinline__ float boxcar_exact_slot(const float* __restrict__ ys,
 // candidate entries: at most every second start is a peak), the next tile's
 // new samples, the bounds' factors, the ladder's mask.
 __host__ __device__ constexpr int sps_lists_words(int wpad) {
-    const int q = 4 * sps_q16(wpad);
+    const int q = 4 * sps_q16(wpad) + (int)kQueue * NT / 2;  // and the search's queues
     return q > 2 * kSpsTile ? q : 2 * kSpsTile;
 }
 
@@ -712,13 +724,13 @@ __host__ __device__ constexpr int sps_lists_words(int wpad) {
 // With 16 warps an SM (128 registers: a thread's starts, their B, the window of
 // a chunk) the tile's chain of short phases is what takes the time, so the
 // phases are kept few and their barriers fewer.  4096 channels x 2^20 samples,
-// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 40.5 ms; of that (clock64) the
-// width search 14.6, waiting for a tile's slowest warp 8.0, block maxima 4.4,
+// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 34.8 ms; of 40.5 before the
+// search's queues (clock64) the width search 14.6, waiting for a tile's slowest warp 8.0, block maxima 4.4,
 // sums of new samples 2.8, candidates' widths 2.1, fresh tiles 1.5, peaks 1.4,
 // sliding 1.4.  Steps on the way: a warp's union of 128-width segments 92, the
 // chunks of each thread by lower bounds 66, their bounds eight at a time in one
 // loop 57, the new samples by cp.async, 32-bit sums, peaks from registers and
-// widths by half-warps 45, chunk numbers packed 40.5.
+// widths by half-warps 45, chunk numbers packed 40.5, queues 34.8.
 template <bool LOW>
 __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t tile_lo, int64_t tile_hi,
                                              float* sm) {
@@ -951,7 +963,8 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
                 }
                 __syncthreads();
             }
-            int chunks = boxcar_search<LOW>(P, tab, gtab, wpad / M, a.max_width, base, bnd, Q, nq, cut, lmask, B, C);
+            int chunks = boxcar_search<LOW>(P, tab, gtab, wpad / M, a.max_width, base, bnd, Q, nq,
+                                            reinterpret_cast<uint16_t*>(Q + 4 * nq) + threadIdx.x, cut, lmask, B, C);
             if (a.evaluated) {
                 chunks = __reduce_add_sync(0xffffffffu, chunks);
                 if (lane == 0) atomicAdd(a.evaluated, (unsigned long long)chunks * M * M);

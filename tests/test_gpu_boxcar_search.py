@@ -27,6 +27,11 @@ def _series(kind):
         y[2, 9000:9001] += 2000
     elif kind == "ramp":  # rising then falling: long stretches of negative sums
         y += torch.linspace(-40, 40, L, device="cuda").round() * torch.tensor([[1.0], [-1.0], [0.0]], device="cuda")
+    elif kind == "flat":  # from one start on sums grow like sqrt(w): it has hundreds of chunks to evaluate
+        y = 4000 + ((y - 4000) / 25).round()
+        for row, s in enumerate((100, 5003, 12000)):
+            k = torch.arange(L - s + 1, device="cuda", dtype=torch.float64)
+            y[row, s:] += torch.diff((2000 * k.sqrt()).round()).float()
     return y
 
 
@@ -43,7 +48,7 @@ def _best(y, W):
 
 
 @pytest.mark.parametrize("W", [1, 16, 17, 127, 129, 1024, 1025, 4100, 8191, 8193, 9000])
-@pytest.mark.parametrize("kind", ["noise", "pulses", "ramp"])
+@pytest.mark.parametrize("kind", ["noise", "pulses", "ramp", "flat"])
 def test_pruned_search_equals_the_map(W, kind):
     plan = Plan(16, 1400.0, -1.0, 64e-6, [(0.0, 0.0, ROWS, 1)])
     plan.bind()
