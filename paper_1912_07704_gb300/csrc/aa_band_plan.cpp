@@ -69,8 +69,8 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
         seg.ntrials = std::min(kBandSegment, ndm - d0);
         seg.nblk = (seg.ntrials + kBandTrials - 1) / kBandTrials;
         seg.blk0 = blk_base;
+        const size_t first_copy = bp.copies.size();
         seg.row0 = (uint32_t)bp.rows.size();
-        uint64_t pre = 0;
         for (int b = 0; b < bp.nbands; ++b) {
             const int c0 = b * k, nch = std::min(k, C - c0);
             const int na = std::min(nch, 4), nb = nch - na;
@@ -125,6 +125,8 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
                 const int q = quad_keys.add(qk, fresh);
                 if (fresh) {
                     BandQuad quad;
+                    quad.blk0 = 0xffff;
+                    quad.blk1 = 0;
                     std::memcpy(quad.r, rr, sizeof rr);
                     for (int j = 0; j < cnt; ++j) max_rq = std::max(max_rq, (int)rr[j]);
                     bp.quads.push_back(quad);
@@ -157,13 +159,6 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
             max_quads = std::max(max_quads, (int)info.nqa + info.nqb);
             bp.max_ulen = std::max(bp.max_ulen, info.ulen);
             bp.max_rows = std::max(bp.max_rows, n);
-            for (int q = 0; q < n; ++q) {
-                BandRow& row = bp.rows[first_row + q];
-                row.pre = (uint32_t)pre;
-                // a window may start up to 3 words early and end up to 3 late
-                pre += (uint64_t)round_up(row.span + 8, 4);
-            }
-            if (pre > UINT32_MAX / 4) return false;
             // the blocks: which rows each uses, at which delays
             for (int g = 0; g < seg.nblk; ++g) {
                 const int i0 = g * kBandTrials, i1 = std::min(seg.ntrials, i0 + kBandTrials);
@@ -191,8 +186,8 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
                     row.blk1 = std::max<uint16_t>(row.blk1, (uint16_t)g);
                     const int32_t at = blo[q] - row.smin;
                     BandCopy c;
-                    c.row = (uint32_t)(first_row + q) - seg.row0;
-                    c.rel = row.pre + (uint32_t)(at & ~3);
+                    c.row = (uint32_t)(first_row + q) - seg.row0;  // its place follows
+                    c.rel = (uint32_t)(at & ~3);
                     c.dst = (uint32_t)dst;
                     c.n = (uint32_t)round_up(kBandWords + (bhi[q] - blo[q]) + (at & 3), 4);
                     bdst[q] = dst + (at & 3) - blo[q];  // slot word of delay s: bdst + s
@@ -216,6 +211,45 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
             bp.infos.push_back(info);
         }
         seg.nrows = (int64_t)bp.rows.size() - seg.row0;
+        BandRow* rows = bp.rows.data() + seg.row0;
+        for (int b = 0; b < bp.nbands; ++b) {
+            const BandInfo& info = bp.infos[bp.infos.size() - bp.nbands + b];
+            for (int q = 0; q < info.nrows; ++q) {
+                const BandRow& row = bp.rows[info.row0 + q];
+                for (const uint16_t at : {row.qa, row.qb}) {
+                    if (at == 0xffff) continue;
+                    BandQuad& quad = bp.quads[info.quad0 + at];
+                    quad.blk0 = std::min(quad.blk0, row.blk0);
+                    quad.blk1 = std::max(quad.blk1, row.blk1);
+                }
+            }
+        }
+        // places by first block, counting sort
+        std::vector<uint32_t> at((size_t)seg.nblk + 1, 0), order((size_t)seg.nrows);
+        for (int64_t i = 0; i < seg.nrows; ++i) ++at[rows[i].blk0 + 1];
+        for (int g = 0; g < seg.nblk; ++g) at[g + 1] += at[g];
+        for (int64_t i = 0; i < seg.nrows; ++i) order[at[rows[i].blk0]++] = (uint32_t)i;
+        uint64_t pre = 0;
+        seg.first.assign((size_t)seg.nblk, BandSegment::Mark{-1, 0});
+        seg.end.assign((size_t)seg.nblk, BandSegment::Mark{0, 0});
+        int reached = 0;  // blocks whose first place is known
+        for (int64_t i = 0; i < seg.nrows; ++i) {
+            BandRow& row = rows[order[(size_t)i]];
+            row.id = (uint32_t)i;
+            row.pre = (uint32_t)pre;
+            for (; reached <= row.blk1; ++reached) seg.first[(size_t)reached] = {i, (int64_t)pre};
+            // a window may start up to 3 words early and end up to 3 late
+            pre += (uint64_t)round_up(row.span + 8, 4);
+            if (pre > UINT32_MAX / 4) return false;
+            seg.end[row.blk0] = {i + 1, (int64_t)pre};
+        }
+        for (int g = 1; g < seg.nblk; ++g)
+            if (seg.end[(size_t)g].id < seg.end[(size_t)g - 1].id) seg.end[(size_t)g] = seg.end[(size_t)g - 1];
+        for (size_t i = first_copy; i < bp.copies.size(); ++i) {
+            const BandRow& row = rows[bp.copies[i].row];
+            bp.copies[i].row = row.id;
+            bp.copies[i].rel += row.pre;
+        }
         seg.pre = (int64_t)pre;
         bp.segs.push_back(seg);
         blk_base += seg.nblk;
@@ -268,6 +302,11 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
 bool band_shifts(const BandPlan& bp, int C, int ndm, int32_t* out) {
     for (size_t q = 0; q < bp.segs.size(); ++q) {
         const BandSegment& seg = bp.segs[q];
+        std::vector<uint32_t> of((size_t)seg.nrows);  // row of each place
+        for (int64_t i = 0; i < seg.nrows; ++i) {
+            if (bp.rows[seg.row0 + i].id >= seg.nrows) return false;
+            of[bp.rows[seg.row0 + i].id] = seg.row0 + (uint32_t)i;
+        }
         for (int i = 0; i < seg.ntrials; ++i)
             for (int b = 0; b < bp.nbands; ++b) {
                 const int npad = (bp.nbands + 1) & ~1;
@@ -282,13 +321,16 @@ bool band_shifts(const BandPlan& bp, int C, int ndm, int32_t* out) {
                 if (!c || off + kBandWords > c->dst + c->n || c->dst + c->n > (uint32_t)h.words + (b & 1 ? bp.heads[bb - 1].words : 0) ||
                     h.place + kBandTrials + c->dst + c->n > (uint32_t)bp.ring_words || c->row >= seg.nrows) return false;
                 const BandInfo& info = bp.infos[q * bp.nbands + b];
-                const BandRow& row = bp.rows[seg.row0 + c->row];
+                const BandRow& row = bp.rows[of[c->row]];
+                if (row.id != c->row || of[c->row] < info.row0 || of[c->row] >= info.row0 + info.nrows) return false;
                 const int32_t at = (int32_t)(c->rel - row.pre + off - c->dst);  // row delay - row.smin
-                const uint32_t next = c->row + 1 < seg.nrows ? bp.rows[seg.row0 + c->row + 1].pre : (uint32_t)seg.pre;
+                const uint32_t next = c->row + 1 < seg.nrows ? bp.rows[of[c->row + 1]].pre : (uint32_t)seg.pre;
                 if (at < 0 || at > row.span || c->rel + c->n > next + kBandWords) return false;
-                if (i / kBandTrials < row.blk0 || i / kBandTrials > row.blk1) return false;
+                const int g = i / kBandTrials;
+                if (g < row.blk0 || g > row.blk1 || c->row < seg.first[(size_t)g].id || c->row >= seg.end[(size_t)g].id) return false;
                 for (int j = 0; j < info.nch; ++j) {
                     const BandQuad& quad = bp.quads[info.quad0 + (j < 4 ? row.qa : row.qb)];
+                    if (g < quad.blk0 || g > quad.blk1) return false;
                     out[(size_t)(seg.trial0 + i) * C + info.c0 + j] = row.smin + at + (j < 4 ? row.ea : row.eb) + quad.r[j & 3];
                 }
             }
@@ -318,22 +360,37 @@ void build_bands(RangePlan& r, int C) {
     if (best.ok && best.cost < 0.6 * direct) r.bands = std::move(best);
 }
 
-static int64_t bytes_for(const BandPlan& bp, int64_t ntiles) {
-    int64_t words = 0;
-    for (const BandSegment& s : bp.segs) words = std::max(words, s.nrows * ntiles * kBandWords + s.pre);
-    return round_up(std::min(words * 4, kBandBytesMax), 256);
+void band_window(const BandSegment& s, int g0, int g1, int64_t& id, int64_t& pre, int64_t& nrows, int64_t& words) {
+    id = s.first[(size_t)g0].id;
+    pre = s.first[(size_t)g0].pre;
+    nrows = s.end[(size_t)g1].id - id;
+    words = s.end[(size_t)g1].pre - pre;
+}
+
+// bytes for ntiles tiles of the rows that any nblk blocks of a segment use
+static int64_t bytes_for(const BandPlan& bp, int64_t ntiles, int nblk) {
+    int64_t most = 0;
+    for (const BandSegment& s : bp.segs)
+        for (int g = 0; g < s.nblk; ++g) {
+            int64_t id, pre, nrows, words;
+            band_window(s, g, std::min(s.nblk, g + nblk) - 1, id, pre, nrows, words);
+            most = std::max(most, nrows * ntiles * kBandWords + words);
+        }
+    return round_up(std::min(most * 4, kBandBytesMax), 256);
 }
 
 int64_t band_bytes(const BandPlan& bp, int64_t length) {
     if (!bp.ok || length <= 0) return 0;
-    return bytes_for(bp, (length + 2 * kBandWords - 1) / (2 * kBandWords));
+    return bytes_for(bp, (length + 2 * kBandWords - 1) / (2 * kBandWords), kBandSegment / kBandTrials);
 }
 
 int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials) {
     if (!bp.ok || length <= 0) return 0;
     const int64_t nblk = std::max(1, trials / kBandTrials);
     const int64_t tiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
-    return bytes_for(bp, std::min<int64_t>(tiles, (2 * 152 + nblk - 1) / nblk));
+    // a stripe that does not begin with a block touches one more
+    return bytes_for(bp, std::min<int64_t>(tiles, std::max<int64_t>(kBandLeastTiles, (2 * 152 + nblk - 1) / nblk)),
+                     (int)nblk + (trials % kBandTrials != 0));
 }
 
 }  // namespace aa

@@ -87,8 +87,7 @@ struct RowArgs {
     const BandInfo* infos;   // of the segment
     const BandRow* rows;     // of the range
     const BandQuad* quads;
-    uint32_t seg_row0;
-    uint32_t* out;
+    uint32_t* out;     // where place 0 would lie (the buffer may begin with a later one)
     int32_t k, tile, raw_words, quad_words, max_quads, nbands;
     int32_t dec;  // EB = 0: samples summed as they are read
 };
@@ -147,16 +146,16 @@ __global__ void __launch_bounds__(kRowThreads, 6) band_rows_kernel(RowArgs a) {
     uint32_t* raw = rsm;
     uint32_t* qs = rsm + a.k * a.raw_words;
     const int nquads = info.nqa + info.nqb;
-    uint32_t* s_quads = qs + a.max_quads * a.quad_words;  // descriptors: 2 words a quad, then 6 a row
-    uint32_t* s_rows = s_quads + 2 * a.max_quads;
+    uint32_t* s_quads = qs + a.max_quads * a.quad_words;  // descriptors: 3 words a quad, then 7 a row
+    uint32_t* s_rows = s_quads + 3 * a.max_quads;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     {
         const uint32_t* gq = reinterpret_cast<const uint32_t*>(a.quads + info.quad0);
         const uint32_t* gr = reinterpret_cast<const uint32_t*>(a.rows + info.row0);
-        static_assert(sizeof(BandQuad) == 8 && sizeof(BandRow) == 24, "descriptor words");
-        for (int i = threadIdx.x; i < 2 * nquads; i += kRowThreads) s_quads[i] = __ldg(gq + i);
-        for (int i = threadIdx.x; i < 6 * info.nrows; i += kRowThreads) s_rows[i] = __ldg(gr + i);
+        static_assert(sizeof(BandQuad) == 12 && sizeof(BandRow) == 28, "descriptor words");
+        for (int i = threadIdx.x; i < 3 * nquads; i += kRowThreads) s_quads[i] = __ldg(gq + i);
+        for (int i = threadIdx.x; i < 7 * info.nrows; i += kRowThreads) s_rows[i] = __ldg(gr + i);
     }
     // channels, one or more warps each: word i = samples at + i and at + hw + i;
     // samples past the row's pitch are zero (no valid output reads them)
@@ -196,7 +195,8 @@ __global__ void __launch_bounds__(kRowThreads, 6) band_rows_kernel(RowArgs a) {
     __syncthreads();
 
     for (int q = warp; q < nquads; q += kRowWarps) {
-        const uint32_t r01 = s_quads[2 * q], r23 = s_quads[2 * q + 1];
+        const uint32_t r01 = s_quads[3 * q], r23 = s_quads[3 * q + 1], blks = s_quads[3 * q + 2];
+        if ((int)(blks >> 16) < a.blk_lo || (int)(blks & 0xffffu) > a.blk_hi) continue;
         const int r1 = (int)(r01 >> 16), r2 = (int)(r23 & 0xffffu), r3 = (int)(r23 >> 16);
         const uint32_t* src = raw + (q < info.nqa ? 0 : 4) * a.raw_words + lane;
         const uint32_t* s0 = src + (r01 & 0xffffu);  // every quad has its first channel
@@ -220,13 +220,12 @@ __global__ void __launch_bounds__(kRowThreads, 6) band_rows_kernel(RowArgs a) {
     __syncthreads();
 
     for (int p = warp; p < info.nrows; p += kRowWarps) {
-        const uint32_t* d = s_rows + 6 * p;
+        const uint32_t* d = s_rows + 7 * p;
         const uint32_t blks = d[5];
         if ((int)(blks >> 16) < a.blk_lo || (int)(blks & 0xffffu) > a.blk_hi) continue;
         const int32_t smin = (int32_t)d[2];
         const int32_t i0 = max(0, smin - ua), n = min(a.tile, smin + (int32_t)d[3] + a.hw - ua) - i0 - lane;
-        const uint32_t id = info.row0 + (uint32_t)p - a.seg_row0;
-        uint32_t* dst = a.out + ((int64_t)id * a.hw + d[4]) + (ua - smin) + i0 + lane;
+        uint32_t* dst = a.out + ((int64_t)d[6] * a.hw + d[4]) + (ua - smin) + i0 + lane;
         const uint32_t* qa = qs + (d[0] & 0xffffu) * a.quad_words + (d[1] & 0xffffu) + i0 + lane;
         if ((d[0] >> 16) == 0xffffu) {
             for (int i = 0; i < n; i += 32) dst[i] = qa[i];
@@ -241,7 +240,7 @@ __global__ void __launch_bounds__(kRowThreads, 6) band_rows_kernel(RowArgs a) {
 // ------------------------------------------------------------------ sums --
 
 struct SumArgs {
-    const uint32_t* rows;
+    const uint32_t* rows;  // where place 0 would lie
     int32_t hw;
     const BandCopy* copies;
     const BandHead* heads;  // of the launch's first block
@@ -397,10 +396,13 @@ bool bands_fit(const DedispArgs& a) {
     if (!a.bands || !a.band_rows || a.length <= 0) return false;
     if (!a.grouped && g_fault_skip_chunk >= 0) return false;  // a test hook of the direct kernel
     const int64_t need = (a.length + 2 * kBandWords - 1) / (2 * kBandWords);
-    const int64_t least = std::min<int64_t>(need, 16);
+    const int64_t least = std::min<int64_t>(need, kBandLeastTiles);
     for (const BandSegment& s : a.bands->segs) {
-        if (s.trial0 >= a.trial0 + a.ndm || s.trial0 + s.ntrials <= a.trial0) continue;
-        if (s.nrows * least * kBandWords + s.pre > a.band_bytes / 4) return false;
+        const int d0 = std::max(a.trial0, s.trial0), d1 = std::min(a.trial0 + a.ndm, s.trial0 + s.ntrials);
+        if (d0 >= d1) continue;
+        int64_t id, pre, nrows, words;
+        band_window(s, (d0 - s.trial0) / kBandTrials, (d1 - 1 - s.trial0) / kBandTrials, id, pre, nrows, words);
+        if (nrows * least * kBandWords + words > a.band_bytes / 4) return false;
     }
     return true;
 }
@@ -425,7 +427,9 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
         // tiles per slab: as many as the row buffer holds, and of the upper half
         // of those counts the one whose CTAs leave the fewest SMs idle in the
         // slabs' last waves
-        const int64_t most = std::min<int64_t>(all_tiles, (a.band_bytes / 4 - seg.pre) / (seg.nrows * kBandWords));
+        int64_t id, pre, nrows, words;
+        band_window(seg, g0, g1, id, pre, nrows, words);
+        const int64_t most = std::min<int64_t>(all_tiles, (a.band_bytes / 4 - words) / (nrows * kBandWords));
         int64_t per = most, best = INT64_MAX;
         for (int64_t n = most; n >= std::max<int64_t>(1, most / 2); --n) {
             const int64_t full = all_tiles / n, rem = all_tiles % n;
@@ -448,8 +452,7 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
             ra.infos = bp.d_infos + q * bp.nbands;
             ra.rows = bp.d_rows;
             ra.quads = bp.d_quads;
-            ra.seg_row0 = seg.row0;
-            ra.out = a.band_rows;
+            ra.out = reinterpret_cast<uint32_t*>(reinterpret_cast<uintptr_t>(a.band_rows) - (uintptr_t)(id * hw + pre) * 4);
             ra.k = bp.k;
             ra.tile = bp.tile;
             ra.raw_words = bp.raw_words;
@@ -462,7 +465,7 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             SumArgs sa{};
-            sa.rows = a.band_rows;
+            sa.rows = ra.out;
             sa.hw = hw;
             sa.copies = bp.d_copies;
             sa.heads = bp.d_heads + (int64_t)(seg.blk0 + g0) * ((bp.nbands + 1) & ~1);

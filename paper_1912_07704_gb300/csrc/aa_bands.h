@@ -26,10 +26,12 @@ constexpr int kBandSegment = 1536;  // trials that share rows
 constexpr int kBandWords = 256;    // words (pairs of samples) per CTA
 constexpr int kBandMaxRows = 32;   // rows of one band used by one block (one lane each)
 constexpr int kBandBars = 32;      // pairs in the summing kernel's ring at most
+constexpr int kBandLeastTiles = 16;  // fewer tiles in the row buffer are left to the other kernels
 constexpr int kBandLag = 3;        // a place is refilled while the third pair behind its own is added
 
 struct BandQuad {  // sum of up to four channels of one half of a band
     uint16_t r[4];  // delays inside the quad, 0xffff: no such channel
+    uint16_t blk0, blk1;  // first and last block of the segment with a row of it
 };
 struct BandRow {
     uint16_t qa, qb;  // quads of the band's halves (index in the band's list, 0xffff: none)
@@ -38,6 +40,7 @@ struct BandRow {
     int32_t span;     // largest - smallest
     uint32_t pre;     // words before this row in the buffer beyond hw per earlier row
     uint16_t blk0, blk1;  // first and last block of the segment using it
+    uint32_t id;      // its place among the segment's rows in the buffer: by first block
 };
 struct BandInfo {  // one band of one segment
     uint32_t row0, quad0;     // first row / quad (in the range's lists)
@@ -47,7 +50,7 @@ struct BandInfo {  // one band of one segment
     int32_t umin, ulen;       // smallest s', and largest - smallest s' over its rows
 };
 struct BandCopy {  // one row's window as a block uses it
-    uint32_t row;  // row of the segment
+    uint32_t row;  // place of the row (BandRow::id)
     uint32_t rel;  // words from the row's first to the window's (plus the tile's), multiple of 4
     uint32_t dst;  // words into the rows of its pair's place
     uint32_t n;    // words, multiple of 4
@@ -68,6 +71,10 @@ struct BandSegment {
     int32_t trial0 = 0, ntrials = 0, nblk = 0, blk0 = 0;
     int64_t nrows = 0, pre = 0;  // rows, and words of the buffer beyond hw per row
     uint32_t row0 = 0;
+    // Rows that blocks g0 .. g1 use lie in places from first[g0] to end[g1]: a
+    // launch over some of the blocks keeps only those in its buffer.
+    struct Mark { int64_t id, pre; };
+    std::vector<Mark> first, end;
 };
 
 struct BandPlan {
@@ -93,5 +100,9 @@ struct BandPlan {
     const BandHead* d_heads = nullptr;
     const uint16_t* d_offs = nullptr;
 };
+
+// Places that the rows of blocks g0 .. g1 of a segment take: from id (with pre
+// words beyond hw per row before it), nrows of them with `words` beyond hw each.
+void band_window(const BandSegment& s, int g0, int g1, int64_t& id, int64_t& pre, int64_t& nrows, int64_t& words);
 
 }  // namespace aa
