@@ -34,7 +34,7 @@ aa_status fail(cudaError_t e, const char* what) {
 // branches the batch runs at 1.00x and 1.05x the speed of the same beams
 // issued one after another; the persistent work-queue form at 0.96x / 0.97x.
 constexpr int kDefaultBranches = 8;
-constexpr int64_t kBranchRowsMax = int64_t(256) << 20;
+constexpr int64_t kBranchRowsMax = int64_t(384) << 20;
 
 struct WaveTables {
     // host copies (uploaded into the arena)
@@ -131,7 +131,7 @@ cudaError_t issue_beam(const aa_batch* b, int bi, int branch, cudaStream_t s) {
     const Layout L = make_layout(pl, b->nsamps[bi], b->max_width);
     const uint8_t* d_in = reinterpret_cast<const uint8_t*>(b->arena + b->in_offset[bi]);
     cudaError_t e = launch_decimation_cascade(pl, L, d_in, b->in_pitch[bi], b->beam_dec_ws[bi], s);
-    const int64_t per = b->rows_bytes / std::max(b->branches, 1) / 256 * 256;
+    const int64_t per = b->rows_bytes / std::max(std::min(b->branches, b->nbeams), 1) / 256 * 256;  // beams are dealt to empty branches first
     for (DedispArgs a : b->beam_dd[bi]) {
         a.band_rows = reinterpret_cast<uint32_t*>(b->rows + branch * per);
         a.band_bytes = per;
@@ -322,7 +322,8 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
             if (uses_bands(plans[i]->ranges[r]))
                 rows = std::max(rows, band_bytes_busy(plans[i]->ranges[r].bands, L.length[r], plans[i]->ranges[r].desc.ndm));
     }
-    rows = std::min({rows, kBranchRowsMax, wave_bytes / kDefaultBranches / 256 * 256}) * kDefaultBranches;
+    const int64_t used = std::min(kDefaultBranches, nbeams);
+    rows = std::min({rows, kBranchRowsMax, wave_bytes / used / 256 * 256}) * used;
     const size_t least = (size_t)(in_bytes + wave_bytes + table_bytes + cand_bytes + chunk_bytes + small_bytes);
     b->arena_bytes = least + (size_t)rows;
     cudaError_t e = cudaMalloc(&b->arena, b->arena_bytes);
