@@ -7,7 +7,9 @@
 // into four 16-byte stores (eight threads 128 bytes of a channel).  Word w of
 // time sample t lies at w ^ 4 (t / 16 mod 8) of its row, so that neither side
 // meets a bank twice.  4096 channels x 2^20 samples: 1.48 ms, 5.8 TB/s (64 x 64 tiles
-// gathered byte by byte 2.28 ms).
+// gathered byte by byte 2.28 ms).  Rows that do not begin at 16 bytes are read by
+// words and shifted into place: 4095 channels x 2^18, 0.41 ms (by bytes, in the
+// small tiles, 1.34; 1000 x 300001: 0.13, 0.36).
 #include <cstdint>
 
 #include "aa_internal.h"
@@ -22,6 +24,7 @@ __global__ void __launch_bounds__(256) corner_turn_kernel(const uint8_t* __restr
                                                           uint8_t* __restrict__ cm, int64_t pitch,
                                                           int64_t ntile_c, int64_t ntiles) {
     __shared__ __align__(16) uint32_t tile[kTile][kTile / 4];  // [t][4 c]
+    const uint8_t* end = tm + (nsamp - 1) * stride + nchans;
     for (int64_t it = blockIdx.x; it < ntiles; it += gridDim.x) {
         const int64_t t0 = (it / ntile_c) * kTile;
         const int c0 = (int)(it % ntile_c) * kTile;
@@ -35,10 +38,18 @@ __global__ void __launch_bounds__(256) corner_turn_kernel(const uint8_t* __restr
                 const int64_t t = t0 + row + 32 * k;
                 const uint8_t* src = tm + t * stride + c;
                 v[k] = make_uint4(0, 0, 0, 0);
-                if (t < nsamp) {
-                    if (c + 16 <= nchans && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+                if (t < nsamp && c < nchans) {
+                    const uintptr_t at = reinterpret_cast<uintptr_t>(src);
+                    if ((at & 15) == 0 && src + 16 <= end) {  // (channels from nchans on are read, not stored)
                         v[k] = __ldcs(reinterpret_cast<const uint4*>(src));
-                    } else {
+                    } else if (src - (at & 3) >= tm && src - (at & 3) + 20 <= end) {
+                        const uint32_t* s4 = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
+                        const int sh = 8 * (int)(at & 3);
+                        const uint32_t w0 = __ldg(s4), w1 = __ldg(s4 + 1), w2 = __ldg(s4 + 2), w3 = __ldg(s4 + 3),
+                                       w4 = __ldg(s4 + 4);
+                        v[k] = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh),
+                                          __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
+                    } else {  // the block's first and last bytes
                         uint32_t w[4] = {0, 0, 0, 0};
                         for (int b = 0; b < 16 && c + b < nchans; ++b) w[b >> 2] |= (uint32_t)src[b] << (8 * (b & 3));
                         v[k] = make_uint4(w[0], w[1], w[2], w[3]);
