@@ -866,6 +866,61 @@ __global__ void __launch_bounds__(256) decimate_batch_kernel(const DecimateJob* 
     }
 }
 
+// Few blocks of the direct kernel leave most SMs idle and take its whole chain
+// of staged chunks one after another; there a CTA takes one trial x 128 samples
+// (4 a lane, words read at their places and shifted), its warps every eighth
+// channel, their sums added in shared memory.
+constexpr int kSmallWarps = 8;
+constexpr int kSmallTau = 128;
+template <int SPW>
+__global__ void __launch_bounds__(kSmallWarps * 32) dedisperse_small_kernel(DedispArgs a, int ntiles) {
+    __shared__ __align__(16) uint32_t part[kSmallWarps][kSmallTau];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = (int)(blockIdx.x / (unsigned)ntiles);
+    const int64_t t0 = (int64_t)(blockIdx.x % (unsigned)ntiles) * kSmallTau, t = t0 + 4 * lane;
+    const int32_t* shifts = a.shifts + (int64_t)d * a.nchans;
+    const int64_t words = a.in_pitch / SPW;  // of a row; reads past it, which no valid output needs, stay at its last
+    const uint32_t* in = static_cast<const uint32_t*>(a.in);
+    uint32_t tot[4] = {0, 0, 0, 0};
+    for (int c0 = warp; c0 < a.nchans; c0 += 256 * kSmallWarps) {  // 16-bit lanes hold 257 samples of 8 bits
+        const int c1 = min(a.nchans, c0 + 256 * kSmallWarps);
+        uint32_t even = 0, odd = 0;
+#pragma unroll 8
+        for (int c = c0; c < c1; c += kSmallWarps) {
+            const int64_t i = t + __ldg(shifts + c), w = i / SPW;
+            const uint32_t* row = in + c * words;
+            const uint32_t w0 = __ldg(row + min(w, words - 1)), w1 = __ldg(row + min(w + 1, words - 1));
+            if constexpr (SPW == 4) {
+                const uint32_t v = __funnelshift_r(w0, w1, 8 * (int)(i & 3));
+                even += v & 0x00ff00ffu;
+                odd += (v >> 8) & 0x00ff00ffu;
+            } else {
+                const uint32_t w2 = __ldg(row + min(w + 2, words - 1));
+                const uint32_t v0 = __funnelshift_r(w0, w1, 16 * (int)(i & 1)), v1 = __funnelshift_r(w1, w2, 16 * (int)(i & 1));
+                tot[0] += v0 & 0xffffu;
+                tot[1] += v0 >> 16;
+                tot[2] += v1 & 0xffffu;
+                tot[3] += v1 >> 16;
+            }
+        }
+        if constexpr (SPW == 4) {
+            tot[0] += even & 0xffffu;
+            tot[1] += odd & 0xffffu;
+            tot[2] += even >> 16;
+            tot[3] += odd >> 16;
+        }
+    }
+    *reinterpret_cast<uint4*>(&part[warp][4 * lane]) = make_uint4(tot[0], tot[1], tot[2], tot[3]);
+    __syncthreads();
+    if (threadIdx.x >= kSmallTau) return;
+    uint32_t v = 0;
+#pragma unroll
+    for (int w = 0; w < kSmallWarps; ++w) v += part[w][threadIdx.x];
+    const bool in_row = t0 + threadIdx.x < a.length;
+    if (in_row) a.out[(int64_t)d * a.out_pitch + t0 + threadIdx.x] = (float)v;
+    if (a.st_acc) add_row_sums(a.st_acc + 3 * (int64_t)d, in_row ? v : 0, in_row ? (unsigned long long)v * v : 0);
+}
+
 }  // namespace
 
 int g_fault_skip_chunk = -1;          // test hook: never issue this chunk
@@ -907,6 +962,19 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
         if (e != cudaSuccess) return e;
         kern<<<(unsigned)nblocks, kDedispThreads, a.smem, s>>>(a, ndmb);
+        return cudaGetLastError();
+    }
+    // Up to one wave of the small kernel's CTAs (155,648 samples on 152 SMs) it is
+    // the faster one: 20 trials x 6000 of 64 channels 9.8 us against 16.5 (16-bit
+    // input 11.6, 16.4), of 1024 channels 58 against 160; at 320,000 samples both
+    // take as long (16.5 and 16.4 us at 64 channels; 16-bit 19.2 and 16.2).
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 0;
+    const int64_t small = (a.length + kSmallTau - 1) / kSmallTau * a.ndm;
+    if (small <= 8 * (int64_t)sms && !a.out16 && g_fault_skip_chunk < 0) {
+        auto kern = a.elem == 1 ? dedisperse_small_kernel<4> : dedisperse_small_kernel<2>;
+        kern<<<(unsigned)small, kSmallWarps * 32, 0, s>>>(a, (int)(small / a.ndm));
         return cudaGetLastError();
     }
     auto kern = a.elem == 1 ? dedisperse_kernel<4> : dedisperse_kernel<2>;
