@@ -384,7 +384,7 @@ constexpr int NT = kSpsThreads;
 constexpr float kBig = 1.2676506002282294e30f;  // 2^100
 
 // The width search of one thread's M starts.  Widths come in chunks of M
-// (chunk c: widths M c + 1 .. M c + M); chunk 0 is evaluated by every thread.
+// (chunk c: widths M c + 1 .. M c + M); chunk 0 is bounded more finely.
 // Of the others a thread evaluates those that can still raise the B of one of
 // its starts, each thread at its own chunk: before a bright pulse the 32
 // threads of a warp need 32 different widths, each of them few.
@@ -480,6 +480,36 @@ __device__ __forceinline__ void eval_chunk(const float* __restrict__ pw, const f
     }
 }
 
+// Can a window of width 1 to 16 reach F (> 0)?  One bound for each of the widths
+// 1 | 2, 3 | 4-7 | 8-15 | 16: the largest end of its windows at each start.  In
+// noise hardly a warp has to evaluate chunk 0 then (2000 series of 48611 samples,
+// W = 64: 0.638 -> 0.554 ms; 2.3e9 starts with pulses, W = 8192: 34.8 -> 32.4).
+__device__ __forceinline__ bool chunk0_reaches(const float* __restrict__ pb, const float (&base)[M], float f, float r, float F) {
+    float win[2 * M];
+#pragma unroll
+    for (int k = 0; k < 2 * M; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(pb + k);
+        win[k] = v.x; win[k + 1] = v.y; win[k + 2] = v.z; win[k + 3] = v.w;
+    }
+    // largest rise from a start to win[start + w], the drift of its widths at least w0 or at most w1
+    auto reach = [&](int w, int w1, float rw) {
+        float top = -FLT_MAX;
+#pragma unroll
+        for (int i = 0; i < M; i += 2) top = max3f(top, win[i + w] - base[i], win[i + 1 + w] - base[i + 1]);
+        return fmaf(-f, (float)(f >= 0.0f ? w : w1), top) * (r * rw) >= F;
+    };
+    bool any = reach(1, 1, 1.0f) | reach(16, 16, 0.25f);
+#pragma unroll
+    for (int k = 2; k + 1 < 2 * M; ++k) win[k] = fmaxf(win[k], win[k + 1]);
+    any |= reach(2, 3, 0.70710678f);
+#pragma unroll
+    for (int k = 4; k + 3 < 2 * M; ++k) win[k] = fmaxf(win[k], win[k + 2]);
+    any |= reach(4, 7, 0.5f);
+#pragma unroll
+    for (int k = 8; k < M + 8; ++k) win[k] = fmaxf(win[k], win[k + 4]);
+    return any | reach(8, 15, 0.35355339f);
+}
+
 // Without a threshold up to kEvery chunks are simply evaluated in turn: noise
 // leaves over a third of them to evaluate and the bounds cost more (B(t) of
 // 96 series of 64006 samples, W = 256 / 1024 / 2048: in turn 220 / 752 / 1449
@@ -519,6 +549,7 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
     }
     const float *s1 = Q + nq + t, *s8 = s1 + nq, *s64 = s8 + nq;
     float F = cut - bnd.S;              // the floor less the bounds' margin
+    const bool first0 = LOW || chunk0_reaches(P + M * t, base, bnd.f, bnd.rs[0], F);
     int evaluated = 0;
     unsigned fill = 0;                  // entries in the queue << 16 | the first one's place (mod kQueue)
     unsigned cur = 0;                   // the taken entry: chunk of its first bit << 5 | bits
@@ -533,7 +564,7 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
     unsigned keep = ~0u;  // bits that the level above lets through
     for (;;) {
         if (step == kEval) {
-            int pend = pass < 0 ? 0 : -1;  // chunk to evaluate: first chunk 0, then the queue's
+            int pend = pass < 0 && first0 ? 0 : -1;  // chunk to evaluate: first chunk 0, then the queue's
             while (pend < 0 && ((cur & 0xffu) || fill >> 16)) {
                 if (!(cur & 0xffu)) {
                     cur = queue[(fill % kQueue) * NT];
@@ -724,13 +755,13 @@ __host__ __device__ constexpr int sps_lists_words(int wpad) {
 // With 16 warps an SM (128 registers: a thread's starts, their B, the window of
 // a chunk) the tile's chain of short phases is what takes the time, so the
 // phases are kept few and their barriers fewer.  4096 channels x 2^20 samples,
-// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 34.8 ms; of 40.5 before the
+// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 32.4 ms; of 40.5 before the
 // search's queues (clock64) the width search 14.6, waiting for a tile's slowest warp 8.0, block maxima 4.4,
 // sums of new samples 2.8, candidates' widths 2.1, fresh tiles 1.5, peaks 1.4,
 // sliding 1.4.  Steps on the way: a warp's union of 128-width segments 92, the
 // chunks of each thread by lower bounds 66, their bounds eight at a time in one
 // loop 57, the new samples by cp.async, 32-bit sums, peaks from registers and
-// widths by half-warps 45, chunk numbers packed 40.5, queues 34.8.
+// widths by half-warps 45, chunk numbers packed 40.5, queues 34.8, chunk 0 by bounds 32.4.
 template <bool LOW>
 __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t tile_lo, int64_t tile_hi,
                                              float* sm) {
