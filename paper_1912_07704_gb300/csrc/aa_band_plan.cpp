@@ -259,6 +259,7 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
     // overlaps is consumed (pairs are consumed in order)
     bp.ring_words = (int)(kSumSmem / 4);
     bp.smem_sum = kSumSmem;
+    bp.by_two_pairs = 4 * k * 255 * dec <= 65535;
     for (int g = 0; g < nblk_all; ++g) {
         BandHead* h = &bp.heads[(size_t)g * npad];
         std::vector<std::pair<int, int>> place;
@@ -271,6 +272,7 @@ bool build(const RangePlan& r, int C, int k, BandPlan& bp) {
             for (int q = after + 1; q < pr; ++q)
                 if (place[q].first < pos + w && pos < place[q].second) after = q;
             if (after >= 0 && after + kBandLag > pr) return false;
+            if (after >= 0 && after + kBandLag > (pr & ~1)) bp.by_two_pairs = false;
             place.push_back({pos, pos + w});
             for (int u = 0; u < 2; ++u) {
                 h[2 * pr + u].place = (uint32_t)pos;

@@ -11,12 +11,13 @@
 //                     16 warps of 4 trials add one row per band and trial, 8
 //                     words a lane.
 //
-// What bounds them (4096 channels, 1500 trials, 2^20 samples: 47 ms of sums and
-// 20 ms of rows; the grouped kernel takes 180):
+// What bounds them (4096 channels, 1500 trials, 2^20 samples: 51.5 ms of sums and
+// 10.3 ms of rows; the grouped kernel takes 180):
 //   sums  shared memory: 64 trials x 8 word reads a lane and band are 512
-//         wavefronts, the ring's fill 74 more; 712 cycles a band measured.  Two
-//         bands are added per round (half the adds and barriers; 308 -> 234
-//         warp instructions a pair), their sum's two 16-bit lanes go straight
+//         wavefronts, the ring's fill 74 more.  Two
+//         pairs of bands are added per round where their rows fit 16 bits (one
+//         band 308 warp instructions a pair, one pair 234 and 712 cycles a band,
+//         57 ms; two pairs 645, 51.5), their sum's two 16-bit lanes go straight
 //         into 32-bit totals by dot products (2.36 ms a slab with 16-bit
 //         accumulators flushed every 32 bands, 1.96 without: the registers they
 //         took held loads back), and a place of the ring is refilled three
@@ -260,6 +261,8 @@ constexpr int kSumThreads = kSumWarps * 32;
 constexpr int kTrialsPerWarp = kBandTrials / kSumWarps;
 constexpr int kQ = kBandWords / 32;  // words per lane and trial
 
+// G: pairs added in a round (2: their four rows in 16 bits before the totals)
+template <int G>
 __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
     extern __shared__ __align__(128) uint32_t ring[];
     __shared__ uint64_t full[kBandBars], empty[kBandBars];  // pair p: p % kBandBars
@@ -306,9 +309,14 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
         tot[i][2 * q] = __dp2a_lo(w, 0x00000001u, tot[i][2 * q]);
         tot[i][2 * q + 1] = __dp2a_lo(w, 0x00000100u, tot[i][2 * q + 1]);
     };
-    int place = 0;
+    int place[G];
+    auto places = [&](int pr) {  // of pairs pr .. pr + G - 1, known to every warp from the heads (read a round ahead)
+#pragma unroll
+        for (int u = 0; u < G; ++u) place[u] = pr + u < npairs ? (int)__ldg(&heads[2 * (pr + u)].place) : 0;
+    };
+    places(0);
     bool ok = true;
-    for (int pr = 0; pr < npairs; ++pr) {
+    for (int pr = 0; pr < npairs; pr += G) {
         while ((int)h.w >> 16 <= pr) {  // at
             const int after = (int16_t)(h.w & 0xffffu);
             if (after >= 0 && !__all_sync(0xffffffffu, mbar_wait(&empty[after % kBandBars], (uint32_t)(after / kBandBars) & 1u, &gave_up))) {
@@ -327,29 +335,54 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
             fetch();
         }
         if (!ok) break;
-        // this pair's place, known to every warp from the heads (read one pair ahead)
-        const uint32_t* sp = ring + place;
-        place = pr + 1 < npairs ? (int)__ldg(&heads[2 * pr + 2].place) : 0;
-        ok = __all_sync(0xffffffffu, mbar_wait(&full[pr % kBandBars], (uint32_t)(pr / kBandBars) & 1u, &gave_up));
+        const uint32_t* sp[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) sp[u] = ring + place[u];
+        places(pr + G);
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+            if (pr + u < npairs)
+                ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[(pr + u) % kBandBars], (uint32_t)((pr + u) / kBandBars) & 1u, &gave_up));
         if (!ok) break;
-        const uint2 o = *reinterpret_cast<const uint2*>(sp + 2 * warp);
-        const uint32_t* z = sp + kBandTrials + lane;
-        const uint32_t* p[kTrialsPerWarp] = {z + (o.x & 0xffffu), z + (o.x >> 16), z + (o.y & 0xffffu), z + (o.y >> 16)};
-        if (2 * pr + 1 < a.nbands) {
-            const uint2 v = *reinterpret_cast<const uint2*>(sp + kBandTrials / 2 + 2 * warp);
-            const uint32_t* p2[kTrialsPerWarp] = {z + (v.x & 0xffffu), z + (v.x >> 16), z + (v.y & 0xffffu), z + (v.y >> 16)};
+        // this warp's trials' words of the first and the second band of a pair
+        auto first = [&](int u) { return *reinterpret_cast<const uint2*>(sp[u] + 2 * warp); };
+        auto second = [&](int u) { return *reinterpret_cast<const uint2*>(sp[u] + kBandTrials / 2 + 2 * warp); };
+        auto word = [](uint2 o, int i) { return i == 0 ? o.x & 0xffffu : i == 1 ? o.x >> 16 : i == 2 ? o.y & 0xffffu : o.y >> 16; };
+        if (G == 2 && 2 * pr + 3 < a.nbands) {
+            const uint2 o0 = first(0), o1 = second(0), o2 = first(G - 1), o3 = second(G - 1);
+            const uint32_t *z0 = sp[0] + kBandTrials + lane, *z1 = sp[G - 1] + kBandTrials + lane;
 #pragma unroll
-            for (int i = 0; i < kTrialsPerWarp; ++i)
+            for (int i = 0; i < kTrialsPerWarp; ++i) {
+                const uint32_t *p0 = z0 + word(o0, i), *p1 = z0 + word(o1, i), *p2 = z1 + word(o2, i), *p3 = z1 + word(o3, i);
 #pragma unroll
-                for (int q = 0; q < kQ; ++q) add(i, q, p[i][32 * q] + p2[i][32 * q]);
+                for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q] + p1[32 * q] + (p2[32 * q] + p3[32 * q]));
+            }
         } else {
 #pragma unroll
-            for (int i = 0; i < kTrialsPerWarp; ++i)
+            for (int u = 0; u < G; ++u) {
+                if (pr + u >= npairs) continue;
+                const uint32_t* z = sp[u] + kBandTrials + lane;
+                const uint2 o = first(u);
+                if (2 * (pr + u) + 1 < a.nbands) {
+                    const uint2 v = second(u);
 #pragma unroll
-                for (int q = 0; q < kQ; ++q) add(i, q, p[i][32 * q]);
+                    for (int i = 0; i < kTrialsPerWarp; ++i) {
+                        const uint32_t *p0 = z + word(o, i), *p1 = z + word(v, i);
+#pragma unroll
+                        for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q] + p1[32 * q]);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kTrialsPerWarp; ++i) {
+                        const uint32_t* p0 = z + word(o, i);
+#pragma unroll
+                        for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q]);
+                    }
+                }
+            }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[pr % kBandBars]);
+        if (lane < G && pr + lane < npairs) mbar_arrive(&empty[(pr + lane) % kBandBars]);
     }
     if (!ok && lane == 0) {
         gave_up = 1;
@@ -412,7 +445,8 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
     auto rows_kern = a.row_dec > 1 ? band_rows_kernel<0> : a.elem == 1 ? band_rows_kernel<1> : band_rows_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(rows_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_rows);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(band_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_sum);
+    auto sum_kern = bp.by_two_pairs ? band_sum_kernel<2> : band_sum_kernel<1>;
+    e = cudaFuncSetAttribute(sum_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_sum);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -481,7 +515,7 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
             sa.pitch = a.out_pitch;
             sa.st_acc = a.st_acc ? a.st_acc + 3 * (int64_t)(d0 - a.trial0) : nullptr;
             sa.err = a.err;
-            band_sum_kernel<<<(unsigned)(nt * nblk), kSumThreads, bp.smem_sum, s>>>(sa);
+            sum_kern<<<(unsigned)(nt * nblk), kSumThreads, bp.smem_sum, s>>>(sa);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }

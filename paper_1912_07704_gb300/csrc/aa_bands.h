@@ -81,6 +81,7 @@ struct BandPlan {
     bool ok = false;
     int k = 0, nbands = 0;
     int ring_words = 0;  // ring of the summing kernel
+    bool by_two_pairs = false;  // two pairs' rows fit 16 bits, and their places fill in time to be added together
     int tile = 0;                    // words per CTA of the row kernel
     int raw_words = 0, quad_words = 0, max_quads = 0, max_rows = 0;
     size_t smem_rows = 0, smem_sum = 0;
