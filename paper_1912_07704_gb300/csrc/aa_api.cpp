@@ -588,11 +588,13 @@ aa_status aa_dedisperse(aa_plan* p, const uint8_t* host_in, int64_t nsamp, int64
     res->device = p->device;
     float* d_out = static_cast<float*>(mem.get((size_t)L.dd_elems * 4 + kErrBlock));
     uint8_t* d_in = static_cast<uint8_t*>(mem.get((size_t)p->nchans * L.in_pitch_min));
-    void* d_ws = mem.get((size_t)L.dedisp_ws);
+    size_t ws_bytes = (size_t)L.dedisp_ws;  // with the band rows' buffer where there is memory for it
+    void* d_ws = mem.get(ws_bytes);
+    if (!d_ws && L.dedisp_base < L.dedisp_ws) d_ws = mem.get(ws_bytes = (size_t)L.dedisp_base);
     if (!d_out || !d_in || !d_ws) {
         delete res;
         set_error("device allocation of %lld bytes failed",
-                  (long long)(L.dd_elems * 4 + p->nchans * L.in_pitch_min + L.dedisp_ws));
+                  (long long)(L.dd_elems * 4 + p->nchans * L.in_pitch_min + L.dedisp_base));
         return AA_ERR_NOMEM;
     }
     if (nsamp > 0) {
@@ -613,7 +615,7 @@ aa_status aa_dedisperse(aa_plan* p, const uint8_t* host_in, int64_t nsamp, int64
         }
         if (e != cudaSuccess) { delete res; return cuda_fail(e, "host-to-device copy"); }
     }
-    st = aa_dedisperse_device(p, d_in, nsamp, L.in_pitch_min, d_out, d_ws, (size_t)L.dedisp_ws, stream);
+    st = aa_dedisperse_device(p, d_in, nsamp, L.in_pitch_min, d_out, d_ws, ws_bytes, stream);
     if (st != AA_OK) { delete res; return st; }
     unsigned* d_err = reinterpret_cast<unsigned*>(d_out + L.dd_elems);
     cudaError_t e = nsamp > 0 ? cudaMemcpyAsync(d_err, d_ws, sizeof(unsigned), cudaMemcpyDeviceToDevice, s)

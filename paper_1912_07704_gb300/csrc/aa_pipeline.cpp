@@ -62,6 +62,7 @@ struct aa_pipeline {
     std::vector<Slot> slots;
     float* d_dd = nullptr;
     void* d_ws_dd = nullptr;
+    size_t ws_dd_bytes = 0;
     void* d_ws_sps = nullptr;
     aa_candidate* d_cands = nullptr;
     unsigned long long* d_count = nullptr;
@@ -153,11 +154,18 @@ aa_status aa_pipeline_create(aa_plan* p, int64_t nsamp, int32_t max_width, float
         if ((e = cudaEventCreateWithFlags(&sl.searched, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
     }
     if ((e = cudaMalloc(&pl->d_dd, (size_t)std::max<int64_t>(L.dd_elems, 1) * 4)) != cudaSuccess) return bail(e, "dedispersed series");
-    if ((e = cudaMalloc(&pl->d_ws_dd, (size_t)L.dedisp_ws)) != cudaSuccess) return bail(e, "dedispersion workspace");
     if ((e = cudaMalloc(&pl->d_ws_sps, (size_t)L.sps_ws)) != cudaSuccess) return bail(e, "search workspace");
     if ((e = cudaMalloc(&pl->d_cands, (size_t)cand_capacity * rec)) != cudaSuccess) return bail(e, "candidates");
     if ((e = cudaMalloc(&pl->d_count, 256)) != cudaSuccess) return bail(e, "count");
     if ((e = cudaMalloc(&pl->d_tmp, tmp)) != cudaSuccess) return bail(e, "ordering scratch");
+    // last, with the band rows' buffer where there is memory for it
+    pl->ws_dd_bytes = (size_t)L.dedisp_ws;
+    if ((e = cudaMalloc(&pl->d_ws_dd, pl->ws_dd_bytes)) != cudaSuccess && L.dedisp_base < L.dedisp_ws) {
+        cudaGetLastError();
+        pl->ws_dd_bytes = (size_t)L.dedisp_base;
+        e = cudaMalloc(&pl->d_ws_dd, pl->ws_dd_bytes);
+    }
+    if (e != cudaSuccess) return bail(e, "dedispersion workspace");
     *out = pl;
     return AA_OK;
 }
@@ -192,7 +200,7 @@ aa_status aa_pipeline_submit(aa_pipeline* pl, const uint8_t* host_in, int64_t ho
     AA_CUDA(cudaStreamWaitEvent(pl->compute, sl.uploaded, 0), "wait upload");
     const aa_stream_t cs = reinterpret_cast<aa_stream_t>(pl->compute);
     aa_status st = aa_dedisperse_device(p, sl.d_in, pl->nsamp, L.in_pitch_min, pl->d_dd, pl->d_ws_dd,
-                                        (size_t)L.dedisp_ws, cs);
+                                        pl->ws_dd_bytes, cs);
     if (st != AA_OK) return st;
     st = aa_sps_search_device(p, pl->nsamp, pl->d_dd, pl->max_width, pl->threshold, pl->d_cands, pl->cap,
                               pl->d_count, nullptr, pl->d_ws_sps, (size_t)L.sps_ws, cs);
