@@ -12,11 +12,13 @@
 // there; only the top depth's rows go to memory.  With one launch per depth every
 // sum read two samples and wrote one: 75 GB and 15.2 ms for 2^17 samples of 4096
 // channels under the four ranges of the SKA plan; in groups of 4-3-5 depths it
-// is 10 GB and 5.9 ms.  Shared memory bounds it (its pipe is 61-68 % busy; two
-// CTAs of an SM hide the loads of each other).  A lane sums four consecutive
+// is 10 GB and 5.5 ms (5.9 with one tile a CTA, its tables read again for each).
+// Shared memory bounds it (its pipe is 61-68 % busy; two CTAs of an SM hide the
+// loads of each other).  A lane sums four consecutive
 // samples: with one sample a lane (12 wavefronts for 128 sums instead of 16, but
 // twice the instructions) it was 7.0 ms; blocks of 52 and 71 KB, four and three to
 // an SM, 8.2 and 6.9 ms (more of their windows is overlap).
+#include <algorithm>
 #include <cstdint>
 
 #include "aa_internal.h"
@@ -40,7 +42,9 @@ struct FdmtArgs {
     float* fout;
     int64_t fpitch, flen;
     int32_t nblocks, tile, levels;
-    int32_t op_words;  // words before the slots
+    int32_t op_words, load_words;  // words of the ops, and of the loads behind them, before the slots
+    int32_t per;       // consecutive tiles of a CTA
+    int64_t ntiles;
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t* dst, const uint32_t* src, int bytes) {
@@ -76,73 +80,81 @@ __device__ __forceinline__ void merge(const uint32_t* slots, const int4& op, int
 template <int EB, bool FINAL>
 __global__ void __launch_bounds__(kFdmtThreads, 2) fdmt_group_kernel(FdmtArgs a) {
     extern __shared__ __align__(16) uint32_t fdmt_smem[];
-    FdmtOp* ops = reinterpret_cast<FdmtOp*>(fdmt_smem);
-    uint32_t* slots = fdmt_smem + a.op_words;
+    const int4* ops = reinterpret_cast<const int4*>(fdmt_smem);                  // src, dst, n, delta
+    const int4* loads = reinterpret_cast<const int4*>(fdmt_smem + a.op_words);  // ref, lo, dst, n
+    uint32_t* slots = fdmt_smem + a.op_words + a.load_words;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const FdmtBlock& b = a.blocks[blockIdx.x % a.nblocks];  // neighbouring blocks share rows: side by side
-    const int64_t t0 = (int64_t)(blockIdx.x / a.nblocks) * a.tile;
     const int load0 = __ldg(&b.load0), nload = __ldg(&b.nload), op0 = __ldg(&b.op0), nops = __ldg(&b.end[a.levels - 1]);
-    for (int i = warp; i < nload; i += kFdmtWarps) {
-        const int4 l = __ldg(reinterpret_cast<const int4*>(a.loads + load0 + i));  // ref, lo, dst, n
-        const int64_t t = t0 + l.y;
-        uint32_t* dst = slots + l.z;
-        if (l.x >= 0) {
-            const uint32_t* src = a.prev + (int64_t)l.x * a.pitch;
-            for (int j = 4 * lane; j < l.w; j += 128) {
-                const bool in = t + j < a.pitch;  // beyond the row: zeros, which no valid output reads
-                cp_async16(dst + j, in ? src + t + j : a.prev, in ? 16 : 0);
-            }
-        } else {
-            const int64_t row = (int64_t)(-(l.x + 1)) * a.leaf_pitch;
-#pragma unroll 4
-            for (int j = 4 * lane; j < l.w; j += 128) {
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (t + j < a.nsamp) {  // the pitch is a multiple of four samples
-                    if constexpr (EB == 1) {
-                        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.leaves) + row + t + j));
-                        v = make_uint4(w & 0xff, (w >> 8) & 0xff, (w >> 16) & 0xff, w >> 24);
-                    } else {
-                        const uint2 w = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(a.leaves) + row + t + j));
-                        v = make_uint4(w.x & 0xffff, w.x >> 16, w.y & 0xffff, w.y >> 16);
-                    }
-                }
-                *reinterpret_cast<uint4*>(dst + j) = v;
-            }
-        }
+    for (int i = threadIdx.x; i < nops + nload; i += kFdmtThreads) {
+        if (i < nops) reinterpret_cast<int4*>(fdmt_smem)[i] = __ldg(reinterpret_cast<const int4*>(a.ops + op0) + i);
+        else reinterpret_cast<int4*>(fdmt_smem + a.op_words)[i - nops] = __ldg(reinterpret_cast<const int4*>(a.loads + load0) + i - nops);
     }
-    for (int i = threadIdx.x; i < nops; i += kFdmtThreads)
-        reinterpret_cast<int4*>(ops)[i] = __ldg(reinterpret_cast<const int4*>(a.ops + op0) + i);
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    int begin = 0;
+    const int64_t tile0 = (int64_t)(blockIdx.x / a.nblocks) * a.per, tile1 = min(a.ntiles, tile0 + a.per);
 #pragma unroll 1
-    for (int lev = 0; lev < a.levels - 1; ++lev) {
-        const int end = __ldg(&b.end[lev]);
-        for (int o = begin + warp; o < end; o += kFdmtWarps) {
-            const int4 op = reinterpret_cast<const int4*>(ops)[o];
-            uint32_t* d = slots + op.y;
-            merge(slots, op, lane, [&](int i, uint4 v) { *reinterpret_cast<uint4*>(d + i) = v; });
-        }
-        begin = end;
-        __syncthreads();
-    }
-    for (int o = begin + warp; o < nops; o += kFdmtWarps) {
-        const int4 op = reinterpret_cast<const int4*>(ops)[o];
-        const int64_t left = (FINAL ? a.flen : a.nsamp - op.w) - t0;
-        const int n = left < op.z ? (int)left : op.z;  // op.z: the tile
-        merge(slots, op, lane, [&](int i, uint4 v) {
-            if constexpr (FINAL) {
-                float* row = a.fout + (int64_t)op.y * a.fpitch + t0 + i;
-                if (i + 4 <= n) *reinterpret_cast<float4*>(row) = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
-                else {
-                    if (i < n) row[0] = (float)v.x;
-                    if (i + 1 < n) row[1] = (float)v.y;
-                    if (i + 2 < n) row[2] = (float)v.z;
+    for (int64_t tile = tile0; tile < tile1; ++tile) {
+        const int64_t t0 = tile * a.tile;
+        __syncthreads();  // tables in place; the tile before is done with the slots
+        for (int i = warp; i < nload; i += kFdmtWarps) {
+            const int4 l = loads[i];
+            const int64_t t = t0 + l.y;
+            uint32_t* dst = slots + l.z;
+            if (l.x >= 0) {
+                const uint32_t* src = a.prev + (int64_t)l.x * a.pitch;
+                for (int j = 4 * lane; j < l.w; j += 128) {
+                    const bool in = t + j < a.pitch;  // beyond the row: zeros, which no valid output reads
+                    cp_async16(dst + j, in ? src + t + j : a.prev, in ? 16 : 0);
                 }
-            } else if (i < n) {  // the pitch is a multiple of four samples; beyond a row's valid part nothing is read
-                *reinterpret_cast<uint4*>(a.out + (int64_t)op.y * a.pitch + t0 + i) = v;
+            } else {
+                const int64_t row = (int64_t)(-(l.x + 1)) * a.leaf_pitch;
+#pragma unroll 4
+                for (int j = 4 * lane; j < l.w; j += 128) {
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (t + j < a.nsamp) {  // the pitch is a multiple of four samples
+                        if constexpr (EB == 1) {
+                            const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.leaves) + row + t + j));
+                            v = make_uint4(w & 0xff, (w >> 8) & 0xff, (w >> 16) & 0xff, w >> 24);
+                        } else {
+                            const uint2 w = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(a.leaves) + row + t + j));
+                            v = make_uint4(w.x & 0xffff, w.x >> 16, w.y & 0xffff, w.y >> 16);
+                        }
+                    }
+                    *reinterpret_cast<uint4*>(dst + j) = v;
+                }
             }
-        });
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        int begin = 0;
+#pragma unroll 1
+        for (int lev = 0; lev < a.levels - 1; ++lev) {
+            const int end = __ldg(&b.end[lev]);
+            for (int o = begin + warp; o < end; o += kFdmtWarps) {
+                const int4 op = ops[o];
+                uint32_t* d = slots + op.y;
+                merge(slots, op, lane, [&](int i, uint4 v) { *reinterpret_cast<uint4*>(d + i) = v; });
+            }
+            begin = end;
+            __syncthreads();
+        }
+        for (int o = begin + warp; o < nops; o += kFdmtWarps) {
+            const int4 op = ops[o];
+            const int64_t left = (FINAL ? a.flen : a.nsamp - op.w) - t0;
+            const int n = left < op.z ? (int)left : op.z;  // op.z: the tile
+            merge(slots, op, lane, [&](int i, uint4 v) {
+                if constexpr (FINAL) {
+                    float* row = a.fout + (int64_t)op.y * a.fpitch + t0 + i;
+                    if (i + 4 <= n) *reinterpret_cast<float4*>(row) = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
+                    else {
+                        if (i < n) row[0] = (float)v.x;
+                        if (i + 1 < n) row[1] = (float)v.y;
+                        if (i + 2 < n) row[2] = (float)v.z;
+                    }
+                } else if (i < n) {  // the pitch is a multiple of four samples; beyond a row's valid part nothing is read
+                    *reinterpret_cast<uint4*>(a.out + (int64_t)op.y * a.pitch + t0 + i) = v;
+                }
+            });
+        }
     }
 }
 
@@ -154,7 +166,14 @@ cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_e
     const bool fin = fout != nullptr;
     const int64_t n = fin ? flen : nsamp;
     if (n <= 0 || g.nblocks <= 0) return cudaSuccess;
-    const int64_t grid = (n + g.tile - 1) / g.tile * g.nblocks;
+    const int64_t ntiles = (n + g.tile - 1) / g.tile;
+    // Up to eight tiles a CTA, which then reads its block's tables once, while
+    // eight CTAs are left for each of the SMs' places.
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 1;
+    const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, ntiles * g.nblocks / (sms * 2 * 8)));
+    const int64_t grid = (ntiles + per - 1) / per * g.nblocks;
     if (grid >= (1ll << 31)) return cudaErrorInvalidConfiguration;
     FdmtArgs a{};
     a.blocks = fd.d_blocks + g.block0;
@@ -173,7 +192,10 @@ cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_e
     a.tile = g.tile;
     a.levels = g.bottom - g.top + 1;
     a.op_words = g.max_ops * 4;
-    const size_t smem = ((size_t)a.op_words + (size_t)g.words) * 4;
+    a.load_words = g.max_loads * 4;
+    a.per = (int32_t)per;
+    a.ntiles = ntiles;
+    const size_t smem = ((size_t)a.op_words + (size_t)a.load_words + (size_t)g.words) * 4;
     auto kern = leaf_elem == 1 ? (fin ? fdmt_group_kernel<1, true> : fdmt_group_kernel<1, false>)
                                : (fin ? fdmt_group_kernel<2, true> : fdmt_group_kernel<2, false>);
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -13,8 +13,6 @@
 namespace aa {
 namespace {
 
-constexpr int kMaxLoads = 1 << 12;
-
 // One block before its tile is chosen: slots instead of word offsets.
 struct Need {
     int32_t row;     // row of its depth, or reference of a load
@@ -167,7 +165,7 @@ bool build_fdmt_groups(FdmtPlan& fd, int32_t nchans, int elem, const std::vector
             bl.forget(top, bottom, b);
             const int W = width_of(b.slots, b.spread);
             const int tile = W ? tile_of(W, b.spread) : 0;
-            if (!W || (int)b.loads.size() > kMaxLoads) return std::numeric_limits<double>::infinity();
+            if (!W) return std::numeric_limits<double>::infinity();
             double bytes = 0;
             for (const Need& l : b.loads) bytes += (l.row < 0 ? elem : 4) * (double)W;
             bytes += 4.0 * tile * (c[j + 1] - c[j]);
@@ -244,6 +242,7 @@ bool build_fdmt_groups(FdmtPlan& fd, int32_t nchans, int elem, const std::vector
             }
             bl.forget(top, bottom, b);
             g.max_ops = std::max(g.max_ops, o.end[k - 1]);
+            g.max_loads = std::max(g.max_loads, o.nload);
             fd.blocks.push_back(o);
         }
         g.nblocks = (int32_t)((int64_t)fd.blocks.size() - g.block0);
@@ -306,7 +305,7 @@ bool fdmt_shifts(const FdmtPlan& fd, int32_t nchans, int32_t ndm, int32_t* out) 
                     }
                 for (Slot& r : made) slot[(size_t)(r.base / g.width)] = std::move(r);
             }
-            if (b.end[g.bottom - g.top] > g.max_ops) return false;
+            if (b.end[g.bottom - g.top] > g.max_ops || b.nload > g.max_loads) return false;
         }
         for (const auto& t : of[q])
             if (t.empty()) return false;

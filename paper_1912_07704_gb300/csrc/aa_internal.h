@@ -116,7 +116,7 @@ static_assert(sizeof(FdmtRow) == 16, "FDMT row layout");
 // top depth, the windows they read loaded into slots of shared memory, the
 // depths between merged there.  Offsets are in 32-bit words of the slots.
 constexpr int kFdmtMaxLevels = 5;
-constexpr int kFdmtSlotWords = 108 * 1024 / 4;  // most words of the slots
+constexpr int kFdmtSlotWords = 106 * 1024 / 4;  // most words of the slots
 struct FdmtLoad {
     int32_t ref;  // row of the next-deeper stored depth, or channel -(ref + 1)
     int32_t lo;   // first sample, relative to the tile (multiple of 4)
@@ -137,7 +137,7 @@ struct FdmtGroup {
     int top = 0, bottom = 0;  // depths merged
     int tile = 0;             // samples of a block
     int32_t width = 0, words = 0;  // words of a slot, of all slots
-    int32_t max_ops = 0;
+    int32_t max_ops = 0, max_loads = 0;  // of a block
     int64_t block0 = 0;
     int32_t nblocks = 0;
 };
