@@ -151,11 +151,12 @@ def build_input(plan, w, device):
 # when the kernel changes until it is captured again.
 NCU_TRAFFIC = {
     ("dedisperse_u8", "grouped"): {
-        "small_read_bytes": 542_687_232, "small_write_bytes": 740_074_496,
+        # band rows: every launch of the row and summing kernels of the range
+        "small_read_bytes": 5_973_090_000, "small_write_bytes": 5_213_680_000,
         "small_output_samples": 1500 * 128687,
-        "capture": "profiles/dedisperse_grouped_u8_ska-4096ch-2^17.md"},
+        "capture": "profiles/dedisperse_bands_u8_ska-4096ch-2^17.md"},
     ("sps_boxcar", "pruned"): {
-        "small_read_bytes": 947_282_688, "small_write_bytes": 42_682_624,
+        "small_read_bytes": 877_592_576, "small_write_bytes": 49_681_408,
         "small_output_samples": 1500 * 128687,
         "capture": "profiles/sps_boxcar_ska-4096ch-2^17.md"},
 }
@@ -472,15 +473,13 @@ def bench_ours(args):
         return per_launch, f"ncu capture {ent['capture']}, scaled x{scale:.2f} by output samples"
 
     if dominant == "dedisperse_fdmt":
-        # HBM-bound gather-adds: every row of every tree depth reads two rows
-        # and writes one (32-bit; leaves are 8/16-bit input rows, counted as 4
-        # bytes: an upper estimate); rows = fdmt_work x ndm x nchans per range
+        # what the tree cannot do without: the (decimated) input once, the
+        # trials' rows once.  Groups of depths are merged in shared memory,
+        # whose pipe bounds them.
         fd_s = kern[dominant]["ms_per_step"] / 1e3
-        nbytes = 0.0
-        for r, g in enumerate(alg["lay"]):
-            info = abi.aa_plan_range(plan.handle, nsamp, r)
-            if info.strategy == 3:
-                nbytes += info.fdmt_work * g.ndm * w.nchans * g.nsamp_dec * 12
+        nbytes = float(sum(w.nchans * g.nsamp_dec * (1 if g.dec == 1 else 2) + 4 * g.ndm * g.length
+                           for r, g in enumerate(alg["lay"])
+                           if abi.aa_plan_range(plan.handle, nsamp, r).strategy == 3))
         nl = kern[dominant]["launches"] / max(args.steps, 1)
         achieved = nbytes / fd_s
         hbm_peak = float(peaks.get("hbm_gbs", 6678.2)) * 1e9
@@ -488,8 +487,8 @@ def bench_ours(args):
                 "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": None,
                 "traffic_source": "no capture of the tree kernels",
                 "algorithmic_bytes_per_launch": nbytes / max(nl, 1),
-                "ops": "per tree row: two rows read and one written, 4 bytes a sample "
-                       "(rows = fdmt_work x ndm x nchans); peak = measured HBM copy bandwidth"}
+                "ops": "input read once and the trials' rows written once; peak = measured HBM "
+                       "copy bandwidth (the kernels are bound by shared memory)"}
     elif dominant == "sps_boxcar":
         achieved = BOXCAR_OPS_PER_WS * evaluated / box_s
         tb, tnote = traffic("sps_boxcar")
@@ -514,7 +513,7 @@ def bench_ours(args):
                 "executed_gops": executed / 1e9, "executed_frac": executed / lane_peak,
                 "ops": "algorithmic channel-adds (sum over trials of nchans x L) per second; "
                        "executed_* counts the adds the chosen strategy performs (grouped: "
-                       "pre-sum adds + group adds); peak = 1 add per lane per clock "
+                       "those of the group sums, an upper bound where band rows run); peak = 1 add per lane per clock "
                        f"({sm_count} SMs (device query) x 128 lanes x {sm_max:.0f} MHz)"}
     hbm = float(peaks.get("hbm_gbs", 6678.2))
     eff_in_gbs = alg["dm_samples"] * w.nchans / step_s / 1e9
