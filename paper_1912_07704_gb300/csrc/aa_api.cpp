@@ -324,7 +324,7 @@ static aa_status launch_fdmt(const aa_plan* p, size_t r, const Layout& L, const 
     return AA_OK;
 }
 
-// Sub-band strategy of range r: stage 1 per band into the 16-bit partial
+// Sub-band strategy of range r: stage 1 of all bands into the 16-bit partial
 // series (direct kernel), stage 2 over all coarse trials into the range's
 // output rows (32-bit sums).
 static aa_status launch_subband(const aa_plan* p, size_t r, const Layout& L, const void* in, int64_t in_pitch,
@@ -349,25 +349,20 @@ static aa_status launch_subband(const aa_plan* p, size_t r, const Layout& L, con
     const int64_t pitch1 = L.sub_pitch[r];
     uint16_t* z = reinterpret_cast<uint16_t*>(ws + L.sub_offset[r]);
     {
-        size_t off = 0;
-        for (int b = 0; b < sb.nsub; ++b) {
-            ProfScope prof(kKSubband1, s);  // one record per launch
-            const int c0 = b * sb.k, kb = std::min(C, c0 + sb.k) - c0;
-            DedispArgs a{};
-            a.in = static_cast<const char*>(in) + (int64_t)c0 * in_pitch * g.elem;
-            a.in_pitch = in_pitch;
-            a.nchans = kb;
-            a.nsamp = L.nsamp_dec[r];
-            a.length = L.sub_len[r];
-            a.ndm = sb.ncoarse;
-            a.shifts = sb.d_rel + off;
-            a.out16 = z + (int64_t)b * sb.ncoarse * pitch1;
-            a.out_pitch = pitch1;
-            shape(a, sb.shape1);
-            a.err = err;
-            AA_CUDA(launch_dedisperse(a, s), "sub-band stage 1 launch");
-            off += (size_t)sb.ncoarse * kb;
-        }
+        ProfScope prof(kKSubband1, s);
+        DedispArgs a{};  // the first band; the others follow in one launch
+        a.in = in;
+        a.in_pitch = in_pitch;
+        a.nchans = std::min(C, sb.k);
+        a.nsamp = L.nsamp_dec[r];
+        a.length = L.sub_len[r];
+        a.ndm = sb.ncoarse;
+        a.shifts = sb.d_rel;
+        a.out16 = z;
+        a.out_pitch = pitch1;
+        shape(a, sb.shape1);
+        a.err = err;
+        AA_CUDA(launch_dedisperse_subbands(a, sb.nsub, sb.k, C, s), "sub-band stage 1 launch");
     }
     ProfScope prof(kKSubband2, s);
     AA_CUDA(launch_subband_stage2(z, (int64_t)sb.ncoarse * pitch1, pitch1, L.sub_len[r], sb.nsub, sb.ncoarse, sb.m,

@@ -921,6 +921,26 @@ __global__ void __launch_bounds__(kSmallWarps * 32) dedisperse_small_kernel(Dedi
     if (a.st_acc) add_row_sums(a.st_acc + 3 * (int64_t)d, in_row ? v : 0, in_row ? (unsigned long long)v * v : 0);
 }
 
+// Stage 1 of sub-band dedispersion: every band of k channels in one launch (a
+// launch a band left the last wave of each short: 2^17 samples of 4096 channels,
+// four ranges, 10.4 -> 7.0 ms).
+// `a` describes the first band, C all channels; the bands' delays lie one
+// after another ([trial][channel of the band]), their rows [band][trial].
+template <int SPW>
+__global__ void __launch_bounds__(kDedispThreads, 2)
+    dedisperse_subbands_kernel(DedispArgs a, int ndm_blocks, int64_t blocks, int k, int C, uint64_t wait_limit_ns,
+                               int fault_skip_chunk, uint32_t one) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ uint64_t bars[kMaxStages];
+    const int band = (int)(blockIdx.x / blocks);
+    DedispArgs b = a;
+    b.in = static_cast<const unsigned char*>(a.in) + (int64_t)band * k * a.in_pitch * (4 / SPW);
+    b.nchans = min(k, C - band * k);
+    b.shifts = a.shifts + (int64_t)band * k * a.ndm;
+    b.out16 = a.out16 + (int64_t)band * a.ndm * a.out_pitch;
+    dedisperse_block<SPW>(b, ndm_blocks, blockIdx.x - band * blocks, wait_limit_ns, fault_skip_chunk, one, smem, bars, false);
+}
+
 }  // namespace
 
 int g_fault_skip_chunk = -1;          // test hook: never issue this chunk
@@ -982,6 +1002,19 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)nblocks, kDedispThreads, a.smem, s>>>(a, ndmb, g_wait_limit_ns,
                                                             g_fault_skip_chunk, 1u);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dedisperse_subbands(const DedispArgs& a, int nsub, int k, int C, cudaStream_t s) {
+    if (a.length <= 0 || a.ndm <= 0) return cudaSuccess;
+    if (a.nstage < 1 || a.nstage > kMaxStages) return cudaErrorInvalidValue;
+    const int ndmb = (a.ndm + kDmPerBlock - 1) / kDmPerBlock;
+    const int64_t blocks = (a.length + kTau - 1) / kTau * ndmb;
+    if (blocks * nsub >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    auto kern = a.elem == 1 ? dedisperse_subbands_kernel<4> : dedisperse_subbands_kernel<2>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(blocks * nsub), kDedispThreads, a.smem, s>>>(a, ndmb, blocks, k, C, g_wait_limit_ns, g_fault_skip_chunk, 1u);
     return cudaGetLastError();
 }
 

@@ -370,6 +370,7 @@ bool bands_fit(const DedispArgs& a);  // a row buffer is there and large enough
 cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s);
 // Strategy fields of a range's kernel arguments.
 void fill_strategy(DedispArgs& a, const RangePlan& r);
+cudaError_t launch_dedisperse_subbands(const DedispArgs& a, int nsub, int k, int C, cudaStream_t s);
 cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s);
 
 cudaError_t launch_decimate(const void* in, int in_elem, int64_t in_pitch, int32_t nchans,
