@@ -259,17 +259,18 @@ struct SumArgs {
 constexpr int kSumWarps = 16;
 constexpr int kSumThreads = kSumWarps * 32;
 constexpr int kTrialsPerWarp = kBandTrials / kSumWarps;
-constexpr int kQ = kBandWords / 32;  // words per lane and trial
 
 // G: pairs added in a round (2: their four rows in 16 bits before the totals)
-template <int G>
+// Q: words a lane and trial (8, or 4 with CTAs of half the tile and windows).
+template <int G, int Q>
 __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
     extern __shared__ __align__(128) uint32_t ring[];
     __shared__ uint64_t full[kBandBars], empty[kBandBars];  // pair p: p % kBandBars
     __shared__ int gave_up, never;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int blk = blockIdx.x % a.nblk;
-    const int tw = (blockIdx.x / a.nblk) * kBandWords;  // first word of the tile
+    constexpr int kLess = kBandWords - 32 * Q;           // words that the tables' windows are longer
+    const int tw = (blockIdx.x / a.nblk) * (32 * Q);     // first word of the tile
     if (threadIdx.x == 0) {
         gave_up = never = 0;
         for (int s = 0; s < kBandBars; ++s) {
@@ -299,11 +300,11 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
     if (nb < 2 * npairs) h_next = __ldg(reinterpret_cast<const uint4*>(heads + nb));
     fetch();
 
-    uint32_t tot[kTrialsPerWarp][2 * kQ];
+    uint32_t tot[kTrialsPerWarp][2 * Q];
 #pragma unroll
     for (int i = 0; i < kTrialsPerWarp; ++i)
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) tot[i][2 * q] = tot[i][2 * q + 1] = 0;
+        for (int q = 0; q < Q; ++q) tot[i][2 * q] = tot[i][2 * q + 1] = 0;
     // both 16-bit lanes of a word into their totals, one dot product each
     auto add = [&](int i, int q, uint32_t w) {
         tot[i][2 * q] = __dp2a_lo(w, 0x00000001u, tot[i][2 * q]);
@@ -326,11 +327,11 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
             uint64_t* bar = &full[(nb >> 1) % kBandBars];
             const uint32_t dst = smem_addr(ring + h.z);
             if (lane == 0) {  // the pair's first band's offsets, then the second's
-                mbar_expect(bar, (h.y >> 16) * 4u + kBandTrials * 2u);
+                mbar_expect(bar, ((h.y >> 16) - (h.y & 0xffffu) * kLess) * 4u + kBandTrials * 2u);
                 bulk_g2s(dst + (nb & 1) * kBandTrials * 2u, offs + (int64_t)nb * kBandTrials, kBandTrials * 2u, bar);
             }
             __syncwarp();
-            if (c.w) bulk_g2s(dst + (kBandTrials + c.z) * 4u, rows + (int64_t)c.x * a.hw + c.y, c.w * 4u, bar);
+            if (c.w) bulk_g2s(dst + (kBandTrials + c.z) * 4u, rows + (int64_t)c.x * a.hw + c.y, (c.w - kLess) * 4u, bar);
             nb += kSumWarps;
             fetch();
         }
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
             for (int i = 0; i < kTrialsPerWarp; ++i) {
                 const uint32_t *p0 = z0 + word(o0, i), *p1 = z0 + word(o1, i), *p2 = z1 + word(o2, i), *p3 = z1 + word(o3, i);
 #pragma unroll
-                for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q] + p1[32 * q] + (p2[32 * q] + p3[32 * q]));
+                for (int q = 0; q < Q; ++q) add(i, q, p0[32 * q] + p1[32 * q] + (p2[32 * q] + p3[32 * q]));
             }
         } else {
 #pragma unroll
@@ -369,14 +370,14 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
                     for (int i = 0; i < kTrialsPerWarp; ++i) {
                         const uint32_t *p0 = z + word(o, i), *p1 = z + word(v, i);
 #pragma unroll
-                        for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q] + p1[32 * q]);
+                        for (int q = 0; q < Q; ++q) add(i, q, p0[32 * q] + p1[32 * q]);
                     }
                 } else {
 #pragma unroll
                     for (int i = 0; i < kTrialsPerWarp; ++i) {
                         const uint32_t* p0 = z + word(o, i);
 #pragma unroll
-                        for (int q = 0; q < kQ; ++q) add(i, q, p0[32 * q]);
+                        for (int q = 0; q < Q; ++q) add(i, q, p0[32 * q]);
                     }
                 }
             }
@@ -404,7 +405,7 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
         float* row = a.out + (int64_t)(d - a.d_lo) * a.pitch;
         unsigned long long s1 = 0, s2 = 0;
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) {
+        for (int q = 0; q < Q; ++q) {
             const uint32_t vl = tot[i][2 * q], vh = tot[i][2 * q + 1];
             if (tl + 32 * q < a.length) {
                 row[tl + 32 * q] = (float)vl;
@@ -445,9 +446,12 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
     auto rows_kern = a.row_dec > 1 ? band_rows_kernel<0> : a.elem == 1 ? band_rows_kernel<1> : band_rows_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(rows_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_rows);
     if (e != cudaSuccess) return e;
-    auto sum_kern = bp.by_two_pairs ? band_sum_kernel<2> : band_sum_kernel<1>;
-    e = cudaFuncSetAttribute(sum_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_sum);
-    if (e != cudaSuccess) return e;
+    auto sum_kern = bp.by_two_pairs ? band_sum_kernel<2, 8> : band_sum_kernel<1, 8>;
+    auto half_kern = bp.by_two_pairs ? band_sum_kernel<2, 4> : band_sum_kernel<1, 4>;
+    for (auto kern : {sum_kern, half_kern}) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_sum);
+        if (e != cudaSuccess) return e;
+    }
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 1;
@@ -515,7 +519,11 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
             sa.pitch = a.out_pitch;
             sa.st_acc = a.st_acc ? a.st_acc + 3 * (int64_t)(d0 - a.trial0) : nullptr;
             sa.err = a.err;
-            sum_kern<<<(unsigned)(nt * nblk), kSumThreads, bp.smem_sum, s>>>(sa);
+            // Half tiles take three quarters of a whole one's time (123 us against 167, a
+            // wave of 512 bands): worth it where twice the CTAs take as many waves.
+            const int64_t waves = (nt * nblk + sms - 1) / sms, half = (2 * nt * nblk + sms - 1) / sms;
+            if (half <= waves) half_kern<<<(unsigned)(2 * nt * nblk), kSumThreads, bp.smem_sum, s>>>(sa);
+            else sum_kern<<<(unsigned)(nt * nblk), kSumThreads, bp.smem_sum, s>>>(sa);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
