@@ -12,7 +12,8 @@
 // there; only the top depth's rows go to memory.  With one launch per depth every
 // sum read two samples and wrote one: 75 GB and 15.2 ms for 2^17 samples of 4096
 // channels under the four ranges of the SKA plan; in groups of 4-3-5 depths it
-// is 10 GB and 5.5 ms (5.9 with one tile a CTA, its tables read again for each).
+// is 10 GB and 5.4 ms (5.9 with one tile a CTA, its tables read again for each,
+// 5.5 with a warp per channel row instead of all rows' pieces dealt out together).
 // Shared memory bounds it (its pipe is 61-68 % busy; two CTAs of an SM hide the
 // loads of each other).  A lane sums four consecutive
 // samples: with one sample a lane (12 wavefronts for 128 sums instead of 16, but
@@ -33,7 +34,7 @@ struct FdmtArgs {
     const FdmtBlock* blocks;
     const FdmtLoad* loads;
     const FdmtOp* ops;
-    const void* leaves;
+    const void* leaf;  // channel rows
     int64_t leaf_pitch;
     const uint32_t* prev;
     uint32_t* out;
@@ -44,6 +45,9 @@ struct FdmtArgs {
     int32_t nblocks, tile, levels;
     int32_t op_words, load_words;  // words of the ops, and of the loads behind them, before the slots
     int32_t per;       // consecutive tiles of a CTA
+    int32_t leaves;    // blocks load channels
+    int32_t quads;     // pieces of four samples of the widest window
+    uint32_t quad_inv;  // 2^22 / quads, up: exact for fewer than 2^15 pieces of 128 at most
     int64_t ntiles;
 };
 
@@ -99,28 +103,40 @@ __global__ void __launch_bounds__(kFdmtThreads, 2) fdmt_group_kernel(FdmtArgs a)
             const int4 l = loads[i];
             const int64_t t = t0 + l.y;
             uint32_t* dst = slots + l.z;
-            if (l.x >= 0) {
-                const uint32_t* src = a.prev + (int64_t)l.x * a.pitch;
-                for (int j = 4 * lane; j < l.w; j += 128) {
-                    const bool in = t + j < a.pitch;  // beyond the row: zeros, which no valid output reads
-                    cp_async16(dst + j, in ? src + t + j : a.prev, in ? 16 : 0);
+            if (l.x < 0) continue;
+            const uint32_t* src = a.prev + (int64_t)l.x * a.pitch;
+            for (int j = 4 * lane; j < l.w; j += 128) {
+                const bool in = t + j < a.pitch;  // beyond the row: zeros, which no valid output reads
+                cp_async16(dst + j, in ? src + t + j : a.prev, in ? 16 : 0);
+            }
+        }
+        // channels, four samples a thread, four such pieces at a time over all of them
+        for (int p0 = threadIdx.x; p0 < (a.leaves ? nload * a.quads : 0); p0 += 4 * kFdmtThreads) {
+            uint2 w[4];
+            uint32_t* dst[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = p0 + u * kFdmtThreads;
+                const int i = (int)(((uint32_t)p * a.quad_inv) >> 22);  // p / quads
+                dst[u] = nullptr;
+                if (i >= nload) continue;
+                const int4 l = loads[i];
+                const int j = 4 * (p - i * a.quads);
+                if (l.x >= 0 || j >= l.w) continue;
+                dst[u] = slots + l.z + j;
+                const int64_t t = t0 + l.y + j, at = (int64_t)(-(l.x + 1)) * a.leaf_pitch + t;
+                w[u] = make_uint2(0, 0);
+                if (t < a.nsamp) {  // the pitch is a multiple of four samples
+                    if constexpr (EB == 1) w[u].x = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.leaf) + at));
+                    else w[u] = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(a.leaf) + at));
                 }
-            } else {
-                const int64_t row = (int64_t)(-(l.x + 1)) * a.leaf_pitch;
-#pragma unroll 4
-                for (int j = 4 * lane; j < l.w; j += 128) {
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (t + j < a.nsamp) {  // the pitch is a multiple of four samples
-                        if constexpr (EB == 1) {
-                            const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.leaves) + row + t + j));
-                            v = make_uint4(w & 0xff, (w >> 8) & 0xff, (w >> 16) & 0xff, w >> 24);
-                        } else {
-                            const uint2 w = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(a.leaves) + row + t + j));
-                            v = make_uint4(w.x & 0xffff, w.x >> 16, w.y & 0xffff, w.y >> 16);
-                        }
-                    }
-                    *reinterpret_cast<uint4*>(dst + j) = v;
-                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (!dst[u]) continue;
+                *reinterpret_cast<uint4*>(dst[u]) = EB == 1
+                    ? make_uint4(w[u].x & 0xff, (w[u].x >> 8) & 0xff, (w[u].x >> 16) & 0xff, w[u].x >> 24)
+                    : make_uint4(w[u].x & 0xffff, w[u].x >> 16, w[u].y & 0xffff, w[u].y >> 16);
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -179,7 +195,7 @@ cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_e
     a.blocks = fd.d_blocks + g.block0;
     a.loads = fd.d_loads;
     a.ops = fd.d_ops;
-    a.leaves = leaves;
+    a.leaf = leaves;
     a.leaf_pitch = leaf_pitch;
     a.prev = prev;
     a.out = out;
@@ -194,6 +210,9 @@ cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_e
     a.op_words = g.max_ops * 4;
     a.load_words = g.max_loads * 4;
     a.per = (int32_t)per;
+    a.leaves = g.leaves;
+    a.quads = g.width / 4;
+    a.quad_inv = ((1u << 22) + a.quads - 1) / a.quads;
     a.ntiles = ntiles;
     const size_t smem = ((size_t)a.op_words + (size_t)a.load_words + (size_t)g.words) * 4;
     auto kern = leaf_elem == 1 ? (fin ? fdmt_group_kernel<1, true> : fdmt_group_kernel<1, false>)

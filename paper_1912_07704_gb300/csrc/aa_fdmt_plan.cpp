@@ -222,8 +222,10 @@ bool build_fdmt_groups(FdmtPlan& fd, int32_t nchans, int elem, const std::vector
             o.load0 = (int32_t)fd.loads.size();
             o.nload = (int32_t)b.loads.size();
             o.op0 = (int32_t)fd.ops.size();
-            for (const Need& n : b.loads)
+            for (const Need& n : b.loads) {
+                g.leaves = g.leaves || n.row < 0;
                 fd.loads.push_back(FdmtLoad{n.row, (int32_t)n.lo, (int32_t)(n.slot * W), (int32_t)(n.hi - n.lo) + tile});
+            }
             const int k = bottom - top + 1;
             for (int i = k - 1, q = 0; i >= 0; --i, ++q) {
                 const int d = top + i;

@@ -138,6 +138,7 @@ struct FdmtGroup {
     int tile = 0;             // samples of a block
     int32_t width = 0, words = 0;  // words of a slot, of all slots
     int32_t max_ops = 0, max_loads = 0;  // of a block
+    bool leaves = false;  // some block loads channels
     int64_t block0 = 0;
     int32_t nblocks = 0;
 };

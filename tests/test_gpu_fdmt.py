@@ -1,4 +1,4 @@
-"""FDMT-style tree dedispersion on the GPU (one launch per depth of the
+"""FDMT-style tree dedispersion on the GPU (groups of depths of the
 channel tree) against the oracle's tree form: bit-exact rows for ragged,
 decimated, rising-band and 4096-channel plans, the single-pulse search on
 tree rows against the oracle's search, and mixed tree / exact ranges."""
