@@ -288,7 +288,7 @@ cudaError_t launch_gather(F32Args a, int32_t span, int64_t out_len, cudaStream_t
     const bool vec = a.src_pitch % 4 == 0 && (reinterpret_cast<uintptr_t>(a.src) & 15) == 0;
     auto kern = kw == 16 ? (vec ? f32_gather_kernel<MODE, 16, true> : f32_gather_kernel<MODE, 16, false>)
                          : (vec ? f32_gather_kernel<MODE, 8, true> : f32_gather_kernel<MODE, 8, false>);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)nblocks, f32_threads(kw), smem, s>>>(a, (int)ntiles);
     return cudaGetLastError();

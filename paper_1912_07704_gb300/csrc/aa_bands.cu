@@ -444,12 +444,12 @@ bool bands_fit(const DedispArgs& a) {
 cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
     const BandPlan& bp = *a.bands;
     auto rows_kern = a.row_dec > 1 ? band_rows_kernel<0> : a.elem == 1 ? band_rows_kernel<1> : band_rows_kernel<2>;
-    cudaError_t e = cudaFuncSetAttribute(rows_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_rows);
+    cudaError_t e = allow_smem((const void*)rows_kern);
     if (e != cudaSuccess) return e;
     auto sum_kern = bp.by_two_pairs ? band_sum_kernel<2, 8> : band_sum_kernel<1, 8>;
     auto half_kern = bp.by_two_pairs ? band_sum_kernel<2, 4> : band_sum_kernel<1, 4>;
     for (auto kern : {sum_kern, half_kern}) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem_sum);
+        e = allow_smem((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     int dev = 0, sms = 0;

@@ -953,7 +953,7 @@ cudaError_t launch_dedisperse_batch(const DedispArgs* d_descs, const int64_t* d_
     if (ndesc <= 0) return cudaSuccess;
     auto kern = grouped ? (elem == 1 ? dedisperse_batch_kernel<true, 1> : dedisperse_batch_kernel<true, 2>)
                         : (elem == 1 ? dedisperse_batch_kernel<false, 1> : dedisperse_batch_kernel<false, 2>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<grid, kDedispThreads, smem, s>>>(d_descs, d_first, d_ndm_blocks, ndesc, d_queue,
                                             g_wait_limit_ns, 1u);
@@ -979,7 +979,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     if (a.grouped) {
         auto kern = a.elem == 1 ? (a.gflush == 0 ? dedisperse_grouped_kernel<1, true> : dedisperse_grouped_kernel<1, false>)
                                 : (a.gflush == 0 ? dedisperse_grouped_kernel<2, true> : dedisperse_grouped_kernel<2, false>);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
+        cudaError_t e = allow_smem((const void*)kern);
         if (e != cudaSuccess) return e;
         kern<<<(unsigned)nblocks, kDedispThreads, a.smem, s>>>(a, ndmb);
         return cudaGetLastError();
@@ -998,7 +998,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
         return cudaGetLastError();
     }
     auto kern = a.elem == 1 ? dedisperse_kernel<4> : dedisperse_kernel<2>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
+    cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)nblocks, kDedispThreads, a.smem, s>>>(a, ndmb, g_wait_limit_ns,
                                                             g_fault_skip_chunk, 1u);
@@ -1012,7 +1012,7 @@ cudaError_t launch_dedisperse_subbands(const DedispArgs& a, int nsub, int k, int
     const int64_t blocks = (a.length + kTau - 1) / kTau * ndmb;
     if (blocks * nsub >= (1ll << 31)) return cudaErrorInvalidConfiguration;
     auto kern = a.elem == 1 ? dedisperse_subbands_kernel<4> : dedisperse_subbands_kernel<2>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
+    cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)(blocks * nsub), kDedispThreads, a.smem, s>>>(a, ndmb, blocks, k, C, g_wait_limit_ns, g_fault_skip_chunk, 1u);
     return cudaGetLastError();

@@ -217,7 +217,7 @@ cudaError_t launch_fdmt_group(const FdmtPlan& fd, const FdmtGroup& g, int leaf_e
     const size_t smem = ((size_t)a.op_words + (size_t)a.load_words + (size_t)g.words) * 4;
     auto kern = leaf_elem == 1 ? (fin ? fdmt_group_kernel<1, true> : fdmt_group_kernel<1, false>)
                                : (fin ? fdmt_group_kernel<2, true> : fdmt_group_kernel<2, false>);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, kFdmtThreads, smem, s>>>(a);
     return cudaGetLastError();

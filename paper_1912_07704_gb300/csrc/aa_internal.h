@@ -448,7 +448,11 @@ size_t sps_boxcar_smem(int wpad);
 // dynamic shared memory of the boxcar kernel that serves (max_width, wpad,
 // dec_w0): the decimated ladder's when dec_w0 > 0
 size_t sps_boxcar_smem_for(int32_t max_width, int32_t wpad, int32_t dec_w0);
-constexpr size_t kMaxBoxcarSmem = 227 * 1024;
+constexpr int kMaxSmem = 227 * 1024;  // shared memory of a block, static and dynamic
+constexpr size_t kMaxBoxcarSmem = kMaxSmem;
+// Before each launch of a kernel that takes dynamic shared memory: lets its
+// blocks have all there is.
+cudaError_t allow_smem(const void* kernel);
 // test hook: boxcar tiles per CTA (0: the launcher's choice)
 extern int g_boxcar_seg_tiles;
 cudaError_t launch_rsqrt_table(double* t, int wpad, cudaStream_t s);

@@ -1632,8 +1632,7 @@ cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s) {
     const size_t smem = sps_boxcar_smem_for(a.max_width, a.wpad, a.dec_w0);
     if (smem > kMaxBoxcarSmem) return cudaErrorInvalidConfiguration;
     if (a.dec_w0 > 0) {
-        cudaError_t e = cudaFuncSetAttribute(sps_boxcar_dec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = allow_smem((const void*)sps_boxcar_dec_kernel);
         if (e != cudaSuccess) return e;
         sps_boxcar_dec_kernel<<<(unsigned)nblocks, NT, smem, s>>>(a, (int)ntiles);
         return cudaGetLastError();
@@ -1648,7 +1647,7 @@ cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s) {
                         : (int)std::max<int64_t>(1, std::min<int64_t>({16, ntiles, nblocks / (sms * 2 * 16)}));
     const int64_t ncta = (int64_t)a.nrows * ((ntiles + seg - 1) / seg);
     auto kern = sps_low(a) ? sps_boxcar_kernel<true> : sps_boxcar_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)ncta, NT, smem, s>>>(a, (int)ntiles, seg);
     return cudaGetLastError();
@@ -1671,8 +1670,7 @@ cudaError_t launch_sps_boxcar_batch(const SpsArgs* d_descs, const int64_t* d_fir
                                     unsigned long long* d_queue, int grid, cudaStream_t s) {
     if (ndesc <= 0) return cudaSuccess;
     if (smem > kMaxBoxcarSmem) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(sps_boxcar_batch_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)sps_boxcar_batch_kernel);
     if (e != cudaSuccess) return e;
     sps_boxcar_batch_kernel<<<grid, NT, smem, s>>>(d_descs, d_first, d_ntiles, ndesc, d_queue);
     return cudaGetLastError();

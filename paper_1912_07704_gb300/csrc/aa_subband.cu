@@ -97,7 +97,7 @@ cudaError_t launch_subband_stage2(const uint16_t* z, int64_t band_stride, int64_
     const int64_t nblocks = ntiles * ncoarse;
     if (nblocks >= (1ll << 31) || m > kSb2Warps || pitch1 % 8 || band_stride % 8)
         return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(subband_stage2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)subband_stage2_kernel);
     if (e != cudaSuccess) return e;
     subband_stage2_kernel<<<(unsigned)nblocks, kSb2Warps * 32, smem, s>>>(
         z, band_stride, pitch1, nsub, ncoarse, m, ndm, s2, swin, nbc, head, out, out_pitch, length);
