@@ -221,12 +221,16 @@ typedef struct aa_candidate {
  *              At most 2 GiB at its end are a row buffer (the sums of 8, 4 or
  *              2 consecutive channels that many trials share); with less
  *              scratch, down to what the decimated inputs and the sub-band and
- *              FDMT ranges take, the call runs without it: same results, slower.
+ *              FDMT ranges take (aa_dedisperse_least_ws_bytes), the call runs
+ *              without it: same results, slower.
  * The plan must be bound.  Stream-ordered, asynchronous; returns
  * AA_ERR_ARG/AA_ERR_STATE on bad arguments, AA_ERR_CUDA if a launch fails. */
 aa_status aa_dedisperse_device(const aa_plan* plan, const uint8_t* d_in, int64_t nsamp,
                                int64_t in_pitch, float* d_out, void* d_ws, size_t ws_bytes,
                                aa_stream_t stream);
+/* The least scratch aa_dedisperse_device accepts for nsamp samples
+ * (aa_plan_info.dedisp_ws_bytes without the row buffer). */
+aa_status aa_dedisperse_least_ws_bytes(const aa_plan* plan, int64_t nsamp, size_t* bytes);
 
 /* Single-pulse search over every dedispersed series in d_dd (layout as
  * written by aa_dedisperse_device for the same nsamp).
@@ -612,11 +616,15 @@ void aa_candidates_destroy(aa_candidates* c);
  * aa_search_fused_device: d_in as in aa_dedisperse_device; candidates as in
  * aa_sps_search_device; d_ws 256-byte aligned, >= the bytes above (for plans
  * whose decimated inputs leave little room for a row buffer these include up
- * to 512 MiB for one, without which the call runs slower).  Its first word is the error word (aa_workspace_status).  Stream-ordered.
+ * to 512 MiB for one, without which the call runs slower: the least it accepts
+ * is aa_search_fused_least_ws_bytes).  Its first word is the error word
+ * (aa_workspace_status).  Stream-ordered.
  * AA_ERR_CONFIG for plans with sub-band or FDMT ranges; AA_ERR_ARG on bad
  * arguments. */
 aa_status aa_search_fused_ws_bytes(const aa_plan* plan, int64_t nsamp, int32_t max_width,
                                    int32_t stripe_trials, size_t* bytes, size_t* sps_ws_offset);
+aa_status aa_search_fused_least_ws_bytes(const aa_plan* plan, int64_t nsamp, int32_t max_width,
+                                         int32_t stripe_trials, size_t* bytes);
 aa_status aa_search_fused_device(const aa_plan* plan, const uint8_t* d_in, int64_t nsamp,
                                  int64_t in_pitch, int32_t max_width, float threshold,
                                  int32_t stripe_trials, aa_candidate* d_cands,

@@ -122,6 +122,8 @@ _SIG = {
     "aa_candidates_destroy": (None, [_P]),
     "aa_search_fused_ws_bytes": (ctypes.c_int, [_P, _I64, _I32, _I32, ctypes.POINTER(ctypes.c_size_t),
                                                 ctypes.POINTER(ctypes.c_size_t)]),
+    "aa_search_fused_least_ws_bytes": (ctypes.c_int, [_P, _I64, _I32, _I32, ctypes.POINTER(ctypes.c_size_t)]),
+    "aa_dedisperse_least_ws_bytes": (ctypes.c_int, [_P, _I64, ctypes.POINTER(ctypes.c_size_t)]),
     "aa_search_fused_device": (ctypes.c_int, [_P, _P, _I64, _I64, _I32, _F32, _I32, _P, _I64, _P, _P,
                                               _P, ctypes.c_size_t, _P]),
     "aa_pipeline_create": (ctypes.c_int, [_P, _I64, _I32, _F32, _I64, _I32, ctypes.POINTER(_P)]),
@@ -315,6 +317,19 @@ def aa_search_fused_ws_bytes(plan, nsamp, max_width, stripe_trials=0) -> tuple:
                                          ctypes.byref(b), ctypes.byref(off)),
           "aa_search_fused_ws_bytes")
     return b.value, off.value
+
+
+def aa_search_fused_least_ws_bytes(plan, nsamp, max_width, stripe_trials=0) -> int:
+    b = ctypes.c_size_t()
+    check(lib().aa_search_fused_least_ws_bytes(plan, int(nsamp), int(max_width), int(stripe_trials), ctypes.byref(b)),
+          "aa_search_fused_least_ws_bytes")
+    return b.value
+
+
+def aa_dedisperse_least_ws_bytes(plan, nsamp) -> int:
+    b = ctypes.c_size_t()
+    check(lib().aa_dedisperse_least_ws_bytes(plan, int(nsamp), ctypes.byref(b)), "aa_dedisperse_least_ws_bytes")
+    return b.value
 
 
 def aa_search_fused_device(plan, d_in, nsamp, in_pitch, max_width, threshold, stripe_trials,

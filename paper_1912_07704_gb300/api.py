@@ -149,13 +149,25 @@ class Plan:
     def alloc_workspace(self, nbytes: int) -> torch.Tensor:
         return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device="cuda")
 
+    def _workspace(self, nbytes: int, least) -> torch.Tensor:
+        """Workspace of nbytes, or of least() where there is no memory for the
+        row buffer in it (the call then runs without)."""
+        try:
+            return self.alloc_workspace(nbytes)
+        except torch.cuda.OutOfMemoryError:
+            smaller = least()
+            if smaller >= nbytes:
+                raise
+        return self.alloc_workspace(smaller)
+
     def dedisperse_device(self, d_in: torch.Tensor, nsamp: int, out=None, ws=None,
                           stream=None) -> torch.Tensor:
         self.bind()
         info = self.query(nsamp)
         out = self.alloc_output(nsamp) if out is None else out
-        ws = self.alloc_workspace(info.dedisp_ws_bytes) if ws is None else ws
-        assert out.numel() >= info.dd_elems and ws.numel() >= info.dedisp_ws_bytes
+        ws = (self._workspace(info.dedisp_ws_bytes, lambda: abi.aa_dedisperse_least_ws_bytes(self.handle, nsamp))
+              if ws is None else ws)
+        assert out.numel() >= info.dd_elems
         abi.aa_dedisperse_device(self.handle, d_in.data_ptr(), nsamp, d_in.stride(0),
                                  out.data_ptr(), ws.data_ptr(), ws.numel(), _stream_handle(stream))
         return out
@@ -189,8 +201,10 @@ class Plan:
         ws[fused_ws_bytes(...)[1]:]."""
         self.bind()
         assert x.dtype == torch.uint8 and x.is_cuda and x.dim() == 2 and x.stride(1) == 1
-        nbytes, _ = self.fused_ws_bytes(nsamp, max_width, stripe_trials)
-        ws = self.alloc_workspace(nbytes) if ws is None else ws
+        if ws is None:
+            nbytes, _ = self.fused_ws_bytes(nsamp, max_width, stripe_trials)
+            ws = self._workspace(nbytes, lambda: abi.aa_search_fused_least_ws_bytes(self.handle, nsamp, max_width,
+                                                                                    stripe_trials))
         cands = (torch.empty(max(capacity, 1) * 16, dtype=torch.uint8, device="cuda")
                  if cands is None else cands)
         count = torch.zeros(1, dtype=torch.int64, device="cuda") if count is None else count

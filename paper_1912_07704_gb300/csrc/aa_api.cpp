@@ -374,6 +374,14 @@ static aa_status launch_subband(const aa_plan* p, size_t r, const Layout& L, con
 
 extern "C" {
 
+aa_status aa_dedisperse_least_ws_bytes(const aa_plan* p, int64_t nsamp, size_t* bytes) {
+    clear_error();
+    if (!p || !bytes) { set_error("plan/bytes is NULL"); return AA_ERR_ARG; }
+    if (nsamp < 0) { set_error("nsamp must be >= 0"); return AA_ERR_ARG; }
+    *bytes = (size_t)make_layout(*p, nsamp, 0).dedisp_base;
+    return AA_OK;
+}
+
 aa_status aa_dedisperse_device(const aa_plan* p, const uint8_t* d_in, int64_t nsamp,
                                int64_t in_pitch, float* d_out, void* d_ws, size_t ws_bytes,
                                aa_stream_t stream) {

@@ -97,19 +97,33 @@ aa_status aa::fused_bytes(const aa_plan& p, int64_t nsamp, int32_t max_width, in
     return st;
 }
 
-extern "C" {
-
-aa_status aa_search_fused_ws_bytes(const aa_plan* p, int64_t nsamp, int32_t max_width, int32_t stripe_trials,
-                                   size_t* bytes, size_t* sps_ws_offset) {
+static aa_status sizes(const aa_plan* p, int64_t nsamp, int32_t max_width, int32_t stripe_trials, const size_t* bytes,
+                       FusedLayout& f) {
     clear_error();
     if (!p || !bytes) { set_error("plan/bytes is NULL"); return AA_ERR_ARG; }
     if (nsamp < 0) { set_error("nsamp must be >= 0"); return AA_ERR_ARG; }
     if (max_width < 1 || max_width > 65535) { set_error("max_width must be in [1, 65535]"); return AA_ERR_ARG; }
+    return fused_layout(*p, nsamp, max_width, stripe_trials, f);
+}
+
+extern "C" {
+
+aa_status aa_search_fused_ws_bytes(const aa_plan* p, int64_t nsamp, int32_t max_width, int32_t stripe_trials,
+                                   size_t* bytes, size_t* sps_ws_offset) {
     FusedLayout f;
-    const aa_status st = fused_layout(*p, nsamp, max_width, stripe_trials, f);
+    const aa_status st = sizes(p, nsamp, max_width, stripe_trials, bytes, f);
     if (st != AA_OK) return st;
     *bytes = (size_t)f.bytes;
     if (sps_ws_offset) *sps_ws_offset = (size_t)f.sps_offset;
+    return AA_OK;
+}
+
+aa_status aa_search_fused_least_ws_bytes(const aa_plan* p, int64_t nsamp, int32_t max_width, int32_t stripe_trials,
+                                         size_t* bytes) {
+    FusedLayout f;
+    const aa_status st = sizes(p, nsamp, max_width, stripe_trials, bytes, f);
+    if (st != AA_OK) return st;
+    *bytes = (size_t)f.base;
     return AA_OK;
 }
 
