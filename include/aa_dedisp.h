@@ -271,8 +271,9 @@ aa_status aa_workspace_status(void* d_ws, aa_stream_t stream);
  *     channels whose delays differ from the block's first trial by the same
  *     amounts at every trial are first summed once; each trial then adds the
  *     group sums.  Available when the plan could build the group tables.
- * Where they are cheaper (AA_DEDISP_GROUPED, or the plan's own choice) and
- * the call's scratch holds their row buffer, band rows run instead: every
+ * Where they are estimated to be faster at the call's length (AA_DEDISP_GROUPED,
+ * or the plan's own choice) and its scratch holds their row buffer, band rows
+ * run instead: every
  * distinct sum of a band of consecutive channels is built once for many
  * trials and each trial adds one per band.  aa_plan_set_strategy with
  * AA_DEDISP_DIRECT, and aa_plan_autotune choosing it, keep the direct kernel. */
@@ -830,9 +831,10 @@ aa_status aa_corner_turn_device(const uint8_t* d_tm, int64_t nsamp, int32_t ncha
  * without writing output; the grouped strategy has no staging waits); what =
  * 2: set the wait limit to `value` nanoseconds (default 2 s); what = 3: the
  * boxcar kernel processes `value` consecutive tiles of a series per CTA
- * (0: its own choice; the results do not depend on it).
- * Returns AA_ERR_ARG for an unknown `what`, a non-positive limit or a tile
- * count outside [0, 4096]. */
+ * (0: its own choice; the results do not depend on it); what = 4: band rows run
+ * wherever they fit (1), or where they are estimated to be faster (0).
+ * Returns AA_ERR_ARG for an unknown `what`, a non-positive limit, a tile count
+ * outside [0, 4096] or a switch outside [0, 1]. */
 aa_status aa_debug_inject(int32_t what, int64_t value);
 
 #ifdef __cplusplus

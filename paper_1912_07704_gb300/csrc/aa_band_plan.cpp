@@ -391,8 +391,85 @@ int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials) {
     const int64_t nblk = std::max(1, trials / kBandTrials);
     const int64_t tiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
     // a stripe that does not begin with a block touches one more
-    return bytes_for(bp, std::min<int64_t>(tiles, std::max<int64_t>(kBandLeastTiles, (2 * 152 + nblk - 1) / nblk)),
+    return bytes_for(bp, std::min<int64_t>(tiles, std::max<int64_t>(kBandLeastTiles, (2 * kBandSms + nblk - 1) / nblk)),
                      (int)nblk + (trials % kBandTrials != 0));
+}
+
+namespace {
+
+int64_t div_up(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Which side a launch takes.  Short outputs leave band rows the worse: a row is
+// as long as the delays it is used at lie apart, whatever the output, so that at
+// 300 samples of 1600 trials (1024 channels, DM step 1) rows and sums took 540 us
+// where the direct kernel takes 160; at 16000 samples it is the other way round.
+// Both times are estimated, in us, from what was measured on 6325 shapes (32 to
+// 4096 channels, DM steps 0.05 to 1, 32 to 1600 trials, 200 to 64000 samples,
+// decimations 1, 2 and 8), each with a row buffer and without: nine tenths of the
+// estimates are within 10 %.  Where they decide, 28 of the shapes are more than
+// 5 % slower than the other side (1.25x at most), 81 more than 5 % slower than
+// band rows would be (1.23x); with band rows wherever they fit it was 1699, up to
+// 3.4x.
+double bands_us(const BandPlan& bp, int trial0, int ndm, int64_t length, int64_t bytes) {
+    const int64_t all = div_up(length, 2 * kBandWords);
+    double us = 0;
+    for (const BandSegment& s : bp.segs) {
+        const int d0 = std::max(trial0, s.trial0), d1 = std::min(trial0 + ndm, s.trial0 + s.ntrials);
+        if (d0 >= d1) continue;
+        const int g0 = (d0 - s.trial0) / kBandTrials, g1 = (d1 - 1 - s.trial0) / kBandTrials;
+        int64_t id, pre, nrows, words;
+        band_window(s, g0, g1, id, pre, nrows, words);
+        const int64_t nt = std::max<int64_t>(1, std::min(all, (bytes / 4 - words) / (nrows * kBandWords)));
+        const double slabs = (double)div_up(all, nt);
+        // row kernel: six CTAs an SM, each a tile of one band's rows; its channels' loads where the rows are few
+        const double ctas = std::max(1.0, (double)(div_up(nt * kBandWords + bp.max_ulen + 15, bp.tile) * bp.nbands) / (6 * kBandSms));
+        const double row_us = std::max(1.02 * ctas * (1.0 + 0.1 * (double)nrows / bp.nbands * bp.tile / kBandWords) +
+                                           0.042 * (double)(nrows * nt * kBandWords + words) / (kBandWords * kBandSms),
+                                       5.0 * ctas * bp.k * bp.tile / 4096);
+        // sums: one CTA an SM, whole tiles or halves as launch_bands takes them
+        const int64_t n = nt * (g1 - g0 + 1), whole = div_up(n, kBandSms), half = div_up(2 * n, kBandSms);
+        const double waves = half <= whole ? 0.74 * half : (double)whole;
+        us += slabs * (5.2 + row_us + waves * (4.9 + 0.3 * bp.nbands));
+    }
+    return us;
+}
+
+// The strategy's own kernel: 16 trials x 512 samples a CTA, two an SM.
+double strategy_us(int nchans, int ndm, int64_t length, bool grouped, double gwork, int elem) {
+    const double c = nchans, wide = elem == 2 ? 1.0 : 0.0;
+    const int64_t small = div_up(length, kSmallDirectTau) * ndm;
+    if (!grouped && small <= kSmallDirect * kBandSms)
+        return 5.6 + c * (0.009 + 0.015 * wide + 0.0585 * (double)small / (kSmallDirect * kBandSms));
+    const int64_t n = div_up(ndm, kDmPerBlock) * div_up(length, kTau), full = n / (2 * kBandSms), rest = n % (2 * kBandSms);
+    const double one = rest > 0 && rest <= kBandSms, two = rest > kBandSms;  // CTAs of an SM in the last wave
+    if (!grouped) return 6.0 + c * ((0.222 + 0.018 * wide) * (double)full + (0.137 + 0.013 * wide) * one + (0.228 + 0.018 * wide) * two);
+    return 10.0 + 2.0 * (1 - wide) + c * ((0.017 + 0.023 * wide + 0.24 * gwork) * (double)full +
+                                          (0.0165 + 0.01 * wide + (0.157 + 0.03 * wide) * gwork) * one +
+                                          (0.0154 + 0.021 * wide + (0.2575 + 0.02 * wide) * gwork) * two);
+}
+
+}  // namespace
+
+int g_bands_always = 0;
+
+bool bands_pay(const DedispArgs& a) {
+    if (g_bands_always) return true;
+    return bands_us(*a.bands, a.trial0, a.ndm, a.length, a.band_bytes) <=
+           strategy_us(a.nchans, a.ndm, a.length, a.grouped != 0, a.gwork, a.elem);
+}
+
+bool bands_pay(const RangePlan& r, int nchans, int64_t length, int32_t trials, int64_t bytes) {
+    if (!r.bands.ok || length <= 0) return false;
+    DedispArgs a{};
+    a.nchans = nchans;
+    a.ndm = std::min(trials, r.desc.ndm);
+    a.length = length;
+    a.elem = r.elem;
+    a.grouped = r.strategy == 1;
+    a.gwork = r.gwork;
+    a.bands = &r.bands;
+    a.band_bytes = bytes;
+    return bands_pay(a);
 }
 
 }  // namespace aa

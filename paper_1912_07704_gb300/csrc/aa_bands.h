@@ -27,6 +27,7 @@ constexpr int kBandWords = 256;    // words (pairs of samples) per CTA
 constexpr int kBandMaxRows = 32;   // rows of one band used by one block (one lane each)
 constexpr int kBandBars = 32;      // pairs in the summing kernel's ring at most
 constexpr int kBandLeastTiles = 16;  // fewer tiles in the row buffer are left to the other kernels
+constexpr int kBandSms = 152;      // SMs that sizes and estimates assume, whatever plan is bound where
 constexpr int kBandLag = 3;        // a place is refilled while the third pair behind its own is added
 
 struct BandQuad {  // sum of up to four channels of one half of a band

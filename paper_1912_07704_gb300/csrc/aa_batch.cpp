@@ -318,9 +318,12 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
     int64_t rows = 0;
     for (int i = 0; i < nbeams; ++i) {
         const Layout L = make_layout(*plans[i], nsamps[i], max_width);
-        for (size_t r = 0; r < plans[i]->ranges.size(); ++r)
-            if (uses_bands(plans[i]->ranges[r]))
-                rows = std::max(rows, band_bytes_busy(plans[i]->ranges[r].bands, L.length[r], plans[i]->ranges[r].desc.ndm));
+        for (size_t r = 0; r < plans[i]->ranges.size(); ++r) {
+            const RangePlan& g = plans[i]->ranges[r];
+            if (!uses_bands(g)) continue;
+            const int64_t busy = band_bytes_busy(g.bands, L.length[r], g.desc.ndm);
+            if (bands_pay(g, plans[i]->nchans, L.length[r], g.desc.ndm, busy)) rows = std::max(rows, busy);
+        }
     }
     const int64_t used = std::min(kDefaultBranches, nbeams);
     rows = std::min({rows, kBranchRowsMax, wave_bytes / used / 256 * 256}) * used;

@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(256) decimate_batch_kernel(const DecimateJob* 
 // (4 a lane, words read at their places and shifted), its warps every eighth
 // channel, their sums added in shared memory.
 constexpr int kSmallWarps = 8;
-constexpr int kSmallTau = 128;
+constexpr int kSmallTau = kSmallDirectTau;
 template <int SPW>
 __global__ void __launch_bounds__(kSmallWarps * 32) dedisperse_small_kernel(DedispArgs a, int ntiles) {
     __shared__ __align__(16) uint32_t part[kSmallWarps][kSmallTau];
@@ -975,7 +975,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     const int64_t ntiles = (a.length + kTau - 1) / kTau;
     const int64_t nblocks = (int64_t)ndmb * ntiles;
     if (nblocks >= (1ll << 31)) return cudaErrorInvalidConfiguration;
-    if (bands_fit(a)) return launch_bands(a, s);
+    if (bands_fit(a) && (a.row_dec > 1 || bands_pay(a))) return launch_bands(a, s);
     if (a.grouped) {
         auto kern = a.elem == 1 ? (a.gflush == 0 ? dedisperse_grouped_kernel<1, true> : dedisperse_grouped_kernel<1, false>)
                                 : (a.gflush == 0 ? dedisperse_grouped_kernel<2, true> : dedisperse_grouped_kernel<2, false>);
@@ -992,7 +992,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 0;
     const int64_t small = (a.length + kSmallTau - 1) / kSmallTau * a.ndm;
-    if (small <= 8 * (int64_t)sms && !a.out16 && g_fault_skip_chunk < 0) {
+    if (small <= kSmallDirect * (int64_t)sms && !a.out16 && g_fault_skip_chunk < 0) {
         auto kern = a.elem == 1 ? dedisperse_small_kernel<4> : dedisperse_small_kernel<2>;
         kern<<<(unsigned)small, kSmallWarps * 32, 0, s>>>(a, (int)(small / a.ndm));
         return cudaGetLastError();

@@ -80,9 +80,11 @@ aa_status fused_layout(const aa_plan& p, int64_t nsamp, int32_t max_width, int32
     f.acc_offset = f.stripe_offset + round_up((int64_t)f.stripe * f.stripe_pitch * 4, 256);
     f.base = f.acc_offset + round_up((int64_t)f.stripe * 3 * 8, 256);
     int64_t rows = 0;
-    for (size_t r = 0; r < p.ranges.size(); ++r)
-        if (uses_bands(p.ranges[r]))
-            rows = std::max(rows, std::min(kRowBufferMax, band_bytes_busy(p.ranges[r].bands, f.L.length[r], f.stripe)));
+    for (size_t r = 0; r < p.ranges.size(); ++r) {
+        if (!uses_bands(p.ranges[r])) continue;
+        const int64_t n = std::min(kRowBufferMax, band_bytes_busy(p.ranges[r].bands, f.L.length[r], f.stripe));
+        if (bands_pay(p.ranges[r], p.nchans, f.L.length[r], f.stripe, n)) rows = std::max(rows, n);
+    }
     f.bytes = f.base + (rows > f.dec_bytes ? rows : 0);
     return AA_OK;
 }
@@ -223,7 +225,7 @@ aa_status aa_search_fused_device(const aa_plan* p, const uint8_t* d_in, int64_t 
                 t.bands = &g.bands;
                 t.band_rows = reinterpret_cast<uint32_t*>(dec_region);
                 t.band_bytes = f.dec_bytes;
-                if (bands_fit(t)) {
+                if (bands_fit(t) && bands_pay(g, C, L.length[r], f.stripe, f.dec_bytes)) {
                     row_buf = dec_region;
                     row_bytes = f.dec_bytes;
                     row_dec = g.desc.dec;

@@ -351,6 +351,7 @@ struct DedispArgs {
     // > 1: `in` is the 8-bit input (in_pitch bytes) and the row kernel sums
     // row_dec samples as it reads it; only for launches that bands_fit takes
     int32_t row_dec;
+    double gwork;  // adds of the grouped strategy / adds of the direct one
 };
 // Given a row buffer, a range runs on band rows where it has them, unless the
 // direct strategy was asked for.
@@ -368,6 +369,15 @@ int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials);
 // the kernels do; false if a table entry is inconsistent
 bool band_shifts(const BandPlan& bp, int nchans, int ndm, int32_t* out);
 bool bands_fit(const DedispArgs& a);  // a row buffer is there and large enough
+// A launch that bands_fit takes is faster on band rows than on its strategy's
+// kernel, by the estimates of aa_band_plan.cpp.
+bool bands_pay(const DedispArgs& a);
+// The same for all trials of a range, or a stripe of so many, given a row
+// buffer of `bytes`: whether one is of use.
+bool bands_pay(const RangePlan& r, int nchans, int64_t length, int32_t trials, int64_t bytes);
+constexpr int kSmallDirect = 8;      // CTAs per SM up to which the direct strategy takes its small kernel ...
+constexpr int kSmallDirectTau = 128; // ... of one trial and this many samples a CTA
+extern int g_bands_always;  // test hook: band rows wherever they fit
 cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s);
 // Strategy fields of a range's kernel arguments.
 void fill_strategy(DedispArgs& a, const RangePlan& r);

@@ -296,6 +296,7 @@ void fill_strategy(DedispArgs& a, const RangePlan& r) {
         a.gmem = nullptr;
     }
     a.bands = uses_bands(r) ? &r.bands : nullptr;
+    a.gwork = r.gwork;
 }
 
 static aa_status build_strategy(aa_plan& p) {
@@ -414,8 +415,12 @@ Layout make_layout(const aa_plan& p, int64_t nsamp, int32_t max_width) {
     }
     L.dedisp_base = ws;  // always holds at least the error word
     int64_t rows = 0;
-    for (size_t q = 0; q < p.ranges.size(); ++q)
-        if (uses_bands(p.ranges[q])) rows = std::max(rows, band_bytes(p.ranges[q].bands, L.length[q]));
+    for (size_t q = 0; q < p.ranges.size(); ++q) {
+        const RangePlan& r = p.ranges[q];
+        if (!uses_bands(r)) continue;
+        const int64_t bytes = band_bytes(r.bands, L.length[q]);
+        if (bands_pay(r, p.nchans, L.length[q], r.desc.ndm, bytes)) rows = std::max(rows, bytes);
+    }
     L.dedisp_ws = ws + rows;
     L.max_width = max_width;
     if (max_width > 0) {

@@ -1,7 +1,8 @@
 """Band rows of the grouped strategy against the direct kernel (bit for bit):
 last bands of 1 to 8 channels, parts of blocks and segments, one tile and
 several slabs, both halves of a word past the series end, and the least
-scratch, with which the grouped kernel runs instead."""
+scratch, with which the grouped kernel runs instead.  Short outputs included:
+band rows run here wherever they fit, not only where they are the faster side."""
 import pytest
 import torch
 
@@ -9,6 +10,14 @@ from paper_1912_07704_gb300 import abi, synth
 from paper_1912_07704_gb300.api import Plan
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _wherever_they_fit():
+    abi.aa_debug_inject(4, 1)
+    yield
+    abi.aa_debug_inject(0, 0)
+
 
 CASES = [  # nchans, foff, ranges, output samples of the first range
     (1024, -300.0 / 1024, ((0.0, 0.1, 600, 1), (60.0, 0.2, 70, 2)), 1),

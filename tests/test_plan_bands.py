@@ -21,8 +21,44 @@ PLANS = {
 }
 
 
+# nchans, DM step, trials, samples, band rows faster (measured, us with / without)
+SIDES = [
+    (1024, 1.0, 1600, 300, False),   # 540 / 160
+    (1024, 1.0, 1600, 16000, True),
+    (256, 0.3, 1600, 300, False),    # 98 / 39
+    (256, 1.0, 700, 1000, False),    # 85 / 45
+    (64, 0.3, 64, 4000, False),      # 18 / 14
+    (64, 0.1, 1500, 64000, True),
+    (4096, 0.1, 1500, 16000, True),
+]
+
+
+@pytest.mark.parametrize("C, step, ndm, length, bands", SIDES)
+def test_row_buffer_is_asked_for_where_band_rows_are_faster(C, step, ndm, length, bands):
+    p = Plan(C, 1508.0, -300.0 / C, 64e-6, [(0.0, step, ndm, 1)])
+    n = length + int(p.shifts(0).max())
+    least = abi.aa_dedisperse_least_ws_bytes(p.handle, n)
+    assert (p.query(n).dedisp_ws_bytes > least) == bands
+    try:
+        abi.aa_debug_inject(4, 1)
+        assert p.query(n).dedisp_ws_bytes > least
+    finally:
+        abi.aa_debug_inject(0, 0)
+    p.set_strategy(0, abi.AA_DEDISP_DIRECT)
+    assert p.query(n).dedisp_ws_bytes == least
+    with pytest.raises(abi.AAError, match="AA_ERR_ARG"):
+        abi.aa_debug_inject(4, 2)
+
+
+@pytest.fixture
+def wherever_they_fit():
+    abi.aa_debug_inject(4, 1)
+    yield
+    abi.aa_debug_inject(0, 0)
+
+
 @pytest.mark.parametrize("name", PLANS)
-def test_band_tables_add_up_to_the_delays(name):
+def test_band_tables_add_up_to_the_delays(name, wherever_they_fit):
     C, fch1, foff, ranges = PLANS[name]
     p = Plan(C, fch1, foff, 64e-6, ranges)
     banded = 0
