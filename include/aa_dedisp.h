@@ -826,10 +826,11 @@ aa_status aa_corner_turn_device(const uint8_t* d_tm, int64_t nsamp, int32_t ncha
 /* Fault injection for tests of the bounded device-side waits; affects every
  * later launch in the process.  what = 0: reset all hooks; what = 1: the
  * direct-strategy dedispersion producer never issues the staging copy of
- * channel chunk `value` (that stage's barrier never completes, so every CTA
- * gives up after the wait limit, sets the workspace error word and exits
- * without writing output; the grouped strategy has no staging waits); what =
- * 2: set the wait limit to `value` nanoseconds (default 2 s); what = 3: the
+ * channel chunk `value`, the sums over band rows never those of band `value`
+ * (that barrier never completes, so every CTA gives up after the wait limit,
+ * sets the workspace error word and exits without writing output; the grouped
+ * strategy's own kernel has no staging waits); what = 2: set the limit of each
+ * wait to `value` nanoseconds (default 2 s); what = 3: the
  * boxcar kernel processes `value` consecutive tiles of a series per CTA
  * (0: its own choice; the results do not depend on it); what = 4: band rows run
  * wherever they fit (1), or where they are estimated to be faster (0).

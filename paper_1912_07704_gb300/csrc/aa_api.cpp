@@ -10,11 +10,6 @@
 
 #include "aa_internal.h"
 
-namespace aa {
-extern int g_fault_skip_chunk;
-extern uint64_t g_wait_limit_ns;
-}  // namespace aa
-
 using namespace aa;
 
 struct aa_dd_result {

@@ -60,16 +60,24 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Tries before a wait gives up: a failed try takes from tens of nanoseconds
-// (at least 0.1 s in all) to the hardware's suspend time; no copy takes long.
-constexpr int kTries = 1 << 23;
-// false if the phase did not complete within kTries, or the CTA gave up
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const volatile int* gave_up) {
-    for (int i = 0; i < kTries; ++i) {
-        if (mbar_try(bar, parity)) return true;
-        if ((i & 63) == 63 && *gave_up) return false;
-    }
-    return false;
+// the clock in units of 1.024 us
+__device__ __forceinline__ uint32_t ticks() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return (uint32_t)(t >> 10);
+}
+// Wait for a phase; false if it did not complete within `limit` ticks, or the CTA
+// gave up.  Only the first try is inline (2^18 samples of 4096 channels, four ranges:
+// 24.04 ms, 24.30 with the clock's loop in line).
+__device__ __noinline__ bool mbar_wait_on(uint64_t* bar, uint32_t parity, uint32_t limit, const volatile int* gave_up) {
+    const uint32_t start = ticks();
+    while (!mbar_try(bar, parity))
+        if (*gave_up || ticks() - start > limit) return false;
+    return true;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit, const volatile int* gave_up) {
+    if (mbar_try(bar, parity)) return true;
+    return mbar_wait_on(bar, parity, limit, gave_up);
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -254,6 +262,8 @@ struct SumArgs {
     int64_t pitch;
     unsigned long long* st_acc;
     unsigned* err;
+    uint32_t wait;      // limit of each wait, ticks of 1.024 us
+    int32_t skip_band;  // test hook: this band's copies are never issued (-1: none)
 };
 
 constexpr int kSumWarps = 16;
@@ -266,13 +276,13 @@ template <int G, int Q>
 __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
     extern __shared__ __align__(128) uint32_t ring[];
     __shared__ uint64_t full[kBandBars], empty[kBandBars];  // pair p: p % kBandBars
-    __shared__ int gave_up, never;
+    __shared__ int gave_up;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int blk = blockIdx.x % a.nblk;
     constexpr int kLess = kBandWords - 32 * Q;           // words that the tables' windows are longer
     const int tw = (blockIdx.x / a.nblk) * (32 * Q);     // first word of the tile
     if (threadIdx.x == 0) {
-        gave_up = never = 0;
+        gave_up = 0;
         for (int s = 0; s < kBandBars; ++s) {
             mbar_init(&full[s], 2);  // a pair's two bands
             mbar_init(&empty[s], kSumWarps);
@@ -320,18 +330,19 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
     for (int pr = 0; pr < npairs; pr += G) {
         while ((int)h.w >> 16 <= pr) {  // at
             const int after = (int16_t)(h.w & 0xffffu);
-            if (after >= 0 && !__all_sync(0xffffffffu, mbar_wait(&empty[after % kBandBars], (uint32_t)(after / kBandBars) & 1u, &gave_up))) {
+            if (after >= 0 && !__all_sync(0xffffffffu, mbar_wait(&empty[after % kBandBars], (uint32_t)(after / kBandBars) & 1u, a.wait, &gave_up))) {
                 ok = false;
                 break;
             }
             uint64_t* bar = &full[(nb >> 1) % kBandBars];
             const uint32_t dst = smem_addr(ring + h.z);
-            if (lane == 0) {  // the pair's first band's offsets, then the second's
+            const bool issue = nb != a.skip_band;
+            if (lane == 0 && issue) {  // the pair's first band's offsets, then the second's
                 mbar_expect(bar, ((h.y >> 16) - (h.y & 0xffffu) * kLess) * 4u + kBandTrials * 2u);
                 bulk_g2s(dst + (nb & 1) * kBandTrials * 2u, offs + (int64_t)nb * kBandTrials, kBandTrials * 2u, bar);
             }
             __syncwarp();
-            if (c.w) bulk_g2s(dst + (kBandTrials + c.z) * 4u, rows + (int64_t)c.x * a.hw + c.y, (c.w - kLess) * 4u, bar);
+            if (c.w && issue) bulk_g2s(dst + (kBandTrials + c.z) * 4u, rows + (int64_t)c.x * a.hw + c.y, (c.w - kLess) * 4u, bar);
             nb += kSumWarps;
             fetch();
         }
@@ -343,7 +354,7 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
 #pragma unroll
         for (int u = 0; u < G; ++u)
             if (pr + u < npairs)
-                ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[(pr + u) % kBandBars], (uint32_t)((pr + u) / kBandBars) & 1u, &gave_up));
+                ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[(pr + u) % kBandBars], (uint32_t)((pr + u) / kBandBars) & 1u, a.wait, &gave_up));
         if (!ok) break;
         // this warp's trials' words of the first and the second band of a pair
         auto first = [&](int u) { return *reinterpret_cast<const uint2*>(sp[u] + 2 * warp); };
@@ -390,9 +401,11 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
         atomicOr(a.err, 1u);
     }
     __syncthreads();
-    if (gave_up) {  // this warp's copies in flight land before the CTA leaves
+    if (gave_up) {  // this warp's copies in flight land before the CTA leaves, one limit for all of them
+        const uint32_t start = ticks();
         for (int i = max(warp, nb - 2 * kBandBars); i < nb; i += kSumWarps)
-            mbar_wait(&full[(i >> 1) % kBandBars], (uint32_t)((i >> 1) / kBandBars) & 1u, &never);
+            while (!mbar_try(&full[(i >> 1) % kBandBars], (uint32_t)((i >> 1) / kBandBars) & 1u))
+                if (ticks() - start > a.wait) break;
         __syncthreads();
         return;
     }
@@ -424,11 +437,8 @@ __global__ void __launch_bounds__(kSumThreads, 1) band_sum_kernel(SumArgs a) {
 
 }  // namespace
 
-extern int g_fault_skip_chunk;
-
 bool bands_fit(const DedispArgs& a) {
     if (!a.bands || !a.band_rows || a.length <= 0) return false;
-    if (!a.grouped && g_fault_skip_chunk >= 0) return false;  // a test hook of the direct kernel
     const int64_t need = (a.length + 2 * kBandWords - 1) / (2 * kBandWords);
     const int64_t least = std::min<int64_t>(need, kBandLeastTiles);
     for (const BandSegment& s : a.bands->segs) {
@@ -519,6 +529,8 @@ cudaError_t launch_bands(const DedispArgs& a, cudaStream_t s) {
             sa.pitch = a.out_pitch;
             sa.st_acc = a.st_acc ? a.st_acc + 3 * (int64_t)(d0 - a.trial0) : nullptr;
             sa.err = a.err;
+            sa.wait = (uint32_t)std::min<uint64_t>((g_wait_limit_ns + 1023) >> 10, UINT32_MAX);
+            sa.skip_band = g_fault_skip_chunk;
             // Half tiles take three quarters of a whole one's time (123 us against 167, a
             // wave of 512 bands): worth it where twice the CTAs take as many waves.
             const int64_t waves = (nt * nblk + sms - 1) / sms, half = (2 * nt * nblk + sms - 1) / sms;

@@ -368,6 +368,10 @@ int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials);
 // the delays [ndm][nchans] that the tables add up to, read back from them as
 // the kernels do; false if a table entry is inconsistent
 bool band_shifts(const BandPlan& bp, int nchans, int ndm, int32_t* out);
+// Limit of each device-side wait, and the test hook that leaves a staging copy
+// out (the direct kernel's channel chunk, the band sums' band; -1: none).
+extern uint64_t g_wait_limit_ns;
+extern int g_fault_skip_chunk;
 bool bands_fit(const DedispArgs& a);  // a row buffer is there and large enough
 // A launch that bands_fit takes is faster on band rows than on its strategy's
 // kernel, by the estimates of aa_band_plan.cpp.

@@ -3,6 +3,8 @@ last bands of 1 to 8 channels, parts of blocks and segments, one tile and
 several slabs, both halves of a word past the series end, and the least
 scratch, with which the grouped kernel runs instead.  Short outputs included:
 band rows run here wherever they fit, not only where they are the faster side."""
+import time
+
 import pytest
 import torch
 
@@ -35,7 +37,7 @@ def _run(plan, x, nsamp, ws_bytes):
     ws = torch.full((ws_bytes,), 0xA5, dtype=torch.uint8, device="cuda")  # the row buffer starts as garbage
     abi.aa_dedisperse_device(plan.handle, x.data_ptr(), nsamp, x.stride(0), out.data_ptr(), ws.data_ptr(), ws.numel(),
                              torch.cuda.current_stream().cuda_stream)
-    abi.aa_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert abi.aa_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream) == abi.AA_OK
     return out
 
 
@@ -61,6 +63,40 @@ def test_bands_equal_the_direct_kernel(case, data):
         got = _run(plan, x, n, nbytes)
         for a, b in zip(plan.range_views(got, n), plan.range_views(want, n)):
             assert torch.equal(a, b), nbytes
+
+
+@pytest.mark.parametrize("band", [0, 1, 34, 99])
+@pytest.mark.parametrize("length, ranges", [(700, ((0.0, 0.1, 70, 1),)), (40000, ((0.0, 0.1, 700, 1),)),
+                                            (1500, ((160.0, 2.0, 70, 16),))])
+def test_bounded_wait_reports_timeout(length, ranges, band):
+    """Copies of a band that are never issued make every CTA of the sums give up
+    after the wait limit without writing output (halves and whole tiles, two
+    pairs of bands a round and one); the next call is clean."""
+    plan = Plan(800, 1508.0, -0.375, 64e-6, ranges)
+    plan.bind()
+    nsamp = (length + int(plan.shifts(0).max())) * ranges[0][3]
+    x, n = plan.device_input(synth.noise_filterbank(800, nsamp, 3, device="cuda"))
+    plan.set_strategy(0, abi.AA_DEDISP_DIRECT)
+    want = _run(plan, x, n, plan.query(n).dedisp_ws_bytes)
+    plan.set_strategy(0, abi.AA_DEDISP_GROUPED)
+    nbytes = plan.query(n).dedisp_ws_bytes
+    assert nbytes > abi.aa_dedisperse_least_ws_bytes(plan.handle, n)
+    out, ws = torch.full_like(want, -1.0), plan.alloc_workspace(nbytes)
+    stream = torch.cuda.current_stream().cuda_stream
+    try:
+        abi.aa_debug_inject(2, 20_000_000)  # 20 ms
+        abi.aa_debug_inject(1, band)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        plan.dedisperse_device(x, n, out=out, ws=ws)
+        assert abi.aa_workspace_status(ws.data_ptr(), stream) == abi.AA_ERR_TIMEOUT
+        assert time.perf_counter() - t0 < 1.5  # six waves of CTAs at most, two limits each; the default limit is 2 s
+    finally:
+        abi.aa_debug_inject(0, 0)
+        abi.aa_debug_inject(4, 1)
+    assert torch.all(out == -1.0)
+    got = _run(plan, x, n, nbytes)
+    assert torch.equal(plan.range_views(got, n)[0], plan.range_views(want, n)[0])
 
 
 @pytest.mark.parametrize("stripe", [16, 64, 0])
