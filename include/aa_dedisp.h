@@ -400,7 +400,7 @@ aa_status aa_plan_autotune(aa_plan* plan, int64_t nsamp_probe, const char* cache
 /* Many independent beams (each with its own plan and length) searched by one
  * CUDA graph.  Beams are grouped into waves whose working set fits
  * wave_budget_bytes (<= 0: half of the free device memory) and waves reuse
- * one buffer region (beside it up to 8 row buffers of at most 384 MiB each and the
+ * one buffer region (beside it up to 8 row buffers, of at most 3 GiB and the
  * region's size in all, where memory allows); within a wave the graph issues each beam's kernels on 8
  * concurrent branches (see aa_batch_set_branches for the other form).
  * Plans are bound to the current device if needed; they must stay alive

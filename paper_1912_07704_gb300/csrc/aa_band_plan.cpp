@@ -370,7 +370,7 @@ void band_window(const BandSegment& s, int g0, int g1, int64_t& id, int64_t& pre
 }
 
 // bytes for ntiles tiles of the rows that any nblk blocks of a segment use
-static int64_t bytes_for(const BandPlan& bp, int64_t ntiles, int nblk) {
+static int64_t bytes_for(const BandPlan& bp, int64_t ntiles, int nblk, int64_t limit = kBandBytesMax) {
     int64_t most = 0;
     for (const BandSegment& s : bp.segs)
         for (int g = 0; g < s.nblk; ++g) {
@@ -378,8 +378,11 @@ static int64_t bytes_for(const BandPlan& bp, int64_t ntiles, int nblk) {
             band_window(s, g, std::min(s.nblk, g + nblk) - 1, id, pre, nrows, words);
             most = std::max(most, nrows * ntiles * kBandWords + words);
         }
-    return round_up(std::min(most * 4, kBandBytesMax), 256);
+    return round_up(std::min(most * 4, limit), 256);
 }
+
+// blocks of a stripe: one that does not begin with a block touches one more
+static int stripe_blocks(int32_t trials) { return std::max(1, trials / kBandTrials) + (trials % kBandTrials != 0); }
 
 int64_t band_bytes(const BandPlan& bp, int64_t length) {
     if (!bp.ok || length <= 0) return 0;
@@ -390,9 +393,13 @@ int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials) {
     if (!bp.ok || length <= 0) return 0;
     const int64_t nblk = std::max(1, trials / kBandTrials);
     const int64_t tiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
-    // a stripe that does not begin with a block touches one more
-    return bytes_for(bp, std::min<int64_t>(tiles, std::max<int64_t>(kBandLeastTiles, (2 * kBandSms + nblk - 1) / nblk)),
-                     (int)nblk + (trials % kBandTrials != 0));
+    return bytes_for(bp, std::min<int64_t>(tiles, std::max<int64_t>(kBandLeastTiles, (2 * kBandSms + nblk - 1) / nblk)), stripe_blocks(trials));
+}
+
+int64_t band_bytes_least(const BandPlan& bp, int64_t length, int32_t trials) {
+    if (!bp.ok || length <= 0) return 0;
+    const int64_t tiles = (length + 2 * kBandWords - 1) / (2 * kBandWords);
+    return bytes_for(bp, std::min<int64_t>(tiles, kBandLeastTiles), stripe_blocks(trials), INT64_MAX);
 }
 
 namespace {
@@ -459,7 +466,7 @@ bool bands_pay(const DedispArgs& a) {
 }
 
 bool bands_pay(const RangePlan& r, int nchans, int64_t length, int32_t trials, int64_t bytes) {
-    if (!r.bands.ok || length <= 0) return false;
+    if (!r.bands.ok || length <= 0 || bytes < band_bytes_least(r.bands, length, std::min(trials, r.desc.ndm))) return false;
     DedispArgs a{};
     a.nchans = nchans;
     a.ndm = std::min(trials, r.desc.ndm);

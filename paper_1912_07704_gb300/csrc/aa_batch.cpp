@@ -93,8 +93,9 @@ struct aa_batch {
     std::vector<std::vector<DedispArgs>> beam_dd;
     std::vector<std::vector<SpsArgs>> beam_sps;
     std::vector<char*> beam_dec_ws;
-    char* rows = nullptr;    // row buffers of the branches' band rows (branched form), shared out evenly
+    char* rows = nullptr;    // row buffers of the branches' band rows (branched form): share_rows
     int64_t rows_bytes = 0;
+    std::vector<int64_t> beam_rows;  // least row buffer of each beam's band rows (0: it has none)
     std::vector<double> beam_work;  // channel-adds + boxcar samples, for dealing beams to branches
 };
 
@@ -123,18 +124,48 @@ void free_batch(aa_batch* b) {
     delete b;
 }
 
+// The k-th largest beam_rows of a wave, over all waves, for k < n.
+std::vector<int64_t> most_rows(const aa_batch& b, int n) {
+    std::vector<int64_t> most((size_t)n, 0);
+    for (const auto& wave : b.waves) {
+        std::vector<int64_t> v;
+        for (int bi : wave) v.push_back(b.beam_rows[bi]);
+        std::sort(v.rbegin(), v.rend());
+        for (int k = 0; k < n && k < (int)v.size(); ++k) most[k] = std::max(most[k], v[k]);
+    }
+    return most;
+}
+
+// Row buffers, falling, of as many branches as there are beams to keep busy:
+// `total` shared out evenly but for the branches that the neediest beams want
+// more on; where it does not hold all of them, fewer branches have one.
+std::vector<int64_t> share_rows(const aa_batch& b, int branches, int64_t total) {
+    for (int n = std::min(branches, b.nbeams); n > 0; --n) {
+        std::vector<int64_t> v = most_rows(b, n);
+        int64_t left = total;
+        for (int k = 0; k < n && left >= 0; ++k) {
+            const int64_t even = left / (n - k) / 256 * 256;
+            if (v[k] <= even) {
+                std::fill(v.begin() + k, v.end(), even);
+                return v;
+            }
+            left -= v[k];
+        }
+    }
+    return {};
+}
+
 // One beam's stages as the single-beam path issues them: decimation cascade,
 // one dedispersion launch per range, then statistics and boxcar + peaks per
 // range.
-cudaError_t issue_beam(const aa_batch* b, int bi, int branch, cudaStream_t s) {
+cudaError_t issue_beam(const aa_batch* b, int bi, char* rows, int64_t rows_bytes, cudaStream_t s) {
     const aa_plan& pl = *b->plans[bi];
     const Layout L = make_layout(pl, b->nsamps[bi], b->max_width);
     const uint8_t* d_in = reinterpret_cast<const uint8_t*>(b->arena + b->in_offset[bi]);
     cudaError_t e = launch_decimation_cascade(pl, L, d_in, b->in_pitch[bi], b->beam_dec_ws[bi], s);
-    const int64_t per = b->rows_bytes / std::max(std::min(b->branches, b->nbeams), 1) / 256 * 256;  // beams are dealt to empty branches first
     for (DedispArgs a : b->beam_dd[bi]) {
-        a.band_rows = reinterpret_cast<uint32_t*>(b->rows + branch * per);
-        a.band_bytes = per;
+        a.band_rows = reinterpret_cast<uint32_t*>(rows);
+        a.band_bytes = rows_bytes;
         if (e == cudaSuccess) e = launch_dedisperse(a, s);
     }
     for (const SpsArgs& a : b->beam_sps[bi]) {
@@ -147,12 +178,16 @@ cudaError_t issue_beam(const aa_batch* b, int bi, int branch, cudaStream_t s) {
 // Records the whole batch (every wave) into b->graph / b->exec: either one
 // persistent work-queue kernel per stage and wave, or each beam's own
 // launches on b->branches concurrent branches (beams of a wave dealt to the
-// least-loaded branch, largest first; a wave starts when every branch of the
-// previous one has finished, since it reuses their buffers).
+// least-loaded branch whose row buffer they fit, largest first; a wave starts
+// when every branch of the previous one has finished, since it reuses their
+// buffers).
 cudaError_t capture_graph(aa_batch* b) {
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     const int nbr = b->branches;
+    const std::vector<int64_t> rows = share_rows(*b, nbr, b->rows_bytes);
+    std::vector<char*> rows_at(rows.size(), b->rows);
+    for (size_t k = 1; k < rows.size(); ++k) rows_at[k] = rows_at[k - 1] + rows[k - 1];
     cudaStream_t cs = nullptr;
     std::vector<cudaStream_t> bs((size_t)nbr, nullptr);
     std::vector<cudaEvent_t> ev((size_t)nbr + 1, nullptr);
@@ -189,7 +224,11 @@ cudaError_t capture_graph(aa_batch* b) {
             std::vector<std::vector<int>> lanes((size_t)nbr);
             std::vector<double> load((size_t)nbr, 0.0);
             for (int bi : order) {
-                const size_t k = std::min_element(load.begin(), load.end()) - load.begin();
+                // (without any row buffer every beam runs on the grouped and direct kernels)
+                const size_t most = b->beam_rows[bi] == 0 || rows.empty() ? (size_t)nbr : rows.size();
+                size_t k = 0;
+                for (size_t j = 1; j < most; ++j)
+                    if (load[j] < load[k] && (most == (size_t)nbr || rows[j] >= b->beam_rows[bi])) k = j;
                 lanes[k].push_back(bi);
                 load[k] += b->beam_work[bi];
             }
@@ -197,7 +236,7 @@ cudaError_t capture_graph(aa_batch* b) {
             for (int k = 0; k < nbr; ++k) {
                 if (lanes[k].empty()) continue;
                 chk(cudaStreamWaitEvent(bs[k], ev[nbr], 0));
-                for (int bi : lanes[k]) chk(issue_beam(b, bi, k, bs[k]));
+                for (int bi : lanes[k]) chk(issue_beam(b, bi, k < (int)rows.size() ? rows_at[k] : nullptr, k < (int)rows.size() ? rows[k] : 0, bs[k]));
                 chk(cudaEventRecord(ev[k], bs[k]));
                 chk(cudaStreamWaitEvent(cs, ev[k], 0));  // join
             }
@@ -312,21 +351,35 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
     const int64_t cand_bytes = round_up(cand_capacity * (int64_t)sizeof(aa_candidate), 256);
     const int64_t chunk_bytes = round_up(b->chunk_cap * (int64_t)sizeof(CandChunk), 256);
     const int64_t small_bytes = 256 + 256 + round_up((int64_t)b->wpad * 8, 256);
-    // row buffers: what keeps a branch's launches busy, kBranchRowsMax a branch
-    // and the waves' working set in all at most; without memory for them the
-    // beams run on the grouped and direct kernels
+    // row buffers: what keeps a branch's launches busy, kBranchRowsMax a branch,
+    // more where a beam's band rows do not run with less; kBranchRowsMax times
+    // the branches and the waves' working set in all at most.  Ranges that do not
+    // run with all of that, and every range where there is no memory for it, run
+    // on the grouped and direct kernels.
+    const int64_t used = std::min(kDefaultBranches, nbeams);
+    const int64_t most = std::min(kBranchRowsMax * kDefaultBranches, wave_bytes) / 256 * 256;
     int64_t rows = 0;
+    b->beam_rows.assign(nbeams, 0);
     for (int i = 0; i < nbeams; ++i) {
         const Layout L = make_layout(*plans[i], nsamps[i], max_width);
         for (size_t r = 0; r < plans[i]->ranges.size(); ++r) {
             const RangePlan& g = plans[i]->ranges[r];
             if (!uses_bands(g)) continue;
-            const int64_t busy = band_bytes_busy(g.bands, L.length[r], g.desc.ndm);
-            if (bands_pay(g, plans[i]->nchans, L.length[r], g.desc.ndm, busy)) rows = std::max(rows, busy);
+            const int64_t need = band_bytes_least(g.bands, L.length[r], g.desc.ndm);
+            if (need > most) continue;
+            const int64_t busy = std::max(need, band_bytes_busy(g.bands, L.length[r], g.desc.ndm));
+            if (!bands_pay(g, plans[i]->nchans, L.length[r], g.desc.ndm, std::min(busy, most))) continue;
+            rows = std::max(rows, busy);
+            b->beam_rows[i] = std::max(b->beam_rows[i], need);
         }
     }
-    const int64_t used = std::min(kDefaultBranches, nbeams);
-    rows = std::min({rows, kBranchRowsMax, wave_bytes / used / 256 * 256}) * used;
+    rows = std::min({rows, kBranchRowsMax, most / used / 256 * 256});
+    {
+        const std::vector<int64_t> v = most_rows(*b, (int)used);
+        int64_t sum = 0;
+        for (int64_t need : v) sum += std::max(rows, need);
+        rows = std::min(sum, most);
+    }
     const size_t least = (size_t)(in_bytes + wave_bytes + table_bytes + cand_bytes + chunk_bytes + small_bytes);
     b->arena_bytes = least + (size_t)rows;
     cudaError_t e = cudaMalloc(&b->arena, b->arena_bytes);

@@ -365,6 +365,8 @@ int64_t band_bytes(const BandPlan& bp, int64_t length);
 // bytes with which launches of `trials` trials keep the SMs busy: two CTAs
 // each, or the whole length where that is less
 int64_t band_bytes_busy(const BandPlan& bp, int64_t length, int32_t trials);
+// bytes without which bands_fit refuses launches of `trials` trials
+int64_t band_bytes_least(const BandPlan& bp, int64_t length, int32_t trials);
 // the delays [ndm][nchans] that the tables add up to, read back from them as
 // the kernels do; false if a table entry is inconsistent
 bool band_shifts(const BandPlan& bp, int nchans, int ndm, int32_t* out);
@@ -376,8 +378,8 @@ bool bands_fit(const DedispArgs& a);  // a row buffer is there and large enough
 // A launch that bands_fit takes is faster on band rows than on its strategy's
 // kernel, by the estimates of aa_band_plan.cpp.
 bool bands_pay(const DedispArgs& a);
-// The same for all trials of a range, or a stripe of so many, given a row
-// buffer of `bytes`: whether one is of use.
+// The same for all trials of a range, or stripes of so many, given a row buffer
+// of `bytes`: whether they run on band rows with it.
 bool bands_pay(const RangePlan& r, int nchans, int64_t length, int32_t trials, int64_t bytes);
 constexpr int kSmallDirect = 8;      // CTAs per SM up to which the direct strategy takes its small kernel ...
 constexpr int kSmallDirectTau = 128; // ... of one trial and this many samples a CTA

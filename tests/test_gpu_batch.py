@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1912_07704_gb300 import synth
+from paper_1912_07704_gb300 import abi, synth
 from paper_1912_07704_gb300.api import Batch, Plan, candidates_from_device
 
 pytestmark = pytest.mark.gpu
@@ -125,3 +125,49 @@ def test_autotune_keeps_results_and_caches(tmp_path, oracle):
     for a, b_, c in zip(p0.range_views(ref, nsamp), p1.range_views(out1, nsamp),
                         p2.range_views(out2, nsamp)):
         assert torch.equal(a, b_) and torch.equal(a, c)
+
+
+@pytest.mark.parametrize("step, nsamp", [(0.3, 100000), (1.0, 110000)])
+def test_row_buffers_hold_what_band_rows_take(step, nsamp):
+    """4096 channels whose rows take 0.8 GB at least: the branches that such
+    beams run on get that much, so that they run on band rows (a wait left to
+    run out by a copy that is never issued shows it: the grouped kernel has no
+    such copy); results are those of the beams alone, for any number of branches."""
+    wide = [(0.0, step, 1500, 1)]
+    specs = [(4096, wide, nsamp), (1024, [(0.0, 0.5, 100, 1), (50.0, 1.0, 64, 2)], 30000), (4096, wide, nsamp - 999), (256, [(0.0, 1.0, 40, 1)], 5000)]
+    plans = [Plan(C, 1508.0, -300.0 / C, 64e-6, ranges) for C, ranges, _ in specs]
+    for i in (0, 2):
+        plans[i].set_strategy(0, abi.AA_DEDISP_GROUPED)
+    xs = [synth.noise_filterbank(C, n, 8 + i, device="cuda") for i, (C, _, n) in enumerate(specs)]
+    cap, thr = 1 << 20, 5.5
+
+    def batch(which):
+        b = Batch([plans[i] for i in which], [specs[i][2] for i in which], 16, thr, capacity=cap)
+        for k, i in enumerate(which):
+            b.input_view(k)[:, : specs[i][2]].copy_(xs[i])
+        return b
+    try:
+        abi.aa_debug_inject(2, 2_000_000)  # 2 ms
+        abi.aa_debug_inject(1, 5)
+        b = batch([0, 2])
+        b.run()
+        with pytest.raises(abi.AAError, match="AA_ERR_TIMEOUT"):
+            b.candidates()
+        b.close()
+    finally:
+        abi.aa_debug_inject(0, 0)
+    alone = []
+    for p, x, (_, _, n) in zip(plans, xs, specs):
+        d, _ = p.device_input(x)
+        c, count, _ = p.sps_search_device(p.dedisperse_device(d, n), n, 16, thr, cap)
+        alone.append(candidates_from_device(c, count, cap))
+    assert sum(len(a) for a in alone) > 0
+    b = batch([0, 1, 2, 3])
+    for branches in (8, 1, 3, 64):
+        b.set_branches(branches)
+        b.run()
+        arr, total = b.candidates()
+        assert total == sum(len(a) for a in alone)
+        for a, want in zip(split(arr, 4), alone):
+            assert np.array_equal(a, want)
+    b.close()
