@@ -273,10 +273,9 @@ aa_status aa_workspace_status(void* d_ws, aa_stream_t stream);
  *     group sums.  Available when the plan could build the group tables.
  * Where they are estimated to be faster at the call's length (AA_DEDISP_GROUPED,
  * or the plan's own choice) and its scratch holds their row buffer, band rows
- * run instead: every
- * distinct sum of a band of consecutive channels is built once for many
+ * run instead: every distinct sum of a band of consecutive channels is built once for many
  * trials and each trial adds one per band.  aa_plan_set_strategy with
- * AA_DEDISP_DIRECT, and aa_plan_autotune choosing it, keep the direct kernel. */
+ * AA_DEDISP_DIRECT keeps the direct kernel. */
 typedef enum { AA_DEDISP_DIRECT = 0, AA_DEDISP_GROUPED = 1, AA_DEDISP_SUBBAND = 2,
                AA_DEDISP_FDMT = 3 } aa_dedisp_strategy;
 
@@ -388,7 +387,9 @@ aa_status aa_plan_set_sps_clip(aa_plan* plan, int32_t c16, int32_t max_iters);
 /* Time the dedispersion kernel of every range of a bound plan over a
  * synthetic probe input of nsamp_probe samples for the grouped strategy (if
  * available) and each feasible direct tile shape (channels per shared-memory
- * stage x staging depth) and keep the fastest in the plan's strategy.  Call before the plan's first dedispersion (the
+ * stage x staging depth) and keep the fastest in the plan's strategy (the
+ * kernel of launches that do not run on band rows; the choice of those is not
+ * tuned).  Call before the plan's first dedispersion (the
  * strategy is fixed from then on).  cache_path: optional text file; shapes
  * found there (keyed by GPU model, SM count, channels, decimation and the
  * staged row size) are applied without timing, new results are appended.

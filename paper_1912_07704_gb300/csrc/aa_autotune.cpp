@@ -2,7 +2,9 @@
 // the kernel over a synthetic probe input for the grouped strategy (when the
 // plan built its tables) and each feasible direct stage shape (channels per
 // shared-memory stage x pipeline depth), and keep the fastest.  Results can
-// be cached in a text file keyed by the GPU and the range's shape.
+// be cached in a text file keyed by the GPU and the range's shape.  What is
+// chosen is the kernel of calls that band rows do not run on; where they do is
+// decided launch by launch, whatever was tuned.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -26,7 +28,8 @@ std::string cache_key(const cudaDeviceProp& prop, const aa_plan& p, const RangeP
     std::ostringstream k;
     std::string name = prop.name;
     std::replace(name.begin(), name.end(), ' ', '_');
-    k << name << ";sm=" << prop.multiProcessorCount << ";C=" << p.nchans << ";dec=" << r.desc.dec
+    // v2: the strategies' own kernels (older lines may hold band rows under "grouped")
+    k << name << ";v2;sm=" << prop.multiProcessorCount << ";C=" << p.nchans << ";dec=" << r.desc.dec
       << ";rw=" << r.rw << ";ndm=" << std::min(r.desc.ndm, kDmPerBlock * 64)
       << ";dmstep=" << r.desc.dm_step << ";dmlo=" << r.desc.dm_lo;
     return k.str();
@@ -78,13 +81,6 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
     void* probe = nullptr;
     void* out = nullptr;
     unsigned* err = nullptr;
-    void* rows = nullptr;  // row buffer of the grouped strategy's bands; without it the grouped kernel is timed
-    int64_t row_bytes = 0;
-    for (size_t r = 0; r < p->ranges.size(); ++r) row_bytes = std::max(row_bytes, band_bytes(p->ranges[r].bands, L.length[r]));
-    if (row_bytes > 0 && cudaMalloc(&rows, (size_t)row_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        rows = nullptr;
-    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     aa_status status = AA_OK;
     if (cudaMalloc(&probe, bytes) != cudaSuccess || cudaMalloc(&out, std::max<size_t>(out_bytes, 256)) != cudaSuccess ||
@@ -138,9 +134,7 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
                     g.strategy = grouped ? 1 : 0;
                     fill_strategy(a, g);
                     g.strategy = saved;
-                    if (!grouped) a.bands = nullptr;
-                    a.band_rows = static_cast<uint32_t*>(rows);
-                    a.band_bytes = rows ? row_bytes : 0;
+                    a.bands = nullptr;
                     if (!grouped) {
                         a.cc = cc;
                         a.nstage = ns;
@@ -170,7 +164,7 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
             new_lines.push_back(line.str());
         }
         g.strategy = best_strategy;
-        g.pinned = true;
+        g.pinned = false;
         g.cc = best_cc;
         g.nstage = best_ns;
         g.flush = (std::min(65535 / (255 * g.desc.dec), 256) / best_cc) * best_cc;
@@ -181,7 +175,6 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
     if (probe) cudaFree(probe);
     if (out) cudaFree(out);
     if (err) cudaFree(err);
-    if (rows) cudaFree(rows);
     if (status == AA_OK && cache_path && !new_lines.empty()) {
         std::ofstream f(cache_path, std::ios::app);
         for (auto& l : new_lines) f << l << "\n";

@@ -202,7 +202,7 @@ struct RangePlan {
     SubbandPlan sb;        // valid once aa_plan_set_subband chose it (strategy 2)
     FdmtPlan fd;           // valid once aa_plan_set_fdmt chose it (strategy 3)
     BandPlan bands;        // band rows (ok: tables exist and pay)
-    bool pinned = false;   // the strategy was set or tuned, not the plan's own choice
+    bool pinned = false;   // the strategy was set, not the plan's or the tuner's choice
 };
 
 }  // namespace aa

@@ -127,6 +127,35 @@ def test_autotune_keeps_results_and_caches(tmp_path, oracle):
         assert torch.equal(a, b_) and torch.equal(a, c)
 
 
+@pytest.mark.parametrize("C, step, trials, kernel", [(256, 1.0, 256, abi.AA_DEDISP_DIRECT),      # hardly a shared delay pattern
+                                                     (1024, 0.1, 300, abi.AA_DEDISP_GROUPED)])
+def test_autotune_leaves_band_rows_to_the_launch(tmp_path, C, step, trials, kernel):
+    """The tuner chooses among the strategies' own kernels (at DM step 1 over
+    256 channels the grouped one is the slower), and neither its choice nor a
+    cached "direct" takes band rows from the plan."""
+    make = lambda: Plan(C, 1508.0, -300.0 / C, 64e-6, [(0.0, step, trials, 1)])
+    n, cache = 40000, tmp_path / "tune.txt"
+    p = make()
+    least = abi.aa_dedisperse_least_ws_bytes(p.handle, n)
+    assert p.query(n).dedisp_ws_bytes > least
+    p.autotune(n, str(cache))
+    assert abi.aa_plan_range(p.handle, n, 0).strategy == kernel
+    assert p.query(n).dedisp_ws_bytes > least
+    p.close()
+    key, _, cc, ns, ms = cache.read_text().split()
+    cache.write_text(f"{key} {abi.AA_DEDISP_DIRECT} 8 2 {ms}\n")
+    p = make()
+    p.autotune(n, str(cache))
+    assert abi.aa_plan_range(p.handle, n, 0).strategy == abi.AA_DEDISP_DIRECT  # served from the cache
+    assert p.query(n).dedisp_ws_bytes > least
+    p.close()
+    cache.write_text(f"{key.replace(';v2', '')} {abi.AA_DEDISP_DIRECT} 8 2 {ms}\n")  # a line of an older library
+    p = make()
+    p.autotune(n, str(cache))
+    assert len(cache.read_text().splitlines()) == 2  # timed again
+    p.close()
+
+
 @pytest.mark.parametrize("step, nsamp", [(0.3, 100000), (1.0, 110000)])
 def test_row_buffers_hold_what_band_rows_take(step, nsamp):
     """4096 channels whose rows take 0.8 GB at least: the branches that such
