@@ -135,6 +135,7 @@ extern "C" aa_status aa_plan_autotune(aa_plan* p, int64_t nsamp_probe, const cha
                     fill_strategy(a, g);
                     g.strategy = saved;
                     a.bands = nullptr;
+                    a.staged = 1;  // (short probes too: the small kernel has no shape)
                     if (!grouped) {
                         a.cc = cc;
                         a.nstage = ns;

@@ -992,7 +992,7 @@ cudaError_t launch_dedisperse(const DedispArgs& a, cudaStream_t s) {
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 0;
     const int64_t small = (a.length + kSmallTau - 1) / kSmallTau * a.ndm;
-    if (small <= kSmallDirect * (int64_t)sms && !a.out16 && g_fault_skip_chunk < 0) {
+    if (small <= kSmallDirect * (int64_t)sms && !a.staged && !a.out16 && g_fault_skip_chunk < 0) {
         auto kern = a.elem == 1 ? dedisperse_small_kernel<4> : dedisperse_small_kernel<2>;
         kern<<<(unsigned)small, kSmallWarps * 32, 0, s>>>(a, (int)(small / a.ndm));
         return cudaGetLastError();

@@ -352,6 +352,7 @@ struct DedispArgs {
     // row_dec samples as it reads it; only for launches that bands_fit takes
     int32_t row_dec;
     double gwork;  // adds of the grouped strategy / adds of the direct one
+    int32_t staged;  // the direct strategy's staged kernel (cc, nstage) also where its small one would run
 };
 // Given a row buffer, a range runs on band rows where it has them, unless the
 // direct strategy was asked for.

@@ -156,6 +156,27 @@ def test_autotune_leaves_band_rows_to_the_launch(tmp_path, C, step, trials, kern
     p.close()
 
 
+def test_autotune_times_the_shapes_on_a_short_probe(tmp_path):
+    """Calls of a few blocks run on a kernel without shapes; the tuner times the
+    staged one all the same (there about three times the small one's time)."""
+    p = Plan(1024, 1508.0, -300.0 / 1024, 64e-6, [(0.0, 5.0, 20, 1)])
+    x, n = p.device_input(synth.noise_filterbank(1024, 6000 + int(p.shifts(0).max()), 4, device="cuda"))
+    p.set_strategy(0, abi.AA_DEDISP_DIRECT)
+    out, ws = p.alloc_output(n), p.alloc_workspace(p.query(n).dedisp_ws_bytes)
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    for _ in range(2):
+        e[0].record()
+        for _ in range(20):
+            p.dedisperse_device(x, n, out=out, ws=ws)
+        e[1].record()
+        torch.cuda.synchronize()
+    small_ms = e[0].elapsed_time(e[1]) / 20
+    p.autotune(n, str(tmp_path / "tune.txt"))
+    line = (tmp_path / "tune.txt").read_text().split()
+    assert int(line[1]) == abi.AA_DEDISP_DIRECT and float(line[4]) > 1.5 * small_ms
+    p.close()
+
+
 @pytest.mark.parametrize("step, nsamp", [(0.3, 100000), (1.0, 110000)])
 def test_row_buffers_hold_what_band_rows_take(step, nsamp):
     """4096 channels whose rows take 0.8 GB at least: the branches that such
