@@ -215,7 +215,7 @@ cudaError_t capture_graph(aa_batch* b) {
                 chk(launch_sps_stats_batch(T.d_sps, T.d_st_first, (int)T.sps.size(), &T.d_queues[4],
                                            b->grid_st, cs));
                 chk(launch_sps_boxcar_batch(T.d_sps, T.d_bx_first, T.d_bx_ntiles, (int)T.sps.size(), T.bx_smem,
-                                            &T.d_queues[5], b->grid_bx, cs));
+                                            !T.sps.empty() && sps_low(T.sps[0]), &T.d_queues[5], b->grid_bx, cs));
                 continue;
             }
             std::vector<int> order(b->waves[wi]);

@@ -454,11 +454,13 @@ cudaError_t launch_sps_stats(const SpsArgs& a, cudaStream_t s);
 // mu, sigma and width tables of a.nrows rows from the sums the dedispersion
 // kernels accumulated (DedispArgs::st_acc; 3 words per row)
 cudaError_t launch_sps_finalize(const SpsArgs& a, const unsigned long long* acc, cudaStream_t s);
+// B below zero counts: B(t) asked for, or a threshold not above zero
+inline bool sps_low(const SpsArgs& a) { return !(a.prune && a.threshold > 0.0f); }
 cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s);
 cudaError_t launch_sps_stats_batch(const SpsArgs* d_descs, const int64_t* d_first, int ndesc,
                                    unsigned long long* d_queue, int grid, cudaStream_t s);
 cudaError_t launch_sps_boxcar_batch(const SpsArgs* d_descs, const int64_t* d_first,
-                                    const int* d_ntiles, int ndesc, size_t smem,
+                                    const int* d_ntiles, int ndesc, size_t smem, bool low,
                                     unsigned long long* d_queue, int grid, cudaStream_t s);
 int sps_boxcar_tiles(int64_t length);
 size_t sps_boxcar_smem(int wpad);

@@ -1142,8 +1142,7 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
 
 // CTA = seg_tiles consecutive tiles of one series (the last segment of a
 // series may be shorter).
-// LOW: B below zero counts (B(t) asked for, or a threshold not above zero).
-__host__ __device__ inline bool sps_low(const SpsArgs& a) { return !(a.prune && a.threshold > 0.0f); }
+// LOW: sps_low.
 template <bool LOW>
 __global__ void __launch_bounds__(NT, 2) sps_boxcar_kernel(SpsArgs a, int ntiles, int seg_tiles) {
     extern __shared__ __align__(16) float sm[];
@@ -1540,6 +1539,7 @@ __global__ void __launch_bounds__(kStatsThreads) sps_stats_batch_kernel(
     }
 }
 
+template <bool LOW>
 __global__ void __launch_bounds__(NT, 2) sps_boxcar_batch_kernel(
     const SpsArgs* __restrict__ descs, const int64_t* __restrict__ first,
     const int* __restrict__ ntiles, int ndesc, unsigned long long* queue) {
@@ -1559,7 +1559,7 @@ __global__ void __launch_bounds__(NT, 2) sps_boxcar_batch_kernel(
         } else {
             const int row = (int)(bid / ntiles[k]);
             const int64_t tile = bid - (int64_t)row * ntiles[k];
-            boxcar_block<true>(descs[k], row, tile, tile + 1, sm);
+            boxcar_block<LOW>(descs[k], row, tile, tile + 1, sm);
         }
     }
 }
@@ -1667,12 +1667,13 @@ cudaError_t launch_sps_stats_batch(const SpsArgs* d_descs, const int64_t* d_firs
 
 cudaError_t launch_sps_boxcar_batch(const SpsArgs* d_descs, const int64_t* d_first,
                                     const int* d_ntiles, int ndesc, size_t smem,
-                                    unsigned long long* d_queue, int grid, cudaStream_t s) {
+                                    bool low, unsigned long long* d_queue, int grid, cudaStream_t s) {
     if (ndesc <= 0) return cudaSuccess;
     if (smem > kMaxBoxcarSmem) return cudaErrorInvalidConfiguration;
-    cudaError_t e = allow_smem((const void*)sps_boxcar_batch_kernel);
+    auto kern = low ? sps_boxcar_batch_kernel<true> : sps_boxcar_batch_kernel<false>;
+    cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
-    sps_boxcar_batch_kernel<<<grid, NT, smem, s>>>(d_descs, d_first, d_ntiles, ndesc, d_queue);
+    kern<<<grid, NT, smem, s>>>(d_descs, d_first, d_ntiles, ndesc, d_queue);
     return cudaGetLastError();
 }
 

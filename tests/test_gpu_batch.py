@@ -127,6 +127,34 @@ def test_autotune_keeps_results_and_caches(tmp_path, oracle):
         assert torch.equal(a, b_) and torch.equal(a, c)
 
 
+@pytest.mark.parametrize("thr", [6.0, -0.25])
+def test_persistent_search_prunes(thr):
+    """The work-queue form's search skips widths by bounds as the branches' does
+    (with every width evaluated noise took it four times their time), and below
+    a threshold of zero finds what they find."""
+    plans = [Plan(64, 1508.0, -300.0 / 64, 64e-6, [(0.0, 1.0, 64, 1)]) for _ in range(4)]
+    xs = [synth.noise_filterbank(64, 30000 + 999 * i, 3 + i, device="cuda") for i in range(4)]
+    b = Batch(plans, [x.shape[1] for x in xs], 1024, thr, capacity=1 << 22)
+    for i, x in enumerate(xs):
+        b.input_view(i)[:, : x.shape[1]].copy_(x)
+    ms, found = {}, {}
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    for branches in (8, 0):
+        b.set_branches(branches)
+        b.run()
+        e[0].record()
+        for _ in range(5):
+            b.run()
+        e[1].record()
+        torch.cuda.synchronize()
+        ms[branches] = e[0].elapsed_time(e[1]) / 5
+        found[branches] = b.candidates()
+    assert found[0][1] == found[8][1] and np.array_equal(found[0][0], found[8][0])
+    assert thr < 0 or ms[0] < 2 * ms[8], ms
+    assert thr > 0 or found[0][1] > 0
+    b.close()
+
+
 @pytest.mark.parametrize("C, step, trials, kernel", [(256, 1.0, 256, abi.AA_DEDISP_DIRECT),      # hardly a shared delay pattern
                                                      (1024, 0.1, 300, abi.AA_DEDISP_GROUPED)])
 def test_autotune_leaves_band_rows_to_the_launch(tmp_path, C, step, trials, kernel):
