@@ -526,6 +526,7 @@ aa_status aa_batch_create(aa_plan* const* plans, const int64_t* nsamps, int32_t 
                 s.clip_iters = pl.clip_iters;
                 s.ladder_g16 = pl.ladder_g16;
                 s.dec_w0 = pl.dec_w0;
+                s.every = kSpsEvery;  // of the persistent kernel
                 T.bx_smem = std::max(T.bx_smem, sps_boxcar_smem_for(s.max_width, s.wpad, s.dec_w0));
                 s.beam = bi;
                 s.chunks = b->d_chunks;

@@ -28,6 +28,8 @@ constexpr int kDedispThreads = kDedispWarps * 32;
 constexpr int kSpsThreads = 256;
 constexpr int kSpsSlots = 16;
 constexpr int kSpsTile = kSpsThreads * kSpsSlots;  // start times per CTA incl. 2 halo
+constexpr int kSpsEvery = 64;        // chunks of 16 widths evaluated in turn where B(t) is asked for ...
+constexpr int kSpsEveryMost = 128;   // ... and where CTAs are few
 constexpr int kSpsOwned = kSpsTile - 2;              // start times owned per CTA
 
 // Grouped strategy.  Within one (DM block, channel chunk), channels whose
@@ -444,6 +446,7 @@ struct SpsArgs {
     int32_t clip_iters;     // clipping passes (0: plain statistics)
     int32_t ladder_g16;     // sparse width ladder growth x16 (0: every width)
     int32_t dec_w0;         // decimated width ladder base widths (0: off)
+    int32_t every;          // chunks up to which a search without a threshold evaluates every width (set by the launch)
     int32_t beam;           // beam id stored in candidate records (batched mode)
     unsigned long long* evaluated;  // width-samples actually evaluated (instrumentation)
     CandChunk* chunks;      // chunk headers (all ranges)

@@ -422,8 +422,12 @@ constexpr float kBig = 1.2676506002282294e30f;  // 2^100
 // further step is within 2^-22 relative of |num| or of the drift |w f|
 // (|f| <= 1/2 since m0 = round(mu)); the factor 1 + 1.02e-4 in rs and the
 // margin S (1.02e-4 and the largest drift's part) bound them many times over.
-constexpr int kTabWidths = 1024;  // widths whose table entries are staged in shared memory
-__host__ __device__ constexpr int sps_tab_smem(int wpad) { return wpad < kTabWidths ? wpad : kTabWidths; }
+// Widths whose table entries are staged in shared memory: all of them where they
+// may be evaluated in turn (low), else the first 1024.
+constexpr int kTabWidths = 1024;
+__host__ __device__ constexpr int sps_tab_smem(int wpad, bool low) {
+    return wpad < kTabWidths || (low && wpad <= kSpsEveryMost * M) ? wpad : kTabWidths;
+}
 // entries of Q16 and of each sliding maximum (the end padded for the longest)
 __host__ __device__ constexpr int sps_q16(int wpad) { return (kSpsTile / M + wpad / M + 1 + 64 + 31) / 32 * 32; }
 // entries of rs: c <= the last chunk + 65, and what a pass reads as it begins
@@ -510,21 +514,17 @@ __device__ __forceinline__ bool chunk0_reaches(const float* __restrict__ pb, con
     return any | reach(8, 15, 0.35355339f);
 }
 
-// Without a threshold up to kEvery chunks are simply evaluated in turn: noise
-// leaves over a third of them to evaluate and the bounds cost more (B(t) of
-// 96 series of 64006 samples, W = 256 / 1024 / 2048: in turn 220 / 752 / 1449
-// us, by bounds 307 / 802 / 1084).
-constexpr int kEvery = kTabWidths / M;
 constexpr unsigned kQueue = 8;
 // Returns the chunks this thread evaluated.  C: the first chunk reaching B[i] in
 // 16-bit halves, starts 2 k and 2 k + 1 in C[k] (16 registers of them spilled).
 // Q: Q16, S1, S8 and S64, nq entries each.  queue: the thread's entries, kQueue of them NT apart.
-// LOW: cut is not above zero.
+// LOW: cut is not above zero; up to `every` chunks are simply evaluated in turn
+// then.
 template <bool LOW>
 __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const float4* tab, const float2* __restrict__ gtab,
                                              int nch, int max_width, const float (&base)[M], const WidthBounds& bnd,
                                              const float* Q, int nq, uint16_t* queue, float cut, const uint32_t* lmask,
-                                             float (&B)[M], uint32_t (&C)[M / 2]) {
+                                             int every, float (&B)[M], uint32_t (&C)[M / 2]) {
     const int t = threadIdx.x;
     const float* pb = P + M * t;
 #pragma unroll
@@ -532,7 +532,7 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
         B[i] = -FLT_MAX;
         C[i / 2] = 0;
     }
-    if (LOW && nch <= kEvery) {
+    if (LOW && nch <= every) {
         for (int c = 0; c < nch; ++c) {
             if (lmask && !ladder_has(lmask, M * c + 1)) continue;
             float Bc[M];
@@ -577,7 +577,7 @@ __device__ __forceinline__ int boxcar_search(const float* __restrict__ P, const 
             __syncwarp();
             if (pend >= 0) {
                 float Bc[M];
-                const bool staged = M * pend < kTabWidths;
+                const bool staged = M * pend < kTabWidths || (LOW && nch <= kSpsEveryMost);
                 eval_chunk(pb + M * pend, staged ? tab + 8 * pend : reinterpret_cast<const float4*>(gtab) + 8 * pend,
                            staged ? pend & 7 : 0, base, Bc);
                 float low = FLT_MAX;  // smallest B over the valid starts (none: the floor is above every bound)
@@ -774,7 +774,7 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
     const int wpad = a.wpad;
     const int ylen = kSpsTile + wpad + M;
     float* ys = sm;
-    const int wtab = sps_tab_smem(wpad);
+    const int wtab = sps_tab_smem(wpad, LOW);
     float4* tab = reinterpret_cast<float4*>(sm + ylen);
     float* lists = sm + ylen + 2 * wtab;
     float* Q = lists;  // block maxima and their sliding maxima, nq each
@@ -971,7 +971,7 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
             bnd.pmin = pmin;
             bnd.pmax = pmax;
             __syncthreads();
-            const bool bounds = wpad > M && !(LOW && wpad <= kEvery * M);  // boxcar_search looks at them
+            const bool bounds = wpad > M && !(LOW && wpad <= a.every * M);  // boxcar_search looks at them
             if (bounds) {
                 for (int j = threadIdx.x; j < nq; j += NT) {
                     const float a1 = fmaxf(Q[j], j + 1 < nq ? Q[j + 1] : -kBig);
@@ -995,7 +995,7 @@ __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t 
                 __syncthreads();
             }
             int chunks = boxcar_search<LOW>(P, tab, gtab, wpad / M, a.max_width, base, bnd, Q, nq,
-                                            reinterpret_cast<uint16_t*>(Q + 4 * nq) + threadIdx.x, cut, lmask, B, C);
+                                            reinterpret_cast<uint16_t*>(Q + 4 * nq) + threadIdx.x, cut, lmask, a.every, B, C);
             if (a.evaluated) {
                 chunks = __reduce_add_sync(0xffffffffu, chunks);
                 if (lane == 0) atomicAdd(a.evaluated, (unsigned long long)chunks * M * M);
@@ -1608,7 +1608,7 @@ cudaError_t launch_rsqrt_table(double* t, int wpad, cudaStream_t s) {
 
 size_t sps_boxcar_smem(int wpad) {
     const int ylen = kSpsTile + wpad + M;
-    return ((size_t)ylen + 2 * sps_tab_smem(wpad) + sps_lists_words(wpad) + kSpsTile + sps_rs(wpad) + ladder_words(wpad)) * 4;
+    return ((size_t)ylen + 2 * sps_tab_smem(wpad, true) + sps_lists_words(wpad) + kSpsTile + sps_rs(wpad) + ladder_words(wpad)) * 4;
 }
 
 int g_boxcar_seg_tiles = 0;
@@ -1646,10 +1646,22 @@ cudaError_t launch_sps_boxcar(const SpsArgs& a, cudaStream_t s) {
                         ? (int)std::min<int64_t>(g_boxcar_seg_tiles, ntiles)
                         : (int)std::max<int64_t>(1, std::min<int64_t>({16, ntiles, nblocks / (sms * 2 * 16)}));
     const int64_t ncta = (int64_t)a.nrows * ((ntiles + seg - 1) / seg);
+    // Chunks up to which B(t) of every start is found by evaluating all widths in
+    // turn: noise leaves over a third of them to evaluate and the bounds cost more
+    // (96 series of 64006 samples, W = 256 / 1024 / 2048: in turn 220 / 752 / 1449
+    // us, by bounds 307 / 802 / 1084).  With one CTA an SM or fewer the bounds'
+    // chain of steps is what takes the time, and in noise more widths are faster
+    // in turn (4 series of 40000 samples, W = 1100 / 2048: in turn 98 / 164 us, by
+    // bounds 150 / 191; with two CTAs an SM, 96 series of 12000, W = 1100: 163 and
+    // 185), short series apart, most of whose windows do not exist (16 of 3000,
+    // W = 2048: 157 both, with a pulse 161 and 45).
+    SpsArgs b = a;
+    const bool whole = a.length >= kSpsTile + a.max_width;
+    b.every = ncta > (whole ? 2 * sms : sms) ? kSpsEvery : ncta > sms ? kSpsEvery * 5 / 4 : whole ? kSpsEveryMost : kSpsEvery * 3 / 2;
     auto kern = sps_low(a) ? sps_boxcar_kernel<true> : sps_boxcar_kernel<false>;
     cudaError_t e = allow_smem((const void*)kern);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)ncta, NT, smem, s>>>(a, (int)ntiles, seg);
+    kern<<<(unsigned)ncta, NT, smem, s>>>(b, (int)ntiles, seg);
     return cudaGetLastError();
 }
 

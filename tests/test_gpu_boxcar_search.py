@@ -1,5 +1,6 @@
 """The boxcar search's pruning, at the widths where its groups of chunks begin
-and end (16, 128, 1024, 8192 widths and one more or less): the B(t) map equals
+and end (16, 128, 1024, 8192 widths and one more or less) and where the map's
+widths cease to be evaluated in turn (2048 for so few series): the B(t) map equals
 the maximum over every width in 64 bits, and the pruned search (no map) finds
 exactly the peaks of the map, for a usual threshold and one below zero."""
 import math
@@ -47,7 +48,7 @@ def _best(y, W):
     return best
 
 
-@pytest.mark.parametrize("W", [1, 16, 17, 127, 129, 1024, 1025, 4100, 8191, 8193, 9000])
+@pytest.mark.parametrize("W", [1, 16, 17, 127, 129, 1024, 1025, 2048, 2049, 4100, 8191, 8193, 9000])
 @pytest.mark.parametrize("kind", ["noise", "pulses", "ramp", "flat"])
 def test_pruned_search_equals_the_map(W, kind):
     plan = Plan(16, 1400.0, -1.0, 64e-6, [(0.0, 0.0, ROWS, 1)])
