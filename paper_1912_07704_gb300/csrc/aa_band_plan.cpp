@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <new>
 #include <utility>
 
 #include "aa_internal.h"
@@ -340,8 +341,7 @@ bool band_shifts(const BandPlan& bp, int C, int ndm, int32_t* out) {
     return true;
 }
 
-void build_bands(RangePlan& r, int C) {
-    r.bands = BandPlan{};
+static void choose_bands(RangePlan& r, int C) {
     if (C > 65535 || r.desc.ndm < kBandTrials / 2) return;
     // SM cycles per 512 output samples of the direct kernel: 64 trials of one
     // channel take 991 (10.4e12 adds/s on 152 SMs at 2.07 GHz, measured).
@@ -360,6 +360,15 @@ void build_bands(RangePlan& r, int C) {
         if (shared) break;
     }
     if (best.ok && best.cost < 0.6 * direct) r.bands = std::move(best);
+}
+
+void build_bands(RangePlan& r, int C) {
+    r.bands = BandPlan{};
+    try {
+        choose_bands(r, C);
+    } catch (const std::bad_alloc&) {  // the plan works without them
+        r.bands = BandPlan{};
+    }
 }
 
 void band_window(const BandSegment& s, int g0, int g1, int64_t& id, int64_t& pre, int64_t& nrows, int64_t& words) {

@@ -610,13 +610,13 @@ aa_status aa_plan_create(const aa_plan_desc* d, aa_plan** out) {
             p->ranges.push_back(std::move(rp));
         }
         p->ndm_total = off;
+        const aa_status st = build_strategy(*p);
+        if (st != AA_OK) { delete p; return st; }
     } catch (const std::bad_alloc&) {
         delete p;
         set_error("host allocation failed");
         return AA_ERR_NOMEM;
     }
-    aa_status st = build_strategy(*p);
-    if (st != AA_OK) { delete p; return st; }
     for (auto& r : p->ranges) {
         p->table_bytes += round_up((int64_t)r.shifts.size() * 4, 256);
         p->table_bytes += round_up((int64_t)r.grec.size() * sizeof(GroupRec), 256);
@@ -929,10 +929,7 @@ aa_status aa_plan_set_subband(aa_plan* p, int32_t r, int32_t band_channels, int3
     return AA_OK;
 }
 
-aa_status aa_plan_set_fdmt(aa_plan* p, int32_t r) {
-    clear_error();
-    if (!p) { set_error("plan is NULL"); return AA_ERR_ARG; }
-    if (r < 0 || r >= (int32_t)p->ranges.size()) { set_error("range %d out of bounds", r); return AA_ERR_ARG; }
+static aa_status set_fdmt(aa_plan* p, int32_t r) {
     RangePlan& g = p->ranges[r];
     const int32_t C = p->nchans, ndm = g.desc.ndm;
     if (C < 2) { set_error("the FDMT tree needs at least two channels"); return AA_ERR_CONFIG; }
@@ -1064,6 +1061,18 @@ aa_status aa_plan_set_fdmt(aa_plan* p, int32_t r) {
     return AA_OK;
 }
 
+aa_status aa_plan_set_fdmt(aa_plan* p, int32_t r) {
+    clear_error();
+    if (!p) { set_error("plan is NULL"); return AA_ERR_ARG; }
+    if (r < 0 || r >= (int32_t)p->ranges.size()) { set_error("range %d out of bounds", r); return AA_ERR_ARG; }
+    try {
+        return set_fdmt(p, r);
+    } catch (const std::bad_alloc&) {  // before the range has changed
+        set_error("host allocation failed");
+        return AA_ERR_NOMEM;
+    }
+}
+
 aa_status aa_plan_effective_shifts(const aa_plan* p, int32_t r, int32_t* out, int64_t cap) {
     clear_error();
     if (!p || !out) { set_error("plan/out is NULL"); return AA_ERR_ARG; }
@@ -1085,15 +1094,20 @@ aa_status aa_plan_effective_shifts(const aa_plan* p, int32_t r, int32_t* out, in
         }
         return AA_OK;
     }
-    if (g.strategy == 3) {
-        if (ndm == 0 || fdmt_shifts(g.fd, C, ndm, out)) return AA_OK;
-        set_error("internal: inconsistent FDMT tables");
-        return AA_ERR_STATE;
-    }
-    if (uses_bands(g)) {
-        if (band_shifts(g.bands, C, ndm, out)) return AA_OK;
-        set_error("internal: inconsistent band tables");
-        return AA_ERR_STATE;
+    try {
+        if (g.strategy == 3) {
+            if (ndm == 0 || fdmt_shifts(g.fd, C, ndm, out)) return AA_OK;
+            set_error("internal: inconsistent FDMT tables");
+            return AA_ERR_STATE;
+        }
+        if (uses_bands(g)) {
+            if (band_shifts(g.bands, C, ndm, out)) return AA_OK;
+            set_error("internal: inconsistent band tables");
+            return AA_ERR_STATE;
+        }
+    } catch (const std::bad_alloc&) {
+        set_error("host allocation failed");
+        return AA_ERR_NOMEM;
     }
     std::memcpy(out, g.shifts.data(), g.shifts.size() * 4);
     return AA_OK;
