@@ -274,7 +274,7 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
         return AA_ERR_NOMEM;
     }
     // the slots' row buffers when the budget has room for all of them
-    s->ws_bytes = (size_t)(avail - nslots * slot_bytes >= nslots * (full - least) ? full : least);
+    const size_t ws_bytes = (size_t)(avail - nslots * slot_bytes >= nslots * (full - least) ? full : least);
     s->beams.resize(nbeams);
     for (auto& b : s->beams) {
         cudaError_t e = cudaMalloc(&b.buf[0], (size_t)plan->nchans * s->pitch);
@@ -286,10 +286,7 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
     for (auto& sl : s->slots) {
         cudaError_t e = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
-        if (s->fused) {  // one fused workspace per slot
-            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, std::max<size_t>(s->ws_bytes, 256));
-        } else {
-            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, s->ws_bytes);
+        if (!s->fused) {  // (one workspace per slot, dd_ws, where the search is fused)
             if (e == cudaSuccess) e = cudaMalloc(&sl.dd, (size_t)std::max<int64_t>(L.dd_elems * 4, 256));
             if (e == cudaSuccess) e = cudaMalloc(&sl.sps_ws, (size_t)L.sps_ws);
         }
@@ -298,6 +295,25 @@ aa_status aa_server_create(aa_plan* plan, int32_t nbeams, int64_t chunk_nsamp, i
         if (e == cudaSuccess) e = cudaMallocHost(&sl.h_count, 64);
         if (e != cudaSuccess) { free_server(s); return fail(e, "slot allocation"); }
     }
+    // last, with the row buffers where there is memory for all of them
+    auto workspaces = [&](size_t bytes) {
+        s->ws_bytes = bytes;
+        cudaError_t e = cudaSuccess;
+        for (auto& sl : s->slots)
+            if (e == cudaSuccess) e = cudaMalloc(&sl.dd_ws, std::max<size_t>(bytes, 256));
+        if (e == cudaSuccess) return e;
+        for (auto& sl : s->slots) {
+            cudaFree(sl.dd_ws);
+            sl.dd_ws = nullptr;
+        }
+        return e;
+    };
+    cudaError_t e = workspaces(ws_bytes);
+    if (e != cudaSuccess && (int64_t)ws_bytes > least) {
+        cudaGetLastError();
+        e = workspaces((size_t)least);
+    }
+    if (e != cudaSuccess) { free_server(s); return fail(e, "slot workspaces"); }
     *out = s;
     return AA_OK;
 }

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 from gpu_common import compare_candidate_lists
-from paper_1912_07704_gb300 import synth
+from paper_1912_07704_gb300 import abi, synth
 from paper_1912_07704_gb300.api import Plan, Server
 
 pytestmark = pytest.mark.gpu
@@ -97,3 +97,36 @@ def test_chunks_match_oracle_on_blocks(oracle, streams):
                 sel["reserved"] = 0
                 compared += compare_candidate_lists(sel, solid, fragile)
     assert compared > 0
+
+
+def test_slots_without_memory_for_row_buffers():
+    """A budget may be larger than the memory that is free: where the slots'
+    row buffers do not fit, the slots are made without them."""
+    plan = Plan(1024, 1508.0, -300.0 / 1024, 64e-6, [(0.0, 0.1, 600, 1)])
+    chunk = synth.noise_filterbank(1024, 1 << 16, seed=6).numpy()
+    plan.bind()
+    slots = 8
+
+    def serve():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        srv = Server(plan, 2, 1 << 16, 64, 4.5, capacity=1 << 16, budget=1 << 45, max_slots=slots)
+        used = free - torch.cuda.mem_get_info()[0]
+        t = srv.submit(0, chunk)
+        srv.drain()
+        st, _, arr = srv.result(t)
+        srv.close()
+        assert st == 0 and len(arr) > 0
+        return used, arr
+    used, want = serve()
+    block = (1 << 16) + -(-(int(plan.shifts(0).max()) + 64 + 2) // 16) * 16
+    rows = slots * (plan.fused_ws_bytes(block, 64)[0] - abi.aa_search_fused_least_ws_bytes(plan.handle, block, 64))
+    assert rows > 512 << 20
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - used + rows // 2, dtype=torch.uint8, device="cuda")
+    less, got = serve()
+    del hog
+    torch.cuda.empty_cache()
+    assert less < used - rows // 2
+    assert np.array_equal(got, want)
+    plan.close()
