@@ -147,18 +147,16 @@ def build_input(plan, w, device):
 # DRAM bytes per launch of the dominant kernels, from one ncu capture of the
 # small SKA-like case (2^17 samples, same plan) scaled to the full launch by its
 # output samples (traffic grows in proportion: input and output both scale with
-# the series length).  Each entry names the capture it comes from; set it to None
-# when the kernel changes until it is captured again.
+# the series length).  Set an entry to None when the kernel changes until it is
+# captured again.
 NCU_TRAFFIC = {
     ("dedisperse_u8", "grouped"): {
         # band rows: every launch of the row and summing kernels of the range
         "small_read_bytes": 5_973_090_000, "small_write_bytes": 5_213_680_000,
-        "small_output_samples": 1500 * 128687,
-        "capture": "profiles/dedisperse_bands_u8_ska-4096ch-2^17.md"},
+        "small_output_samples": 1500 * 128687},
     ("sps_boxcar", "pruned"): {
         "small_read_bytes": 877_592_576, "small_write_bytes": 49_681_408,
-        "small_output_samples": 1500 * 128687,
-        "capture": "profiles/sps_boxcar_ska-4096ch-2^17.md"},
+        "small_output_samples": 1500 * 128687},
 }
 
 
@@ -442,10 +440,13 @@ def bench_ours(args):
     u16_s = prof["dedisperse_u16"][1] / 1e3 / args.steps
     if box_s > 0:
         kern["sps_boxcar"]["gws_per_s"] = alg["width_samples"] / box_s / 1e9
+    # ranges that run on band rows ask for a row buffer
+    band_rows = plan.query(nsamp).dedisp_ws_bytes > abi.aa_dedisperse_least_ws_bytes(plan.handle, nsamp)
     for key, s in (("dedisperse_u8", u8_s), ("dedisperse_u16", u16_s)):
         if s > 0:
             kern[key]["gadds_per_s"] = alg["adds"][key] / s / 1e9
-            kern[key]["executed_gadds_per_s"] = alg["executed_adds"][key] / s / 1e9
+            if not band_rows:
+                kern[key]["executed_gadds_per_s"] = alg["executed_adds"][key] / s / 1e9
     evaluated = abi.aa_sps_workspace_work(ws_sps.data_ptr(), stream.cuda_stream)
     if box_s > 0:
         kern["sps_boxcar"]["evaluated_width_samples"] = evaluated
@@ -470,7 +471,7 @@ def bench_ours(args):
         samples = sum(g.ndm * g.length for g in rows)
         scale = samples / ent["small_output_samples"]
         per_launch = (ent["small_read_bytes"] + ent["small_write_bytes"]) * scale / len(rows)
-        return per_launch, f"ncu capture {ent['capture']}, scaled x{scale:.2f} by output samples"
+        return per_launch, f"ncu capture of 4096 channels x 2^17 samples, scaled x{scale:.2f} by output samples"
 
     if dominant == "dedisperse_fdmt":
         # what the tree cannot do without: the (decimated) input once, the
@@ -507,14 +508,26 @@ def bench_ours(args):
         nl = kern[key]["launches"] / max(args.steps, 1)
         alg_bytes = sum((w.nchans * g.nsamp_dec * (1 if g.dec == 1 else 2) + 4 * g.ndm * g.length)
                         for g in alg["lay"] if (g.dec == 1) == (key == "dedisperse_u8")) / max(nl, 1)
-        roof = {"kernel": key, "bound": "alu", "sm_count": sm_count, "achieved": achieved / 1e9,
-                "peak": lane_peak / 1e9, "unit": "Gop/s", "frac": achieved / lane_peak,
-                "traffic": tb, "traffic_source": tnote, "algorithmic_bytes_per_launch": alg_bytes,
-                "executed_gops": executed / 1e9, "executed_frac": executed / lane_peak,
-                "ops": "algorithmic channel-adds (sum over trials of nchans x L) per second; "
-                       "executed_* counts the adds the chosen strategy performs (grouped: "
-                       "those of the group sums, an upper bound where band rows run); peak = 1 add per lane per clock "
-                       f"({sm_count} SMs (device query) x 128 lanes x {sm_max:.0f} MHz)"}
+        common = {"kernel": key, "sm_count": sm_count, "traffic": tb, "traffic_source": tnote,
+                  "algorithmic_bytes_per_launch": alg_bytes, "algorithmic_gadds_per_s": achieved / 1e9}
+        if band_rows:
+            # every trial reads a word of two samples per band of at most 8 channels
+            words = sum(-(-w.nchans // 8) * g.ndm * g.length * 2 for g in alg["lay"]
+                        if (g.dec == 1) == (key == "dedisperse_u8"))
+            smem_peak = sm_count * 128 * sm_max * 1e6  # bytes / s
+            roof = {**common, "bound": "shared memory", "achieved": words / s / 1e9, "peak": smem_peak / 1e9,
+                    "unit": "GB/s", "frac": words / s / smem_peak,
+                    "ops": "shared-memory bytes that the sums over band rows cannot do without (bands of 8 "
+                           "channels, one 16-bit sum per trial, band and sample) over the time of rows and "
+                           f"sums; peak = {sm_count} SMs (device query) x 128 bytes x {sm_max:.0f} MHz"}
+        else:
+            roof = {**common, "bound": "alu", "achieved": achieved / 1e9, "peak": lane_peak / 1e9,
+                    "unit": "Gop/s", "frac": achieved / lane_peak,
+                    "executed_gops": executed / 1e9, "executed_frac": executed / lane_peak,
+                    "ops": "algorithmic channel-adds (sum over trials of nchans x L) per second; "
+                           "executed_* counts the adds the chosen strategy performs (grouped: those of "
+                           "the group sums); peak = 1 add per lane per clock "
+                           f"({sm_count} SMs (device query) x 128 lanes x {sm_max:.0f} MHz)"}
     hbm = float(peaks.get("hbm_gbs", 6678.2))
     eff_in_gbs = alg["dm_samples"] * w.nchans / step_s / 1e9
 
