@@ -778,8 +778,9 @@ def bench_stream(args):
     from paper_1912_07704_gb300 import abi as _abi
     block = st_rt.history_nsamp + N
     qi = plan.query(block, base.max_width)
-    unfused = qi.dd_elems * 4 + qi.dedisp_ws_bytes + qi.sps_ws_bytes
-    fused, _ = _abi.aa_search_fused_ws_bytes(plan.handle, block, base.max_width, 0)
+    # (what a slot is counted by: without row buffers)
+    unfused = qi.dd_elems * 4 + _abi.aa_dedisperse_least_ws_bytes(plan.handle, block) + qi.sps_ws_bytes
+    fused = _abi.aa_search_fused_least_ws_bytes(plan.handle, block, base.max_width, 0)
     resident = 2 * nbeams * base.nchans * plan.query(block).in_pitch_min
     per_slot = lambda work: work + (1 << 22) * 16 + 4096
     budget = 48 << 30

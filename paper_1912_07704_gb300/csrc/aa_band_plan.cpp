@@ -343,12 +343,13 @@ bool band_shifts(const BandPlan& bp, int C, int ndm, int32_t* out) {
 
 static void choose_bands(RangePlan& r, int C) {
     if (C > 65535 || r.desc.ndm < kBandTrials / 2) return;
-    // SM cycles per 512 output samples of the direct kernel: 64 trials of one
-    // channel take 991 (10.4e12 adds/s on 152 SMs at 2.07 GHz, measured).
-    // Bands of 8 channels cost about a seventh of that under fine DM steps;
-    // at DM step 1 over 256 channels, bands of 2 to 8 cost about half and run
-    // in 153 us against 180 (few CTAs: 1.5 waves).  Under half a block of
-    // trials the row kernel's launch is not repaid.
+    // Which ranges get tables at all (a launch looks at its length again, see
+    // bands_pay): SM cycles per 512 output samples against the direct kernel's,
+    // of which 64 trials of one channel take 991 (10.4e12 adds/s on 152 SMs at
+    // 2.07 GHz, measured).  Bands of 8 channels cost about a seventh of that under
+    // fine DM steps; at DM step 1 over 256 channels, bands of 2 to 8 cost about
+    // half and run in 143 us against 180 (few CTAs: 1.5 waves).  Under half a
+    // block of trials the row kernel's launch is not repaid.
     const double direct = 991.0 / 64 * (double)r.desc.ndm * C;
     BandPlan best;
     for (int k = 8; k >= 2; k /= 2) {

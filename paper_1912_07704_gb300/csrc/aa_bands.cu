@@ -11,23 +11,22 @@
 //                     16 warps of 4 trials add one row per band and trial, 8
 //                     words a lane.
 //
-// What bounds them (4096 channels, 1500 trials, 2^20 samples: 51.5 ms of sums and
-// 10.3 ms of rows; the grouped kernel takes 180):
-//   sums  shared memory: 64 trials x 8 word reads a lane and band are 512
-//         wavefronts, the ring's fill 74 more.  Two
+// What bounds them (4096 channels, 1500 trials, 2^20 samples: 61.4 ms, 51 of them
+// sums; the grouped kernel takes 180):
+//   sums  shared memory (its pipe 85 % busy): 64 trials x 8 word reads a lane and
+//         band are 512 wavefronts, the ring's fill 74 more, of 645 cycles.  Two
 //         pairs of bands are added per round where their rows fit 16 bits (one
-//         band 308 warp instructions a pair, one pair 234 and 712 cycles a band,
-//         57 ms; two pairs 645, 51.5), their sum's two 16-bit lanes go straight
-//         into 32-bit totals by dot products (2.36 ms a slab with 16-bit
-//         accumulators flushed every 32 bands, 1.96 without: the registers they
-//         took held loads back), and a place of the ring is refilled three
-//         pairs after its own (one pair after: 3.31, every pair then waits for
-//         the slowest warp).
-//   rows  latency and shared memory (63 % of its wavefronts): 2 reads a word
-//         and row plus the quads, 6 CTAs an SM (tiles of 256 words; 0.86 ms
-//         with two CTAs of 1024, 0.73 with six).
-// Segments of 256 / 512 / 1024 / 1536 trials, the same range: 91.4 / 77.2 /
-// 72.1 / 67.3 ms (rows shared by more trials are written once; the blocks of a
+//         pair: 712 cycles a band), their sum's two 16-bit lanes go straight into
+//         32-bit totals by dot products (16-bit accumulators flushed every 32
+//         bands hold loads back by the registers they take), and a place of the
+//         ring is refilled three pairs after its own (one pair after, every pair
+//         waits for the slowest warp: 1.7 times the time, measured on the form
+//         that adds one pair a round).
+//   rows  latency and shared memory (71 % of its pipe): 2 reads a word and row
+//         plus the quads, 6 CTAs an SM (tiles of 256 words; two CTAs of 1024 took
+//         1.18 times the time).
+// Segments of 256 / 512 / 1024 / 1536 trials, the same range: 86.0 / 71.4 /
+// 66.4 / 61.5 ms (rows shared by more trials are written once; the blocks of a
 // tile still find them in L2: 2.4 GB read for 2.1 written a slab).
 #include <algorithm>
 #include <cstdint>

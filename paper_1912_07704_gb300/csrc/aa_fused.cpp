@@ -195,9 +195,9 @@ aa_status aa_search_fused_device(const aa_plan* p, const uint8_t* d_in, int64_t 
         const int C = p->nchans;
         const void* in = d_in;
         int64_t pitch_in = in_pitch;
-        // (163072 samples of 4096 channels, four ranges: dedispersion 48.0 -> 29.1
-        // ms; a stripe builds the rows of its own trials, which takes over half
-        // of that.)
+        // (163072 samples of 4096 channels, four ranges: dedispersion 23.6 ms, 48.0
+        // on the grouped kernel; a stripe builds the rows of its own trials, which
+        // takes over half of that.)
         // Row buffer: what the range's decimated input leaves of its region, or
         // the scratch behind base.  Where neither keeps the SMs busy, the row
         // kernel decimates the 8-bit input itself and the whole region is the

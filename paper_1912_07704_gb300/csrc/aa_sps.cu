@@ -402,20 +402,17 @@ constexpr float kBig = 1.2676506002282294e30f;  // 2^100
 // warp at the same c, with sliding maxima over 2, 9 and 65 blocks: S1, S8,
 // S64): the first 8 chunks one by one, then groups of 8, from 64 on groups of
 // 64, opened where a thread's bound reaches its floor.  Eight bounds of one
-// level are computed side by side before the warp looks at them (one by one,
-// each with its vote, they took 330 cycles each).  The chunks to evaluate wait
-// in a queue of the thread, eight groups of eight as their bits, and are looked
-// at again when their turn comes: a warp evaluates when a queue is full and at
-// the end of the pass, so that most of its threads take part (a beam of 1024
-// channels x 48611 samples with two pulses, 2000 trials, W = 8192: 3.14 ms with
-// one chunk waiting, 2.23 with the queue; without pulses 0.92).  Both are
-// written down once, in one loop: with an evaluation and bounds at each place
-// that wants them the kernel waited for instructions more than for anything
-// else (2.6 of 10 stalls).
-// Skipping below
-// the running B, or below a lower bound of it, is exact for every start (such
-// a chunk changes neither B nor the first chunk that reaches it; the chunk
-// that the lower bound comes from is not skipped); below the threshold's cut
+// level are computed side by side before the warp looks at them.  The chunks to
+// evaluate wait in a queue of the thread, eight groups of eight as their bits,
+// and are looked at again when their turn comes: a warp evaluates when a queue is
+// full and at the end of the pass, so that most of its threads take part (a beam
+// of 1024 channels x 48611 samples with two pulses, 2000 trials, W = 8192: 2.1 ms,
+// 0.84 without the pulses; with one chunk waiting, before chunk 0 had bounds of its
+// own, 3.14 against 2.23).  Evaluation and bounds are written down once, in one
+// loop: with one at each place that wants them the kernel waits for instructions.
+// Skipping below the running B, or below a lower bound of it, is exact for every
+// start (such a chunk changes neither B nor the first chunk that reaches it; the
+// chunk that the lower bound comes from is not skipped); below the threshold's cut
 // it is exact for every B >= threshold and for every peak decision.
 //
 // FP32 with the roundings covered: P's differences are exact integers, each
@@ -487,7 +484,7 @@ __device__ __forceinline__ void eval_chunk(const float* __restrict__ pw, const f
 // Can a window of width 1 to 16 reach F (> 0)?  One bound for each of the widths
 // 1 | 2, 3 | 4-7 | 8-15 | 16: the largest end of its windows at each start.  In
 // noise hardly a warp has to evaluate chunk 0 then (2000 series of 48611 samples,
-// W = 64: 0.638 -> 0.554 ms; 2.3e9 starts with pulses, W = 8192: 34.8 -> 32.4).
+// W = 64: 0.554 ms, 0.638 without).
 __device__ __forceinline__ bool chunk0_reaches(const float* __restrict__ pb, const float (&base)[M], float f, float r, float F) {
     float win[2 * M];
 #pragma unroll
@@ -753,15 +750,10 @@ __host__ __device__ constexpr int sps_lists_words(int wpad) {
 // widths are searched.
 //
 // With 16 warps an SM (128 registers: a thread's starts, their B, the window of
-// a chunk) the tile's chain of short phases is what takes the time, so the
-// phases are kept few and their barriers fewer.  4096 channels x 2^20 samples,
-// W = 8192, 2.3e9 starts, 27 M candidates: 92 -> 32.4 ms; of 40.5 before the
-// search's queues (clock64) the width search 14.6, waiting for a tile's slowest warp 8.0, block maxima 4.4,
-// sums of new samples 2.8, candidates' widths 2.1, fresh tiles 1.5, peaks 1.4,
-// sliding 1.4.  Steps on the way: a warp's union of 128-width segments 92, the
-// chunks of each thread by lower bounds 66, their bounds eight at a time in one
-// loop 57, the new samples by cp.async, 32-bit sums, peaks from registers and
-// widths by half-warps 45, chunk numbers packed 40.5, queues 34.8, chunk 0 by bounds 32.4.
+// a chunk) the tile's chain of short phases is what takes the time (issue 50 %,
+// no pipe above 50 %), so the phases are kept few and their barriers fewer.  4096
+// channels x 2^20 samples, W = 8192, 2.3e9 starts, 20 M candidates: 30.6 ms (bounds
+// of 128-width segments for a whole warp: 80.9).
 template <bool LOW>
 __device__ __forceinline__ void boxcar_block(const SpsArgs& a, int row, int64_t tile_lo, int64_t tile_hi,
                                              float* sm) {
